@@ -145,8 +145,8 @@ def _points(data, n, d, g, shared):
         return z @ shared["a"].T + 0.01 * torch.randn(n, d, generator=g, device="cuda")
     # powerlaw: Gaussian, eigenvalue i ~ i^-1.5, a random rotation
     if "m" not in shared:
-        q, r = torch.linalg.qr(torch.randn(d, d, generator=g, device="cuda", dtype=torch.float64))
-        q = q * torch.sign(torch.diagonal(r))[None, :]
+        q, r = torch.linalg.qr(torch.randn(d, d, generator=g, device="cuda", dtype=torch.float64).cpu())
+        q = (q * torch.sign(torch.diagonal(r))[None, :]).cuda()
         scale = torch.arange(1, d + 1, device="cuda", dtype=torch.float64) ** -0.75
         shared["m"] = (q * scale[None, :]).float()
     return torch.randn(n, d, generator=g, device="cuda") @ shared["m"].T
