@@ -9,25 +9,22 @@
 // components choosing the same edge).
 //
 // One round on the GPU, all in kernels:
-//   1. node labels: a node's component when all its points share one, else
-//      -1 (leaves first, then each level up);
-//   2. for every point, its nearest point outside its component (one warp
-//      per point, a depth-first walk of the tree nearer child first, the
-//      same walk as kfn.cuh): Algorithm 3's Score with the pruning of the
-//      Boruvka Score -- a node is pruned when its d_min exceeds the point's
-//      best so far (strictly: an equal length may still have a lower rank)
-//      or when all its points lie in the point's own component; BaseCase
-//      distances in float64, the oracle's arithmetic;
-//   3. every component's shortest edge: an atomicMin over the squared
-//      lengths (kept up to date during step 2, whose walks prune with it),
-//      then over the endpoint pairs among the points that reach it;
-//   4. hooks: each component points to the component across its edge (a
+//   1. node labels: a node's component when all its points share one, else -1;
+//   2. a length no longer than which every component's shortest edge must be:
+//      from the edges of earlier rounds that still leave the component and
+//      from the pairs inside a packet (k_emst_prep, not in the first round);
+//   3. for every point that can still hold its component's shortest edge, its
+//      nearest point outside the component (k_emst_nn);
+//   4. every component's shortest edge: an atomicMin over the squared lengths
+//      (at the end of step 3), then over the endpoint pairs among the points
+//      that reach it;
+//   5. hooks: each component points to the component across its edge (a
 //      two-cycle keeps the lower id as the root), and each edge is written
-//      once, in component-id order after an in-kernel scan; then pointer
-//      jumping to the roots and relabelling of the points.
+//      once, in component-id order; then the roots are found and the points
+//      relabelled.
 #pragma once
 
-#include "knn_tile.cuh"
+#include "packet.cuh"
 
 namespace dt {
 
@@ -39,11 +36,18 @@ struct EmstArgs {
     const float* box;
     int64_t n;
     int hr;
-    int32_t* comp;          // per point: its component (a root point's tree position)
+    Packets pk;             // the points as packets of up to 32
+    int first;              // the first round: no earlier results, no bounds
+    const int32_t* comp;    // per point: its component (a root point's tree position)
     const int32_t* nlab;    // per node: its component if all its points share one, else -1
-    double* bd;             // per point: the squared length of its best edge out (inf: none)
-    int32_t* br;            // per point: the other end of that edge (tree position), or -1
-    unsigned long long* ck1;    // per component: the key of its shortest edge found so far
+    // per point, kept from round to round
+    double* bd;             // the squared length of its edge br
+    int32_t* br;            // the other end of its best edge out (tree position), or -1
+    float* lb;              // no point outside its component is nearer than this (squared)
+    unsigned char* done;    // br is its nearest point outside the component
+    // per component, of this round
+    uint32_t* cub;          // bits of a float no smaller than its shortest edge's squared length
+    unsigned long long* ck1;    // the key of its shortest edge
     unsigned long long* stats;  // [0] point distances, [1] leaves visited
 };
 
@@ -52,173 +56,203 @@ __device__ __forceinline__ unsigned long long dkey(double v) {
     return (unsigned long long)__double_as_longlong(v);
 }
 
+// Lowers a component's bound to v (bits of a non-negative float order like it).
+__device__ __forceinline__ void emst_publish(uint32_t* cub, float v) {
+    if (__float_as_uint(v) < *reinterpret_cast<volatile uint32_t*>(cub)) atomicMin(cub, __float_as_uint(v));
+}
+
+// Upper bounds of the components' shortest edges before the search: each
+// point's edge of an earlier round, where it still leaves the component, and
+// the pairs of points in its packet.  They let the search skip every point
+// whose lower bound exceeds its component's (on 1M uniform points in d = 3 all
+// but a few per cent from the third round on).
+template <int DP>
+__global__ void __launch_bounds__(128) k_emst_prep(const EmstArgs a) {
+    const int lane = threadIdx.x & 31;
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (w >= a.pk.count) return;
+    const int2 pr = packet_range(a.pk, a.nbeg, a.ncnt, w);
+    if (pr.y == 0) return;
+    const bool in = lane < pr.y;
+    const int64_t pos = pr.x + (in ? lane : 0);
+    const int32_t mine = in ? a.comp[pos] : -1;
+    float best = INFINITY;
+    if (in) {
+        const int32_t r = a.br[pos];
+        if (r >= 0 && a.comp[r] != mine) {
+            best = __double2float_ru(a.bd[pos]);
+        } else if (r >= 0) {
+            a.br[pos] = -1;
+            a.done[pos] = 0;
+        }
+    }
+    if (!__all_sync(0xffffffffu, mine == __shfl_sync(0xffffffffu, mine, 0) || !in)) {
+        float q[DP];
+        load_row<DP>(q, a.pts + pos * DP);
+        float key = INFINITY;
+        for (int e = 0; e < pr.y; ++e)
+            if (__shfl_sync(0xffffffffu, mine, e) != mine)
+                key = fminf(key, approx_d2<DP>(q, a.pts + (int64_t)(pr.x + e) * DP));
+        best = fminf(best, key_up<DP>(key));
+    }
+    // one update per component of the packet, by its first lane
+    const unsigned peers = __match_any_sync(0xffffffffu, mine);
+    best = __uint_as_float(__reduce_min_sync(peers, __float_as_uint(best)));
+    if (in && lane == __ffs(peers) - 1 && best < INFINITY) emst_publish(a.cub + mine, best);
+}
+
+// The nearest point outside its component of every point that can still hold
+// its component's shortest edge.  A warp takes a packet of up to 32 points of
+// one tree node, one per lane, and walks the tree depth first for all of
+// them: a node is visited while any lane needs it, its two child boxes and a
+// leaf's points are read once (the same address in every lane), and each lane
+// keeps its own bound.  Per visited node the warp spends about one lane's
+// work where a walk per point spent a whole warp's on each of the 32 points.
+//
+// Score: a lane prunes a node when all the node's points lie in its own
+// component, or when the squared d_min, rounded down, exceeds the smaller of
+// its own best and its component's (strictly: an equal length may still have
+// a lower rank; the holder of the component's shortest edge never prunes that
+// edge's other end).
+// BaseCase: float32 keys decide wherever their error cannot matter: a key
+// clearly below the best's replaces it, one clearly above is dropped, and
+// only between them (ties, near-ties) are both recomputed in float64 and
+// ranked by (length, endpoints).  Each point's final edge gets its float64
+// length at the end.
+// Points are skipped without a walk when an earlier round's answer still
+// leaves the component and was the nearest (the points outside a component
+// only become fewer), or when no outside point can be as near as the
+// component's bound.
+//
+// Tree and edges of 1M uniform points, d = 3: 240 -> 8.3 ms; of 60k points of the
+// 16-dimensional mixture: 198 -> 15.8 ms (against a float64 walk per point).
 template <int DP>
 __global__ void __launch_bounds__(128) k_emst_nn(const EmstArgs a) {
-    constexpr int NT = (2 * DP + 31) / 32;
+    __shared__ PacketStack stacks[4];
+    PacketStack& st = stacks[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const double shrink = 1.0 - (DP + 4) * 2.3e-16;  // d_min^2 rounded down
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (w >= a.pk.count) return;
+    const int2 pr = packet_range(a.pk, a.nbeg, a.ncnt, w);
+    if (pr.y == 0) return;
+    const bool in = lane < pr.y;
+    const int64_t pos = pr.x + (in ? lane : 0);
+    const int32_t mine = a.comp[pos];
+    double bd = INFINITY;   // float64 length of the best edge (valid only where have64)
+    int32_t br = -1;
+    bool have64 = false, need = in, done = false;
+    float cub = INFINITY;
+    if (!a.first && in) {
+        cub = __uint_as_float(*reinterpret_cast<volatile uint32_t*>(a.cub + mine));
+        br = a.br[pos];
+        bd = a.bd[pos];
+        have64 = br >= 0;
+        done = br >= 0 && a.done[pos];
+        need = !done && !(a.lb[pos] > cub);
+        if (!done && !need) br = -1;  // no outside point is near enough: not the holder
+    }
     unsigned long long n_pts = 0, n_leaves = 0;
-    for (int64_t pos = w0; pos < a.n; pos += nw) {
-        const int32_t mine = a.comp[pos];
-        const int32_t op = a.idx[pos];
-        const float* qp = a.pts + pos * DP;
+    if (__any_sync(0xffffffffu, need) && a.nlab[0] == -1) {
         float q[DP];
-#pragma unroll
-        for (int j = 0; j < DP / 4; ++j) {
-            const float4 v = reinterpret_cast<const float4*>(qp)[j];
-            q[4 * j] = v.x;
-            q[4 * j + 1] = v.y;
-            q[4 * j + 2] = v.z;
-            q[4 * j + 3] = v.w;
-        }
-        float qd[NT];
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            const int e = lane + 32 * t;
-            qd[t] = e < 2 * DP ? qp[e % DP] : 0.f;
-        }
-        // the best edge out: (bd2, blo, bhi) ranks by length, then endpoints
-        double bd2 = INFINITY;
-        uint32_t blo = 0xffffffffu, bhi = 0xffffffffu;
-        int32_t bestr = -1;
-        auto better = [](double d1, uint32_t l1, uint32_t h1, double d2, uint32_t l2, uint32_t h2) {
-            return d1 < d2 || (d1 == d2 && (l1 < l2 || (l1 == l2 && h1 < h2)));
-        };
-        // the stack: entry `lane` in (sn, sd = d_min^2 rounded down)
-        int32_t sn = 0;
-        double sd = 0.0;
-        // the pruning bound: the shortest edge out of this point's component
-        // found so far by any of its points (the point that holds the
-        // component's shortest edge never prunes that edge's other end)
-        volatile unsigned long long* cbest = a.ck1 + mine;
-        double bound = bd2;
-        int sp = a.nlab[0] == mine ? 0 : 1;
+        load_row<DP>(q, a.pts + pos * DP);
+        float bk = need && br >= 0 ? approx_d2<DP>(q, a.pts + (int64_t)br * DP) : INFINITY;  // br's key
+        float bound = fminf(key_up<DP>(bk), cub);
+        const uint32_t op = (uint32_t)a.idx[pos];
+        int sp = 0;
+        st.push(sp, 0, 0.f, lane);
         while (sp > 0) {
             --sp;
-            const int32_t n = __shfl_sync(0xffffffffu, sn, sp);
-            const double dm = __shfl_sync(0xffffffffu, sd, sp);
-            bound = fmin(bd2, __longlong_as_double((long long)*cbest));  // (fmin skips the NaN of "none")
-            bound = __shfl_sync(0xffffffffu, bound, 0);
-            if (dm > bound) continue;
+            const int32_t n = st.node[sp];
+            const float dm = st.d[sp][lane];
+            const bool want = need && !(dm > bound);
+            const unsigned wants = __ballot_sync(0xffffffffu, want);
+            if (!wants) continue;
             if (level_of_node(n) == a.hr) {
-                ++n_leaves;
                 const int rb = a.nbeg[n], rc = a.ncnt[n];
-                n_pts += rc;
+                ++n_leaves;
+                n_pts += (unsigned long long)rc * __popc(wants);
                 for (int r0 = 0; r0 < rc; r0 += 32) {
-                    const int r = rb + r0 + lane;
-                    bool valid = r0 + lane < rc;
-                    double d2 = INFINITY;
-                    uint32_t lo = 0xffffffffu, hi = 0xffffffffu;
-                    if (valid && a.comp[r] != mine) {
-                        d2 = exact_d2<DP>(q, a.pts + (int64_t)r * DP);
-                        const uint32_t o = (uint32_t)a.idx[r];
-                        lo = min((uint32_t)op, o);
-                        hi = max((uint32_t)op, o);
-                    } else {
-                        valid = false;
+                    // the points whose key may beat the best before them (few:
+                    // a running minimum), gathered without branches
+                    const int rn = min(32, rc - r0);
+                    float hi = key_hi<DP>(bk);  // a larger key cannot be as near as br
+                    unsigned m = 0;
+#pragma unroll 4
+                    for (int e = 0; e < rn; ++e) {
+                        const int r = rb + r0 + e;
+                        const float d = approx_d2<DP>(q, a.pts + (int64_t)r * DP);
+                        const float key = a.comp[r] == mine ? INFINITY : d;
+                        m |= (key <= hi ? 1u : 0u) << e;
+                        hi = fminf(hi, key_hi<DP>(key));
                     }
-                    // the warp's best candidate
-                    int cr = valid ? r : -1;
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) {
-                        const double od = __shfl_xor_sync(0xffffffffu, d2, off);
-                        const uint32_t ol = __shfl_xor_sync(0xffffffffu, lo, off);
-                        const uint32_t oh = __shfl_xor_sync(0xffffffffu, hi, off);
-                        const int orr = __shfl_xor_sync(0xffffffffu, cr, off);
-                        if (better(od, ol, oh, d2, lo, hi)) {
-                            d2 = od;
-                            lo = ol;
-                            hi = oh;
-                            cr = orr;
+                    if (!want) m = 0;
+                    while (m) {
+                        const int r = rb + r0 + __ffs(m) - 1;
+                        m &= m - 1;
+                        if (a.comp[r] == mine) continue;  // (an overflowing key)
+                        const float key = approx_d2<DP>(q, a.pts + (int64_t)r * DP);
+                        if (key > key_hi<DP>(bk)) continue;
+                        if (br < 0 || key < key_lo<DP>(bk)) {
+                            br = r;
+                            bk = key;
+                            have64 = false;
+                            continue;
+                        }
+                        // too close to call in float32: float64 lengths, then endpoints
+                        if (!have64) bd = exact_d2<DP>(q, a.pts + (int64_t)br * DP);
+                        have64 = true;
+                        const double d = exact_d2<DP>(q, a.pts + (int64_t)r * DP);
+                        const uint32_t o1 = (uint32_t)a.idx[br], o2 = (uint32_t)a.idx[r];
+                        const uint32_t l1 = min(op, o1), l2 = min(op, o2);
+                        if (d < bd || (d == bd && (l2 < l1 || (l2 == l1 && max(op, o2) < max(op, o1))))) {
+                            bd = d;
+                            br = r;
+                            bk = key;
                         }
                     }
-                    if (cr >= 0 && better(d2, lo, hi, bd2, blo, bhi)) {
-                        bd2 = d2;
-                        blo = lo;
-                        bhi = hi;
-                        bestr = cr;
-                        if (lane == 0) atomicMin(a.ck1 + mine, dkey(bd2));
-                        bound = fmin(bound, bd2);
-                    }
+                }
+                if (want) {
+                    const float up = key_up<DP>(bk);
+                    if (up < cub) emst_publish(a.cub + mine, up);
+                    cub = fminf(cub, __uint_as_float(*reinterpret_cast<volatile uint32_t*>(a.cub + mine)));
+                    bound = fminf(up, cub);
                 }
                 continue;
             }
-            // the two children: squared d_min from the point to each box
             const int64_t l = 2 * (int64_t)n + 1;
-            const float* bx = a.box + l * 2 * DP;
-            double s0 = 0.0, s1 = 0.0;
-#pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                const int e = lane + 32 * t;
-                if (e < 2 * DP) {
-                    const int c = e / DP, dd = e % DP;
-                    const double qv = qd[t], lo = bx[c * 2 * DP + dd], hi = bx[c * 2 * DP + DP + dd];
-                    const double g = fmax(fmax(lo - qv, qv - hi), 0.0);
-                    if (c == 0) s0 += g * g;
-                    else s1 += g * g;
-                }
-            }
-            double d0, d1;
-            if (2 * DP <= 32) {
-                double sv = s0 + s1;
-#pragma unroll
-                for (int off = DP / 2; off > 0; off >>= 1) sv += __shfl_xor_sync(0xffffffffu, sv, off);
-                d0 = __shfl_sync(0xffffffffu, sv, 0);
-                d1 = __shfl_sync(0xffffffffu, sv, DP);
-            } else {
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) {
-                    s0 += __shfl_xor_sync(0xffffffffu, s0, off);
-                    s1 += __shfl_xor_sync(0xffffffffu, s1, off);
-                }
-                d0 = s0;
-                d1 = s1;
-            }
-            d0 *= shrink;
-            d1 *= shrink;
-            // push the farther child first, so that the nearer one is taken next
-            const bool right_near = d1 < d0;
-            const int32_t cf = (int32_t)(right_near ? l : l + 1), cn = (int32_t)(right_near ? l + 1 : l);
-            const double df = right_near ? d0 : d1, dn = right_near ? d1 : d0;
-            if (a.nlab[cf] != mine && !(df > bound)) {
-                if (lane == sp) {
-                    sn = cf;
-                    sd = df;
-                }
-                ++sp;
-            }
-            if (a.nlab[cn] != mine && !(dn > bound)) {
-                if (lane == sp) {
-                    sn = cn;
-                    sd = dn;
-                }
-                ++sp;
-            }
+            float d0, d1;
+            packet_child_dmin<DP>(q, a.box + l * 2 * DP, d0, d1);
+            const bool w0 = want && a.nlab[l] != mine && !(d0 > bound);
+            const bool w1 = want && a.nlab[l + 1] != mine && !(d1 > bound);
+            packet_push_near_first(st, sp, (int32_t)l, w0 ? d0 : INFINITY, w1 ? d1 : INFINITY, w0, w1, lane);
         }
-        if (lane == 0) {
-            a.bd[pos] = bd2;
-            a.br[pos] = bestr;
+        if (need) {
+            const float up = key_up<DP>(bk);
+            done = br >= 0 && up <= cub;
+            a.lb[pos] = fmaxf(__fmul_rd(fminf(bk, cub), 1.f - 8.f * rel_eps<DP>()) - kKeyTiny, 0.f);
+            if (br >= 0 && !have64) bd = exact_d2<DP>(q, a.pts + (int64_t)br * DP);
         }
     }
-    if (a.stats) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            n_pts += __shfl_xor_sync(0xffffffffu, n_pts, off);
-            n_leaves += __shfl_xor_sync(0xffffffffu, n_leaves, off);
+    if (in) {
+        a.bd[pos] = bd;
+        a.br[pos] = br;
+        a.done[pos] = done;
+        if (br >= 0) {
+            const unsigned long long k = dkey(bd);
+            if (k < *reinterpret_cast<volatile unsigned long long*>(a.ck1 + mine)) atomicMin(a.ck1 + mine, k);
         }
-        if (lane == 0) {
-            atomicAdd(&a.stats[0], n_pts / 32);
-            atomicAdd(&a.stats[1], n_leaves / 32);
-        }
+    }
+    if (lane == 0 && n_leaves) {
+        atomicAdd(&a.stats[0], n_pts);
+        atomicAdd(&a.stats[1], n_leaves);
     }
 }
 
 template <int DP>
-int launch_emst_nn(const EmstArgs& a, int grid, cudaStream_t s) {
-    auto kern = k_emst_nn<DP>;
-    DT_LAUNCH(kern, grid, 128, 0, s, a);
+int launch_emst_nn(const EmstArgs& a, cudaStream_t s) {
+    const int grid = (int)((a.pk.count + 3) / 4);
+    if (!a.first) DT_LAUNCH(k_emst_prep<DP>, grid, 128, 0, s, a);
+    DT_LAUNCH(k_emst_nn<DP>, grid, 128, 0, s, a);
     return DTREE_OK;
 }
 

@@ -2,5 +2,5 @@
 #include "emst.cuh"
 
 namespace dt {
-template int launch_emst_nn<4>(const EmstArgs&, int, cudaStream_t);
+template int launch_emst_nn<4>(const EmstArgs&, cudaStream_t);
 }  // namespace dt
