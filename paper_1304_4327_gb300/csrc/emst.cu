@@ -5,6 +5,7 @@
 #include <cstring>
 
 #include "emst.cuh"
+#include "scan.cuh"
 
 namespace dt {
 namespace {
@@ -120,29 +121,6 @@ __global__ void __launch_bounds__(kHookCta) k_emst_hook(const int32_t* comp, con
     const int64_t c = blockIdx.x * (int64_t)kHookCta + threadIdx.x;
     const int cnt = __syncthreads_count(emst_hook_of(c, n, comp, br, pick, ck1, ck2, par));
     if (threadIdx.x == 0) adds[blockIdx.x] = cnt;
-}
-
-// In place: a[0..n) -> exclusive prefix sums, a[n] = the total (one CTA,
-// 1024 consecutive entries at a time).
-__global__ void __launch_bounds__(1024) k_emst_scan(int64_t* a, int64_t n) {
-    __shared__ int64_t part[1024];
-    const int t = threadIdx.x;
-    int64_t carry = 0;
-    for (int64_t b = 0; b < n; b += 1024) {
-        const int64_t v = b + t < n ? a[b + t] : 0;
-        part[t] = v;
-        __syncthreads();
-        for (int off = 1; off < 1024; off <<= 1) {
-            const int64_t u = t >= off ? part[t - off] : 0;
-            __syncthreads();
-            part[t] += u;
-            __syncthreads();
-        }
-        if (b + t < n) a[b + t] = carry + part[t] - v;
-        carry += part[1023];
-        __syncthreads();
-    }
-    if (t == 0) a[n] = carry;
 }
 
 // The round's edges, in component-id order after the ones written before.
@@ -263,7 +241,10 @@ extern "C" int dtree_emst(const dtree_t* t, int64_t* out_edges, float* out_dist,
     a.box = t->box;
     a.n = n;
     a.hr = t->height;
-    a.pk = make_packets(t);
+    a.pk1 = make_packets(t, 0);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    a.pk = make_packets(t, packet_lanes(n, sms));
     a.first = 1;
     a.comp = comp;
     a.nlab = nlab;
@@ -304,7 +285,7 @@ extern "C" int dtree_emst(const dtree_t* t, int64_t* out_edges, float* out_dist,
             k_emst_min2<<<g256(n), 256, 0, s>>>(comp, bd, br, t->idx, n, ck1, ck2);
             k_emst_pick<<<g256(n), 256, 0, s>>>(comp, bd, br, t->idx, n, ck1, ck2, pick);
             k_emst_hook<<<(int)nhook, kHookCta, 0, s>>>(comp, br, pick, ck1, ck2, n, par, adds);
-            k_emst_scan<<<1, 1024, 0, s>>>(adds, nhook);
+            k_scan_sums<<<1, kScanThreads, 0, s>>>(adds, nhook, adds + nhook);
             k_emst_emit<<<(int)nhook, kHookCta, 0, s>>>(comp, pick, br, bd, t->idx, ck1, ck2, adds, n, base,
                                                         out_edges, out_dist);
             k_emst_roots<<<g256(n), 256, 0, s>>>(par, n);

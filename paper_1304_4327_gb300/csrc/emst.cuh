@@ -36,7 +36,7 @@ struct EmstArgs {
     const float* box;
     int64_t n;
     int hr;
-    Packets pk;             // the points as packets of up to 32
+    Packets pk, pk1;        // the points as packets, and as packets of up to 32
     int first;              // the first round: no earlier results, no bounds
     const int32_t* comp;    // per point: its component (a root point's tree position)
     const int32_t* nlab;    // per node: its component if all its points share one, else -1
@@ -61,6 +61,13 @@ __device__ __forceinline__ void emst_publish(uint32_t* cub, float v) {
     if (__float_as_uint(v) < *reinterpret_cast<volatile uint32_t*>(cub)) atomicMin(cub, __float_as_uint(v));
 }
 
+// Edges from the point with original index o: is the one of squared length d
+// to r before the one of squared length e to t?
+__device__ __forceinline__ bool emst_before(double d, uint32_t o, uint32_t r, double e, uint32_t t) {
+    const uint32_t l1 = min(o, r), l2 = min(o, t);
+    return d < e || (d == e && (l1 < l2 || (l1 == l2 && max(o, r) < max(o, t))));
+}
+
 // Upper bounds of the components' shortest edges before the search: each
 // point's edge of an earlier round, where it still leaves the component, and
 // the pairs of points in its packet.  They let the search skip every point
@@ -70,8 +77,8 @@ template <int DP>
 __global__ void __launch_bounds__(128) k_emst_prep(const EmstArgs a) {
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= a.pk.count) return;
-    const int2 pr = packet_range(a.pk, a.nbeg, a.ncnt, w);
+    if (w >= a.pk1.count) return;
+    const int2 pr = packet_range(a.pk1, a.nbeg, a.ncnt, w);
     if (pr.y == 0) return;
     const bool in = lane < pr.y;
     const int64_t pos = pr.x + (in ? lane : 0);
@@ -102,12 +109,9 @@ __global__ void __launch_bounds__(128) k_emst_prep(const EmstArgs a) {
 }
 
 // The nearest point outside its component of every point that can still hold
-// its component's shortest edge.  A warp takes a packet of up to 32 points of
-// one tree node, one per lane, and walks the tree depth first for all of
-// them: a node is visited while any lane needs it, its two child boxes and a
-// leaf's points are read once (the same address in every lane), and each lane
-// keeps its own bound.  Per visited node the warp spends about one lane's
-// work where a walk per point spent a whole warp's on each of the 32 points.
+// its component's shortest edge, by packets (packet.cuh) that walk the tree
+// nearer child first.  The G lanes of a point share its bound and keep a best
+// edge each, the best of which is taken at the end.
 //
 // Score: a lane prunes a node when all the node's points lie in its own
 // component, or when the squared d_min, rounded down, exceeds the smaller of
@@ -124,8 +128,8 @@ __global__ void __launch_bounds__(128) k_emst_prep(const EmstArgs a) {
 // only become fewer), or when no outside point can be as near as the
 // component's bound.
 //
-// Tree and edges of 1M uniform points, d = 3: 240 -> 8.3 ms; of 60k points of the
-// 16-dimensional mixture: 198 -> 15.8 ms (against a float64 walk per point).
+// Tree and edges of 1M uniform points, d = 3: 240 -> 8.4 ms; of 60k points of the
+// 16-dimensional mixture: 198 -> 9.9 ms (against a float64 walk per point).
 template <int DP>
 __global__ void __launch_bounds__(128) k_emst_nn(const EmstArgs a) {
     __shared__ PacketStack stacks[4];
@@ -135,8 +139,10 @@ __global__ void __launch_bounds__(128) k_emst_nn(const EmstArgs a) {
     if (w >= a.pk.count) return;
     const int2 pr = packet_range(a.pk, a.nbeg, a.ncnt, w);
     if (pr.y == 0) return;
-    const bool in = lane < pr.y;
-    const int64_t pos = pr.x + (in ? lane : 0);
+    const int gs = a.pk.gs, G = 1 << gs;
+    const int qi = lane >> gs, sub = lane & (G - 1);
+    const bool in = qi < pr.y;
+    const int64_t pos = pr.x + (in ? qi : 0);
     const int32_t mine = a.comp[pos];
     double bd = INFINITY;   // float64 length of the best edge (valid only where have64)
     int32_t br = -1;
@@ -170,7 +176,7 @@ __global__ void __launch_bounds__(128) k_emst_nn(const EmstArgs a) {
             if (level_of_node(n) == a.hr) {
                 const int rb = a.nbeg[n], rc = a.ncnt[n];
                 ++n_leaves;
-                n_pts += (unsigned long long)rc * __popc(wants);
+                n_pts += (unsigned long long)rc * (__popc(wants) >> gs);
                 for (int r0 = 0; r0 < rc; r0 += 32) {
                     // the points whose key may beat the best before them (few:
                     // a running minimum), gathered without branches
@@ -178,7 +184,7 @@ __global__ void __launch_bounds__(128) k_emst_nn(const EmstArgs a) {
                     float hi = key_hi<DP>(bk);  // a larger key cannot be as near as br
                     unsigned m = 0;
 #pragma unroll 4
-                    for (int e = 0; e < rn; ++e) {
+                    for (int e = sub; e < rn; e += G) {
                         const int r = rb + r0 + e;
                         const float d = approx_d2<DP>(q, a.pts + (int64_t)r * DP);
                         const float key = a.comp[r] == mine ? INFINITY : d;
@@ -202,17 +208,17 @@ __global__ void __launch_bounds__(128) k_emst_nn(const EmstArgs a) {
                         if (!have64) bd = exact_d2<DP>(q, a.pts + (int64_t)br * DP);
                         have64 = true;
                         const double d = exact_d2<DP>(q, a.pts + (int64_t)r * DP);
-                        const uint32_t o1 = (uint32_t)a.idx[br], o2 = (uint32_t)a.idx[r];
-                        const uint32_t l1 = min(op, o1), l2 = min(op, o2);
-                        if (d < bd || (d == bd && (l2 < l1 || (l2 == l1 && max(op, o2) < max(op, o1))))) {
+                        if (emst_before(d, op, (uint32_t)a.idx[r], bd, (uint32_t)a.idx[br])) {
                             bd = d;
                             br = r;
                             bk = key;
                         }
                     }
                 }
+                float best = bk;
+                for (int off = G >> 1; off > 0; off >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, off));
                 if (want) {
-                    const float up = key_up<DP>(bk);
+                    const float up = key_up<DP>(best);
                     if (up < cub) emst_publish(a.cub + mine, up);
                     cub = fminf(cub, __uint_as_float(*reinterpret_cast<volatile uint32_t*>(a.cub + mine)));
                     bound = fminf(up, cub);
@@ -226,14 +232,25 @@ __global__ void __launch_bounds__(128) k_emst_nn(const EmstArgs a) {
             const bool w1 = want && a.nlab[l + 1] != mine && !(d1 > bound);
             packet_push_near_first(st, sp, (int32_t)l, w0 ? d0 : INFINITY, w1 ? d1 : INFINITY, w0, w1, lane);
         }
+        // the best of the point's G lanes, in float64 and by endpoints
+        if (need && br >= 0 && !have64) bd = exact_d2<DP>(q, a.pts + (int64_t)br * DP);
+        if (br < 0) bd = INFINITY;
+        float best = bk;
+        for (int off = G >> 1; off > 0; off >>= 1) {
+            best = fminf(best, __shfl_xor_sync(0xffffffffu, best, off));
+            const double d = __shfl_xor_sync(0xffffffffu, bd, off);
+            const int32_t r = __shfl_xor_sync(0xffffffffu, br, off);
+            if (r >= 0 && (br < 0 || emst_before(d, op, (uint32_t)a.idx[r], bd, (uint32_t)a.idx[br]))) {
+                bd = d;
+                br = r;
+            }
+        }
         if (need) {
-            const float up = key_up<DP>(bk);
-            done = br >= 0 && up <= cub;
-            a.lb[pos] = fmaxf(__fmul_rd(fminf(bk, cub), 1.f - 8.f * rel_eps<DP>()) - kKeyTiny, 0.f);
-            if (br >= 0 && !have64) bd = exact_d2<DP>(q, a.pts + (int64_t)br * DP);
+            done = br >= 0 && key_up<DP>(best) <= cub;
+            if (sub == 0) a.lb[pos] = fmaxf(__fmul_rd(fminf(best, cub), 1.f - 8.f * rel_eps<DP>()) - kKeyTiny, 0.f);
         }
     }
-    if (in) {
+    if (in && sub == 0) {
         a.bd[pos] = bd;
         a.br[pos] = br;
         a.done[pos] = done;
@@ -250,9 +267,8 @@ __global__ void __launch_bounds__(128) k_emst_nn(const EmstArgs a) {
 
 template <int DP>
 int launch_emst_nn(const EmstArgs& a, cudaStream_t s) {
-    const int grid = (int)((a.pk.count + 3) / 4);
-    if (!a.first) DT_LAUNCH(k_emst_prep<DP>, grid, 128, 0, s, a);
-    DT_LAUNCH(k_emst_nn<DP>, grid, 128, 0, s, a);
+    if (!a.first) DT_LAUNCH(k_emst_prep<DP>, (int)((a.pk1.count + 3) / 4), 128, 0, s, a);
+    DT_LAUNCH(k_emst_nn<DP>, (int)((a.pk.count + 3) / 4), 128, 0, s, a);
     return DTREE_OK;
 }
 

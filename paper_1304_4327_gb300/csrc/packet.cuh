@@ -1,43 +1,54 @@
-// packet.cuh -- walks of a tree by packets of points, shared by the searches
-// whose query node is a single point (spanning tree, furthest neighbours,
-// ranges).
+// packet.cuh -- walks of a tree by packets of points (the spanning tree's
+// nearest-edge search).
 //
-// A packet is up to 32 points of one query-tree node, one per lane of a warp.
-// Neighbours in the tree want almost the same reference nodes, so the warp
-// walks the reference tree once for all of them: every box and every
-// reference point is read at one address for the whole warp, each lane
-// computes its own bound from registers with no shuffles, and a node is
-// entered while any lane wants it.  What this costs is the distances of lanes
-// that would have pruned the node; what it saves is 31 of 32 node visits.
+// A packet is up to 32 / G points of one query-tree node, G lanes of a warp
+// for each (G a power of two).  Neighbours in the tree want almost the same
+// reference nodes, so the warp walks the reference tree once for all of them:
+// every box is read at one address for the whole warp, each lane computes its
+// point's bound from registers with no shuffles, and a node is entered while
+// any lane wants it; a leaf's points are dealt out to the G lanes of a point.
+// What this costs is the distances of points that would have pruned the node;
+// what it saves is all but one of 32 / G node visits.  G = 1 does the least
+// work; few points take a larger G, so that their packets fill the GPU.
 #pragma once
 
 #include "knn_tile.cuh"
 
 namespace dt {
 
-// The points of a tree as packets: the nodes [first, first + 2^level) in
-// chunks of 32 (cpn of them per node; more than one only where leaves hold
-// more than 32 points).
+// The points of a tree as packets of up to `size` = 32 >> gs points: the nodes
+// [first, first + 2^level) in chunks (cpn of them per node; more than one only
+// where leaves hold more than a packet).
 struct Packets {
     int64_t first, count;
-    int cpn;
+    int cpn, gs;
 };
 
-inline Packets make_packets(const dtree_t* t) {
-    const int level = t->height < level_of_count(t->n, 32) ? t->height : level_of_count(t->n, 32);
+inline Packets make_packets(const dtree_t* t, int gs) {
+    const int size = 32 >> gs;
+    const int level = t->height < level_of_count(t->n, size) ? t->height : level_of_count(t->n, size);
     const int64_t nodes = (int64_t)1 << level;
     Packets p;
+    p.gs = gs;
     p.first = nodes - 1;
-    p.cpn = (int)(((t->n + nodes - 1) / nodes + 31) / 32);
+    p.cpn = (int)(((t->n + nodes - 1) / nodes + size - 1) / size);
     p.count = nodes * p.cpn;
     return p;
+}
+
+// log2 of the lanes per point for n points: G = 1 once their packets give every
+// SM sixteen warps, else the G (up to 8) that does.
+inline int packet_lanes(int64_t n, int sms) {
+    int gs = 0;
+    while (gs < 3 && (n << gs) < (int64_t)sms * 16 * 32) ++gs;
+    return gs;
 }
 
 // First tree position and number of points of packet w.
 __device__ __forceinline__ int2 packet_range(const Packets& p, const int32_t* nbeg, const int32_t* ncnt, int64_t w) {
     const int64_t node = p.first + w / p.cpn;
-    const int c = (int)(w % p.cpn);
-    return make_int2(nbeg[node] + 32 * c, max(0, min(32, ncnt[node] - 32 * c)));
+    const int size = 32 >> p.gs, c = (int)(w % p.cpn) * size;
+    return make_int2(nbeg[node] + c, max(0, min(size, ncnt[node] - c)));
 }
 
 // The depth-first walk's stack, one per warp: per entry the node and each
@@ -73,6 +84,7 @@ __device__ __forceinline__ void load_row(float (&q)[DP], const float* p) {
 //   key_lo(k)  a key below it belongs to a strictly smaller distance than k's
 //   key_hi(k)  a key above it belongs to a strictly larger distance than k's
 constexpr float kKeyTiny = 1e-37f;
+constexpr float kKeyMax = 3.4028234e38f;  // what an overflowing key stands for at least (but for its error)
 
 template <int DP>
 __device__ __forceinline__ float key_up(float k) {
@@ -112,8 +124,8 @@ __device__ __forceinline__ void packet_child_dmin(const float (&q)[DP], const fl
         }
     }
     const float f = 1.f - 2.f * rel_eps<DP>();
-    d0 = fmaxf(__fsub_rd(__fmul_rd(fminf(s[0], 3.4028234e38f), f), kKeyTiny), 0.f);
-    d1 = fmaxf(__fsub_rd(__fmul_rd(fminf(s[1], 3.4028234e38f), f), kKeyTiny), 0.f);
+    d0 = fmaxf(__fsub_rd(__fmul_rd(fminf(s[0], kKeyMax), f), kKeyTiny), 0.f);
+    d1 = fmaxf(__fsub_rd(__fmul_rd(fminf(s[1], kKeyMax), f), kKeyTiny), 0.f);
 }
 
 // Push the wanted ones of two siblings (l, l + 1) so that the one nearer to

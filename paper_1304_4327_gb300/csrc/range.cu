@@ -1,41 +1,14 @@
 // range.cu -- dtree_range_count / dtree_range_fill: exact range search, host
-// side, and the scan that turns per-query counts into segment offsets (the
-// kernels and their reading of Section 6 are in range.cuh).
+// side (the kernels and their reading of Section 6 are in range.cuh).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 
 #include "range.cuh"
+#include "scan.cuh"
 
 namespace dt {
 namespace {
-
-// In place: counts c[0..n) -> exclusive prefix sums, and c[n] = the total.
-// One CTA; each thread sums a contiguous chunk, the chunk sums are scanned in
-// shared memory, then each thread rewrites its chunk.
-__global__ void __launch_bounds__(1024) k_range_scan(int64_t* c, int64_t n) {
-    __shared__ int64_t part[1024];
-    const int t = threadIdx.x;
-    const int64_t chunk = (n + 1023) / 1024;
-    const int64_t b0 = t * chunk, b = b0 < n ? b0 : n, e = b + chunk < n ? b + chunk : n;
-    int64_t s = 0;
-    for (int64_t i = b; i < e; ++i) s += c[i];
-    part[t] = s;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const int64_t v = t >= off ? part[t - off] : 0;
-        __syncthreads();
-        part[t] += v;
-        __syncthreads();
-    }
-    int64_t run = part[t] - s;  // exclusive
-    for (int64_t i = b; i < e; ++i) {
-        const int64_t v = c[i];
-        c[i] = run;
-        run += v;
-    }
-    if (t == 1023) c[n] = part[1023];
-}
 
 int range_launch(int dp, const RangeArgs& a, bool fill, int grid, cudaStream_t s) {
     switch (dp) {
@@ -108,8 +81,10 @@ extern "C" int dtree_range_count(const dtree_t* query, const dtree_t* ref, doubl
     if (!offsets || !total) return DTREE_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t launches0 = g_launches.load();
+    // scratch: four counters and the scan's block sums
     unsigned long long* cnt = nullptr;
-    DT_CHECK(cudaMallocAsync((void**)&cnt, 4 * sizeof(unsigned long long), s));
+    DT_CHECK(cudaMallocAsync((void**)&cnt, (4 + (size_t)scan_blocks(a.nq)) * sizeof(unsigned long long), s));
+    int64_t* sums = reinterpret_cast<int64_t*>(cnt + 4);
     g_allocs.fetch_add(1, std::memory_order_relaxed);
     a.counts = offsets;
     a.stats = cnt;
@@ -125,12 +100,8 @@ extern "C" int dtree_range_count(const dtree_t* query, const dtree_t* ref, doubl
         if (timed) cudaEventRecord(ev[0], s);
         rc = range_launch(ref->dp, a, false, range_grid(a.nq), s);
         if (rc != DTREE_OK) break;
-        k_range_scan<<<1, 1024, 0, s>>>(offsets, a.nq);
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-        if (cudaGetLastError() != cudaSuccess) {
-            rc = DTREE_ERR_CUDA;
-            break;
-        }
+        rc = exclusive_scan(offsets, a.nq, sums, s);
+        if (rc != DTREE_OK) break;
         if (timed) cudaEventRecord(ev[1], s);
         if (cudaMemcpyAsync(total, offsets + a.nq, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaMemcpyAsync(h, cnt, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess) {
