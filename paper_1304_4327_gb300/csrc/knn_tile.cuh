@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(kQB) k_query_cap(const TileArgs a, float* qcap
     const int nq = min(kQB, P.qcnt[qnode] - wi.y * kQB);
     const int kq = P.k, hr = P.hr;
     const bool mono = P.mono != 0;
-    for (int qi = warp; qi < nq; qi += kQB / 32) {
+    for (int qi = warp + blockIdx.y * (kQB / 32); qi < nq; qi += gridDim.y * (kQB / 32)) {
         const int myq = P.qbeg[qnode] + wi.y * kQB + qi;
         const int64_t row = P.q0 + myq;
         const float* qp = P.qpts + (int64_t)myq * DP;
@@ -992,10 +992,14 @@ int launch_query_cap(const TileArgs& a, int kc, int budget, float* qcap, cudaStr
     if (a.nitems <= 0) return DTREE_OK;
     if (budget < 1 || kc != a.kc_rows) return DTREE_ERR_UNSUPPORTED;
     budget = std::min(budget, kCapMaxLeaves);
+    // one CTA per work item, or, where the items alone do not fill the GPU, as
+    // many as do (a warp then serves a few of the item's queries instead of 32
+    // in a row: 64 items at d = 16, 0.60 -> 0.08 ms)
 #define DT_CAP_CASE(KCV)                                                   \
     case KCV: {                                                            \
         auto kern = k_query_cap<DP, KCV>;                                  \
-        DT_LAUNCH(kern, a.nitems, kQB, 0, s, a, qcap, budget);             \
+        const int split = std::max(1, std::min(32, occupancy_grid((const void*)kern, kQB, 0) / a.nitems)); \
+        DT_LAUNCH(kern, dim3(a.nitems, split), kQB, 0, s, a, qcap, budget); \
         return DTREE_OK;                                                   \
     }
     switch (kc) {
