@@ -94,6 +94,8 @@ struct TcShape {
     // slots fit shared memory
     static constexpr int TN = DP <= 16 ? 256 : 128;
     static constexpr int TN8 = TN / 8;
+    // accumulators: as many as TMEM's 512 columns hold
+    static constexpr int NACC = 512 / TN;
     __host__ __device__ static constexpr int astep(int m) {
         return !REUSE ? m : m < 2 * H ? m : m < 3 * H ? m - 2 * H : 2 * H;
     }
@@ -349,10 +351,13 @@ static_assert(TT_N <= 32, "the diagnostic timer buffer holds 32 counters");
 //              lane) per thread; each warp reads its own 32 lanes of an
 //              accumulator, examines the keys and keeps its queries' lists,
 //              and hands the accumulator and the tile's row-group table back
-//              by mbarrier arrivals, independently of the other warps.  Tiles alternate
-//              between two accumulators: with NG = 1 the group reads both in
-//              turn; with NG = 2 group g reads accumulator g and keeps its own
-//              lists, which are merged when the block is done
+//              by mbarrier arrivals, independently of the other warps.  Tiles take the
+//              accumulators in turn: with NG = 1 the group reads them all;
+//              with NG = 2 group g reads every second one and keeps its own
+//              lists, which are merged when the block is done.  Four
+//              accumulators (TN = 128) let the MMAs run on while one of the
+//              four warps inserts: an accumulator is free only when all four
+//              have read it
 //   warp 4 NG  planner: prepares a window of the block's candidate leaves at
 //              a time (Algorithm 3's test against the block's bound, each
 //              kept leaf's range and its place in the window's run of 8-row
@@ -361,7 +366,7 @@ static_assert(TT_N <= 32, "the diagnostic timer buffer holds 32 counters");
 //              the groups' first rows (a ring of GR tables, deeper than the
 //              slots: a slot is free again once its MMAs are done)
 //   warp 4 NG + 1  MMA issuer: one thread turns a filled slot into an
-//              accumulator (two in turn) with tcgen05.mma
+//              accumulator with tcgen05.mma
 // Hand-over by mbarriers: op_full (planner -> MMA: its arrival plus the
 // copied bytes), acc_full (MMA -> epilogue: the MMA's commit plus the
 // issuer's arrival with the tile's row-group table and columns), acc_empty (epilogue ->
@@ -375,7 +380,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
     using S = TcShape<FMT, DP>;
     using L = TcSmem<FMT, DP, KC, NG>;
     using Bd = TcBound<FMT, DP>;
-    constexpr int TN = S::TN, TN8 = S::TN8, NB = L::NB, GR = L::GR, CB = L::CB, WIN = L::WIN;
+    constexpr int TN = S::TN, TN8 = S::TN8, NACC = S::NACC, NB = L::NB, GR = L::GR, CB = L::CB, WIN = L::WIN;
     constexpr int PW = 4 * NG, MW = 4 * NG + 1;  // the planner's and the MMA issuer's warps
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* sA = smem + L::OFF_A;
@@ -387,10 +392,10 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
     float* sscr = reinterpret_cast<float*>(smem + L::OFF_SCR);
     float* sbuf = reinterpret_cast<float*>(smem + L::OFF_BUF);
     float* scen = reinterpret_cast<float*>(smem + L::OFF_CEN);
-    __shared__ uint64_t op_full[NB], op_empty[NB], gr_empty[GR], acc_full[2], acc_empty[2], never;
+    __shared__ uint64_t op_full[NB], op_empty[NB], gr_empty[GR], acc_full[NACC], acc_empty[NACC], never;
     __shared__ int ometa[NB];
     __shared__ long long s_handoff[NB];  // diagnostics: when the planner handed each slot over
-    __shared__ int2 amet[2];  // the tile in each accumulator: (table, columns), columns < 0 ends the block
+    __shared__ int2 amet[NACC];  // the tile in each accumulator: (table, columns), columns < 0 ends the block
     __shared__ uint32_t s_tmem;
     __shared__ int s_item;
     __shared__ ProbDev s_prob;
@@ -410,7 +415,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
             tc::mbar_init(&op_empty[i], 1);  // tcgen05.commit
         }
         for (int i = 0; i < GR; ++i) tc::mbar_init(&gr_empty[i], 4);  // the four epilogue warps
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < NACC; ++i) {
             tc::mbar_init(&acc_full[i], 2);   // tcgen05.commit + the issuer's arrival
             tc::mbar_init(&acc_empty[i], 4);  // the four epilogue warps
         }
@@ -418,7 +423,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
         tc::fence_mbar_init();
         s_fail = 0;
     }
-    if (warp == MW) tc::tmem_alloc(&s_tmem, 2 * TN);
+    if (warp == MW) tc::tmem_alloc(&s_tmem, NACC * TN);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -431,7 +436,9 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
     // of accumulator b, bit b of aused whether it was used (bit masks, not an
     // array: a dynamically indexed array would live in local memory)
     uint32_t aph = 0u, aused = 0u;
-    uint32_t acur = 0;                   // MMA issuer / each epilogue warp: the next accumulator
+    // MMA issuer / each epilogue warp: the next accumulator; tiles (and the
+    // markers that end a block) take them in turn, group g every NG-th
+    uint32_t acur = epi ? (uint32_t)grp_id : 0u;
 
     const ProbDev& P = s_prob;
     for (;;) {
@@ -729,7 +736,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
                                 tc::mbar_arrive(&acc_full[b], 2);
                                 aph ^= 1u << b;
                                 aused |= 1u << b;
-                                acur ^= 1u;
+                                acur = (acur + 1) % NACC;
                             }
                         }
                         if (!ok) {
@@ -765,7 +772,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
                     tc::mbar_arrive(&acc_full[b], 1);
                     aph ^= 1u << b;
                     aused |= 1u << b;
-                    acur ^= 1u;
+                    acur = (acur + 1) % NACC;
                 }
             }
             __syncwarp();
@@ -775,7 +782,6 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
             float* scr = sscr + grp_id * 32 * kQB + qt;
             float* bw = sbuf + grp_id * CB * kQB + qt;
             int32_t* bi = reinterpret_cast<int32_t*>(sbuf + NG * CB * kQB) + grp_id * CB * kQB + qt;
-            if (NG == 2) acur = (uint32_t)grp_id;  // group g reads accumulator g
             // insertion threshold in w units: below the list's last key and
             // inside the error band of the current k-th key (a key above the
             // band can never be a true k-nearest neighbour); it changes only
@@ -880,7 +886,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
                 const int2 am = amet[b];
                 aph ^= 1u << b;
                 aused |= 1u << b;
-                if (NG == 1) acur ^= 1u;
+                acur = (acur + NG) % NACC;
                 if (am.y < 0) {  // the end of the block
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(&acc_empty[b], 1);
@@ -1063,14 +1069,14 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
             for (uint32_t i = i0; i < otile; ++i) tc::mbar_wait(&op_full[i % NB], (i / NB) & 1u, kDrainPolls);
         }
         if (warp == MW && lane == 0)
-            for (int b = 0; b < 2; ++b)
+            for (int b = 0; b < NACC; ++b)
                 if ((aused >> b) & 1u) tc::mbar_wait(&acc_full[b], ((aph >> b) & 1u) ^ 1u, kDrainPolls);
         if (tid == 0) atomicExch(x.err, 1);
     }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    if (warp == MW) tc::tmem_dealloc(tmem, 2 * TN);
+    if (warp == MW) tc::tmem_dealloc(tmem, NACC * TN);
     if (n_skip) atomicAdd(&a.stats[ST_SKIPPED], n_skip);
     if (n_eval) atomicAdd(&a.stats[ST_EVALUATED], n_eval);
     if (n_pp) atomicAdd(&a.stats[ST_POINT_PAIRS], n_pp);
@@ -1078,7 +1084,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
     if (TC_TIMED && n_ins) atomicAdd(&x.timers[TT_INSERTS], n_ins);
 }
 
-// The kernel allocates 2 TN TMEM columns; at most one CTA may be resident per
+// The kernel allocates all of TMEM; at most one CTA may be resident per
 // SM: the request is raised above half the SM's shared memory.
 template <int FMT, int DP, int KC, int NG>
 inline size_t tc_smem_bytes() {
