@@ -1027,32 +1027,88 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
             if (ovf) {
                 a.fbq_list[atomicAdd(a.fbq_count, 1)] = make_int4(myq, blk, __float_as_int(ubk), 0);
             } else if (act) {
-                // float64 re-rank of the band candidates in shared memory
+                // exact order of the band's candidates, in shared memory:
+                // entry j is rk / rd[j kQB + qt] with its position ri[...]
+                uint64_t* rk = reinterpret_cast<uint64_t*>(smem);
                 double* rd = reinterpret_cast<double*>(smem);
                 int32_t* ri = reinterpret_cast<int32_t*>(smem + kQB * KC * 8);
                 const float* qp = P.qpts + (int64_t)myq * DP;
                 int nr = 0;
 #pragma unroll
-                for (int j = 0; j < KC; ++j) {
-                    if (li[j] != kEmptyIdx && !(ld[j] > band)) {
-                        rd[nr * kQB + qt] = exact_d2<DP>(qp, P.rpts + (int64_t)li[j] * DP);
-                        ri[nr * kQB + qt] = P.ridx[li[j]];
-                        ++nr;
-                    }
-                }
+                for (int j = 0; j < KC; ++j)
+                    if (li[j] != kEmptyIdx && !(ld[j] > band)) ri[nr++ * kQB + qt] = li[j];
                 n_re += nr;
                 const int64_t base = (int64_t)P.qidx[myq] * kq;
-                for (int j = 0; j < kq; ++j) {
-                    int best = j;
-                    for (int c = j + 1; c < nr; ++c)
-                        if (key_less(rd[c * kQB + qt], ri[c * kQB + qt], rd[best * kQB + qt], ri[best * kQB + qt]))
-                            best = c;
-                    const double bd = rd[best * kQB + qt];
-                    const int bix = ri[best * kQB + qt];
-                    rd[best * kQB + qt] = rd[j * kQB + qt];
-                    ri[best * kQB + qt] = ri[j * kQB + qt];
-                    P.out_idx[base + j] = bix;
-                    P.out_dist[base + j] = (float)sqrt(bd);
+                // pairs of float32 settle it unless two of them, or a distance
+                // and a rounding boundary, are too close; the band comes nearly
+                // sorted, so insertion moves little
+                bool sure = true;
+                {
+                    float q[DP];
+#pragma unroll
+                    for (int j4 = 0; j4 < DP / 4; ++j4) {
+                        const float4 v = reinterpret_cast<const float4*>(qp)[j4];
+                        q[4 * j4] = v.x;
+                        q[4 * j4 + 1] = v.y;
+                        q[4 * j4 + 2] = v.z;
+                        q[4 * j4 + 3] = v.w;
+                    }
+#pragma unroll 1
+                    for (int c = 0; c < nr; ++c) {
+                        const int pos = ri[c * kQB + qt];
+                        float h, l;
+                        sure &= pair_d2<DP>(q, P.rpts + (int64_t)pos * DP, h, l);
+                        const uint64_t v = ((uint64_t)f2o(h) << 32) | f2o(l);
+                        int j = c;
+                        for (; j > 0 && rk[(j - 1) * kQB + qt] > v; --j) {
+                            rk[j * kQB + qt] = rk[(j - 1) * kQB + qt];
+                            ri[j * kQB + qt] = ri[(j - 1) * kQB + qt];
+                        }
+                        rk[j * kQB + qt] = v;
+                        ri[j * kQB + qt] = pos;
+                    }
+                }
+                if (sure) {
+                    float ph = 0.f, pl = 0.f;
+                    for (int j = 0; j < nr && j <= kq; ++j) {
+                        const uint64_t v = rk[j * kQB + qt];
+                        const float h = o2f((uint32_t)(v >> 32)), l = o2f((uint32_t)v);
+                        // equal zeros are ties too
+                        if (j > 0 && !((h - ph) + (l - pl) > h * ((DP + 4) * 2.2737368e-13f))) sure = false;  // 2^-42
+                        ph = h;
+                        pl = l;
+                    }
+                }
+                if (sure) {
+                    for (int j = 0; j < kq; ++j) {
+                        const uint64_t v = rk[j * kQB + qt];
+                        const int pos = ri[j * kQB + qt];
+                        float dist;
+                        if (!pair_dist<DP>(o2f((uint32_t)(v >> 32)), o2f((uint32_t)v), dist))
+                            dist = (float)sqrt(exact_d2<DP>(qp, P.rpts + (int64_t)pos * DP));
+                        P.out_idx[base + j] = P.ridx[pos];
+                        P.out_dist[base + j] = dist;
+                    }
+                } else {
+                    // ties and near-ties: float64 throughout
+#pragma unroll 1
+                    for (int c = 0; c < nr; ++c) {
+                        const int pos = ri[c * kQB + qt];
+                        rd[c * kQB + qt] = exact_d2<DP>(qp, P.rpts + (int64_t)pos * DP);
+                        ri[c * kQB + qt] = P.ridx[pos];
+                    }
+                    for (int j = 0; j < kq; ++j) {
+                        int best = j;
+                        for (int c = j + 1; c < nr; ++c)
+                            if (key_less(rd[c * kQB + qt], ri[c * kQB + qt], rd[best * kQB + qt], ri[best * kQB + qt]))
+                                best = c;
+                        const double bd = rd[best * kQB + qt];
+                        const int bix = ri[best * kQB + qt];
+                        rd[best * kQB + qt] = rd[j * kQB + qt];
+                        ri[best * kQB + qt] = ri[j * kQB + qt];
+                        P.out_idx[base + j] = bix;
+                        P.out_dist[base + j] = (float)sqrt(bd);
+                    }
                 }
             }
             if (TC_TIMED && qt == 0)

@@ -139,6 +139,64 @@ __device__ __forceinline__ double exact_d2(const float* q, const float* r) {
     return s;
 }
 
+// The same sum in pairs of float32 (value h + l, |l| <= ulp(h) / 2), on the
+// FP32 pipe: this GPU's FP64 pipe does two operations per clock and SM, and the
+// re-rank's k x DP x 5 of them per query held up every work item (at d = 64,
+// k = 50 a fifth of the tile kernel's time).
+//   t = q_j - r_j exactly as th + tl; t^2 as a product and its remainder plus
+//   2 th tl; the running sum renormalised at each step.
+// With S the true sum, |h + l - S| <= (DP + 4) 2^-44 S: per step the remainder
+// terms round by at most 2 x 2^-46 of the running sum, tl^2 is left out (2^-48
+// of its term).  The float64 sum itself is within (DP + 2) 2^-53 S of S.
+// Returns false where the bound does not hold: a sum whose squares may have
+// underflowed or overflowed (zero is exact when every difference is zero).
+template <int DP>
+__device__ __forceinline__ bool pair_d2(const float (&q)[DP], const float* r, float& h, float& l) {
+    const float4* r4 = reinterpret_cast<const float4*>(r);
+    float sh = 0.f, sl = 0.f, mx = 0.f;
+#pragma unroll
+    for (int j4 = 0; j4 < DP / 4; ++j4) {
+        const float4 v = r4[j4];
+        const float rv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float a = q[4 * j4 + u], b = -rv[u];
+            const float th = __fadd_rn(a, b), bb = __fsub_rn(th, a);
+            const float tl = __fadd_rn(__fsub_rn(a, __fsub_rn(th, bb)), __fsub_rn(b, bb));
+            const float p = __fmul_rn(th, th);
+            const float e = __fmaf_rn(__fadd_rn(th, th), tl, __fmaf_rn(th, th, -p));
+            const float s = __fadd_rn(sh, p), sb = __fsub_rn(s, sh);
+            const float se = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, sb)), __fsub_rn(p, sb));
+            const float lo = __fadd_rn(sl, __fadd_rn(se, e));
+            sh = __fadd_rn(s, lo);
+            sl = __fsub_rn(lo, __fsub_rn(sh, s));
+            mx = fmaxf(mx, fabsf(th));
+        }
+    }
+    h = sh;
+    l = sl;
+    return (sh >= 1e-20f && sh <= 1e37f) || mx == 0.f;
+}
+
+// The float32 distance of a float64 squared distance D known as h + l within
+// (DP + 4) 2^-44 D: (float)sqrt(D) as float64 rounds it, or false where D is
+// too close to a rounding boundary to tell.
+template <int DP>
+__device__ __forceinline__ bool pair_dist(float h, float l, float& out) {
+    out = 0.f;
+    if (h == 0.f) return true;
+    const float s0 = __fsqrt_rn(h);
+    // sqrt(h + l) = s0 + c, c small and known to 2^-22 of itself
+    const float c = __fmul_rn(__fadd_rn(__fmaf_rn(-s0, s0, h), l), __fdiv_rn(0.5f, s0));
+    const float f = __fadd_rn(s0, c);
+    const float e = __fsub_rn(c, __fsub_rn(f, s0));  // what the rounding to f left out
+    const float half = 0.5f * (__uint_as_float(__float_as_uint(f) + 1u) - f);
+    out = f;
+    // (a power of two has a nearer boundary below: left to float64)
+    return (__float_as_uint(f) & 0x7fffffu) != 0u &&
+           half - fabsf(e) > f * ((DP + 4) * 1.1368684e-13f);  // 2^-43
+}
+
 template <typename T, int DP>
 __device__ __forceinline__ float ub_of(T kth) {
     if (sizeof(T) == 8) return __double2float_ru(__dsqrt_ru((double)kth));
