@@ -130,6 +130,16 @@ struct TcSmem {
     static_assert(S::TN8 * 8 == S::TN && S::TN8 <= 32, "tiles hold whole 8-row groups, one per lane");
 };
 
+// An upper bound on sqrt(x), x >= 0, in three instructions: the approximate
+// root is within 2^-22 of itself (and flushes what is below 1.2e-38 to zero).
+// The bounds below are recomputed at every insertion that moves a k-th key;
+// directed square roots were a third of that code.
+__device__ __forceinline__ float sqrt_up(float x) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return __fmaf_ru(r, 1.f + 4.7683716e-07f, 1.2e-19f);
+}
+
 template <int FMT, int DP>
 struct TcBound {
     static constexpr float u = 5.9604645e-08f;
@@ -141,10 +151,10 @@ struct TcBound {
     // upper bound on the true k-th distance of a query with k-th key S
     __device__ static float ub(float S, float a) {
         if (!(S < INFINITY)) return INFINITY;
-        float sq = __fsqrt_ru(fmaxf(S, 0.f));
+        float sq = sqrt_up(fmaxf(S, 0.f));
         float bb = __fmul_ru(1.03f, __fadd_ru(a, sq));
         float n2 = __fmaf_ru(a, a, __fmul_ru(bb, bb));
-        float r = __fsqrt_ru(__fmaf_ru(alpha, n2, S));
+        float r = sqrt_up(fmaxf(__fmaf_ru(alpha, n2, S), 0.f));
         return __fmaf_ru(e1, __fadd_ru(a, bb), r);
     }
     // band: every true k-nearest neighbour has a key <= band(ub, a)
@@ -786,10 +796,9 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
             // inside the error band of the current k-th key (a key above the
             // band can never be a true k-nearest neighbour); it changes only
             // when the list does
-            // the list's k-th entry, kept at hand: it changes only when an
+            // the list's k-th key, kept at hand: it changes only when an
             // insertion lands before it
             float kd = list_at(ld, kq - 1);
-            int ki = list_at(li, kq - 1);
             auto threshold = [&]() {
                 const float bnd = Bd::band(fminf(Bd::ub(kd, qa), qc), qa);
                 return __fsub_ru(fminf(ld[KC - 1], bnd), qn);
@@ -804,13 +813,12 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
                     const float sv = qn + bw[e * kQB];
                     const int rp = bi[e * kQB];
                     // (the cap pass may have listed this point already)
-                    if (key_less(sv, rp, ld[KC - 1], li[KC - 1]) && !(mono && rp == myq) && !listed(li, rp)) {
+                    if (sv < ld[KC - 1] && !(mono && rp == myq) && !listed(li, rp)) {
                         // the band moves only when the k-th key does
-                        const bool kth_moves = key_less(sv, rp, kd, ki);
-                        list_insert_par(ld, li, sv, rp);
+                        const bool kth_moves = sv < kd;
+                        list_insert_key(ld, li, sv, rp);
                         if (kth_moves) {
                             kd = list_at(ld, kq - 1);
-                            ki = list_at(li, kq - 1);
                             t = threshold();
                         } else {
                             t = fminf(t, __fsub_ru(ld[KC - 1], qn));
@@ -845,9 +853,24 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
                 }
                 if (!(mm <= t)) return;  // per-lane control flow only: no warp collective inside
                 if (TC_TIMED) atomicAdd(&x.timers[TT_EPI_RARE], 1ull);
-                uint32_t m = 0;
+                // which of them pass, in four chains
+                uint32_t m4[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-                for (int i = 0; i < 32; ++i) m |= (__uint_as_float(v[i]) <= t ? 1u : 0u) << i;
+                for (int i = 0; i < 32; ++i) m4[i & 3] |= (__uint_as_float(v[i]) <= t ? 1u : 0u) << i;
+                uint32_t m = (m4[0] | m4[1]) | (m4[2] | m4[3]);
+                auto take = [&](int i, float w) {
+                    const int cidx = cb + i;
+                    const int2 gq = grp[cidx >> 3];
+                    const int r = cidx & 7;
+                    bw[nb * kQB] = w;
+                    bi[nb * kQB] = r < gq.y ? gq.x + r : kEmptyIdx;
+                    ++nb;
+                };
+                if ((m & (m - 1)) == 0 && nb < CB) {
+                    // one key (by far the most common): it is the minimum
+                    take(__ffs(m) - 1, mm);
+                    return;
+                }
 #pragma unroll
                 for (int i = 0; i < 32; ++i) scr[i * kQB] = __uint_as_float(v[i]);
                 while (m) {
@@ -859,12 +882,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
                         flush();
                         if (!(w <= t)) continue;
                     }
-                    const int cidx = cb + i;
-                    const int2 gq = grp[cidx >> 3];
-                    const int r = cidx & 7;
-                    bw[nb * kQB] = w;
-                    bi[nb * kQB] = r < gq.y ? gq.x + r : kEmptyIdx;
-                    ++nb;
+                    take(i, w);
                 }
             };
             int since_pub = 0;

@@ -56,26 +56,23 @@ __device__ __forceinline__ void list_insert(T (&ld)[KC], int (&li)[KC], T d, int
     }
 }
 
-// The same insertion without a serial chain: every comparison against the
-// new key is independent (the list is sorted, so the smaller entries form a
-// prefix), then each slot either keeps its entry, takes the new one or takes
-// its predecessor.  Descending order reads each predecessor before it moves.
-template <typename T, int KC>
-__device__ __forceinline__ void list_insert_par(T (&ld)[KC], int (&li)[KC], T d, int i) {
-    bool lt[KC];
+// The same insertion by key alone and without a serial chain: every
+// comparison against the new key is independent, then each slot either keeps
+// its entry, takes the new one or takes its predecessor (descending order
+// reads each predecessor before it moves).  Entries of equal keys stay in the
+// order they came: the tensor-core lists' order among them never matters,
+// since the re-rank settles it and a band that reaches the last key overflows.
+template <int KC>
+__device__ __forceinline__ void list_insert_key(float (&ld)[KC], int (&li)[KC], float d, int i) {
 #pragma unroll
-    for (int j = 0; j < KC; ++j) lt[j] = key_less(ld[j], li[j], d, i);
-#pragma unroll
-    for (int j = KC - 1; j >= 0; --j) {
-        if (!lt[j]) {
-            if (j == 0 || lt[j - 1]) {
-                ld[j] = d;
-                li[j] = i;
-            } else {
-                ld[j] = ld[j - 1];
-                li[j] = li[j - 1];
-            }
-        }
+    for (int j = KC - 1; j > 0; --j) {
+        const bool here = d < ld[j], before = d < ld[j - 1];
+        li[j] = here ? (before ? li[j - 1] : i) : li[j];
+        ld[j] = here ? (before ? ld[j - 1] : d) : ld[j];
+    }
+    if (d < ld[0]) {
+        ld[0] = d;
+        li[0] = i;
     }
 }
 
