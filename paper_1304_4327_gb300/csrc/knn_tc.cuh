@@ -93,7 +93,7 @@ struct TcShape {
     // reference points per tile: 256 (the MMA's widest N) where the operand
     // slots fit shared memory
     static constexpr int TN = DP <= 16 ? 256 : 128;
-    static constexpr int TN8 = TN / 8;
+    static constexpr int TN8 = TN / 8;  // at most 32: a lane per group
     // accumulators: as many as TMEM's 512 columns hold
     static constexpr int NACC = 512 / TN;
     __host__ __device__ static constexpr int astep(int m) {
@@ -356,7 +356,7 @@ enum TcTimer {
 };
 static_assert(TT_N <= 32, "the diagnostic timer buffer holds 32 counters");
 
-// One persistent CTA per SM, 4 NG + 2 warps:
+// One persistent CTA per SM, 4 NG + 3 warps:
 //   warps 0 .. 4 NG - 1  NG epilogue groups of four warps: one query row (TMEM
 //              lane) per thread; each warp reads its own 32 lanes of an
 //              accumulator, examines the keys and keeps its queries' lists,
@@ -368,14 +368,17 @@ static_assert(TT_N <= 32, "the diagnostic timer buffer holds 32 counters");
 //              accumulators (TN = 128) let the MMAs run on while one of the
 //              four warps inserts: an accumulator is free only when all four
 //              have read it
-//   warp 4 NG  planner: prepares a window of the block's candidate leaves at
-//              a time (Algorithm 3's test against the block's bound, each
-//              kept leaf's range and its place in the window's run of 8-row
-//              groups), then fills operand slots with whole 8-row groups by
-//              bulk copies (TMA) of the leaves' operand rows, and a table of
-//              the groups' first rows (a ring of GR tables, deeper than the
-//              slots: a slot is free again once its MMAs are done)
-//   warp 4 NG + 1  MMA issuer: one thread turns a filled slot into an
+//   warps 4 NG, 4 NG + 1  planners: prepare a window of the block's candidate
+//              leaves at a time, half of it each (Algorithm 3's test against
+//              the block's bound, each kept leaf's range and its place in the
+//              window's run of 8-row groups), then in turn fill operand slots
+//              with whole 8-row groups by bulk copies (TMA) of the leaves'
+//              operand rows, and a table of the groups' first rows (a ring of
+//              GR tables, deeper than the slots: a slot is free again once its
+//              MMAs are done).  One planner took 1,650 cycles per tile of 256
+//              rows at d = 16, of which a copy's issue is about 75, and bound
+//              the kernel; two of them with a table built by shuffles do not
+//   warp 4 NG + 2  MMA issuer: one thread turns a filled slot into an
 //              accumulator with tcgen05.mma
 // Hand-over by mbarriers: op_full (planner -> MMA: its arrival plus the
 // copied bytes), acc_full (MMA -> epilogue: the MMA's commit plus the
@@ -386,12 +389,12 @@ static_assert(TT_N <= 32, "the diagnostic timer buffer holds 32 counters");
 // failed wait the item's work is abandoned, the kernel drains its own copies
 // and MMAs, releases TMEM and reports through x.err.
 template <int FMT, int DP, int KC, int NG>
-__global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs a, const TcExtra x) {
+__global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs a, const TcExtra x) {
     using S = TcShape<FMT, DP>;
     using L = TcSmem<FMT, DP, KC, NG>;
     using Bd = TcBound<FMT, DP>;
     constexpr int TN = S::TN, TN8 = S::TN8, NACC = S::NACC, NB = L::NB, GR = L::GR, CB = L::CB, WIN = L::WIN;
-    constexpr int PW = 4 * NG, MW = 4 * NG + 1;  // the planner's and the MMA issuer's warps
+    constexpr int PW = 4 * NG, MW = 4 * NG + 2;  // the first planner's and the MMA issuer's warps
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* sA = smem + L::OFF_A;
     unsigned char* sB = smem + L::OFF_B;
@@ -411,6 +414,8 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
     __shared__ ProbDev s_prob;
     __shared__ volatile int s_fail;
     __shared__ volatile float s_wmax[4 * NG], s_wmin[4 * NG];
+    __shared__ int s_pk[2], s_pg[2];     // each planner's kept leaves and their groups in the window
+    __shared__ int s_pfail[2];           // a planner gave up in an earlier window
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool epi = warp < 4 * NG;
@@ -432,6 +437,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
         tc::mbar_init(&never, 1);  // nothing arrives on it (the stall diagnostic)
         tc::fence_mbar_init();
         s_fail = 0;
+        s_pfail[0] = s_pfail[1] = 0;
     }
     if (warp == MW) tc::tmem_alloc(&s_tmem, NACC * TN);
     tc::fence_before_sync();
@@ -440,8 +446,9 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
     const uint32_t tmem = s_tmem;
     const uint32_t idesc = tc::idesc(TcFmt<FMT>::hw, kQB, TN);
     // the barriers' phases carry over from item to item, so the counters do too
-    uint32_t otile = 0;                  // planner / MMA issuer: operand slot uses
-    uint32_t gtile = 0;                  // planner / MMA issuer: tiles (row-group table uses)
+    uint32_t otile = 0;                  // planners / MMA issuer: operand slot uses
+    uint32_t gtile = 0;                  // planners / MMA issuer: tiles (row-group table uses)
+    uint32_t olast = 0;                  // planners: one past the last slot use this planner filled
     // MMA issuer / each epilogue warp: bit b of aph is the parity of the uses
     // of accumulator b, bit b of aused whether it was used (bit masks, not an
     // array: a dynamically indexed array would live in local memory)
@@ -531,8 +538,9 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
             atomicAdd(&x.timers[TT_ITEMS], 1ull);
         }
 
-        if (warp == PW) {
-            // ================= planner =================
+        if (warp == PW || warp == PW + 1) {
+            // ================= planners =================
+            const int pl = warp - PW;
             const float Bq = a.Bn ? a.Bn[P.node0 + qnode] : INFINITY;
             const int64_t c0 = a.csr_off[blk], c1 = a.csr_off[blk + 1];
             // the candidates: the block's proposed cells the seed pass left
@@ -542,14 +550,18 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
             const int64_t ntot = npro + (c1 - c0);
             const unsigned char* rops = static_cast<const unsigned char*>(P.rops);
             const int64_t ls8 = P.rls8;
-            bool fail = false;
+            constexpr int NR = WIN / 64;  // a planner prepares every second 32 entries of a window
+            bool fail = false, quit = false;
             // window w's leaves and d_min land in buffer w & 1 by cp.async,
-            // issued while the previous window is processed
+            // issued while the previous window is processed (each planner
+            // fetches the entries it prepares)
             auto fetch = [&](int64_t w0, int buf) {
                 const int wn = (int)(ntot - w0 < WIN ? ntot - w0 : WIN);
-                for (int i = lane; i < wn; i += 32) {
+#pragma unroll
+                for (int r = 0; r < NR; ++r) {
+                    const int i = (pl * NR + r) * 32 + lane;
                     const int64_t ci = w0 + i - npro;  // entry of the traversal's list
-                    if (ci >= 0) {
+                    if (i < wn && ci >= 0) {
                         tc::cp_async4(swleaf + buf * WIN + i, a.csr_leaf + c0 + ci);
                         tc::cp_async4(swdmin + buf * WIN + i, a.csr_dmin + c0 + ci);
                     }
@@ -558,7 +570,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
             };
             if (ntot > 0) fetch(0, 0);
             int wbuf = 0;
-            for (int64_t w0 = 0; w0 < ntot && !fail; w0 += WIN, wbuf ^= 1) {
+            for (int64_t w0 = 0; w0 < ntot; w0 += WIN, wbuf ^= 1) {
                 const int wn = (int)(ntot - w0 < WIN ? ntot - w0 : WIN);
                 long long t0 = TC_TIMED ? clock64() : 0;
                 tc::cp_async_wait_all();
@@ -580,11 +592,10 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
                 // exceeds the bound is pruned), their ranges, and where each
                 // starts in the window's run of 8-row groups
                 // (every entry's range is read first, so the loads overlap)
-                constexpr int NR = WIN / 32;
                 int eleaf[NR], ebeg[NR], ecnt[NR];
 #pragma unroll
                 for (int r = 0; r < NR; ++r) {
-                    const int i = r * 32 + lane;
+                    const int i = (pl * NR + r) * 32 + lane;
                     const bool pro = w0 + i < npro;  // a proposed cell's leaf (never pruned)
                     const bool keep = i < wn && (pro || !(swdmin[wbuf * WIN + i] > b));
                     eleaf[r] = !keep ? -1
@@ -593,35 +604,56 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
                     ebeg[r] = keep ? P.rbeg[P.rleaf0 + eleaf[r]] : 0;
                     ecnt[r] = keep ? P.rcnt[P.rleaf0 + eleaf[r]] : 0;
                 }
-                int G = 0;
+                // this planner's part: places among its own kept leaves
+                int G = 0, K = 0, rows = 0;
+                int eg[NR], ek[NR];
 #pragma unroll
                 for (int r = 0; r < NR; ++r) {
-                    const int i = r * 32 + lane;
-                    const bool valid = i < wn;
                     const int g = (ecnt[r] + 7) >> 3;
-                    int4 e = make_int4(ebeg[r], ecnt[r], eleaf[r], 0);
                     int incl = g;
 #pragma unroll
                     for (int off = 1; off < 32; off <<= 1) {
                         const int v = __shfl_up_sync(0xffffffffu, incl, off);
                         if (lane >= off) incl += v;
                     }
-                    e.w = G + incl - g;
-                    if (valid) went[i] = e;
-                    const unsigned kept = __ballot_sync(0xffffffffu, valid && g > 0);
-                    const unsigned all = __ballot_sync(0xffffffffu, valid);
-                    if (lane == 0) {
-                        n_eval += __popc(kept);
-                        n_skip += __popc(all & ~kept);
-                    }
+                    const unsigned kept = __ballot_sync(0xffffffffu, g > 0);
+                    eg[r] = G + incl - g;
+                    ek[r] = K + __popc(kept & ((1u << lane) - 1u));
                     G += __shfl_sync(0xffffffffu, incl, 31);
+                    K += __popc(kept);
+                    rows += ecnt[r];
                 }
-                __syncwarp();
-                if (TC_TIMED && lane == 0)
+                rows = __reduce_add_sync(0xffffffffu, rows);
+                if (lane == 0) {
+                    const int mine = max(0, min(wn - pl * NR * 32, NR * 32));
+                    n_eval += K;
+                    n_skip += mine - K;
+                    n_pp += (unsigned long long)rows * nq;
+                    s_pk[pl] = K;
+                    s_pg[pl] = G;
+                    if (fail) s_pfail[pl] = 1;
+                }
+                // both planners are done with the previous window's entries
+                tc::named_sync(2, 64);
+                // (read between the two barriers, written before the first:
+                // both planners see the same)
+                quit = s_pfail[0] || s_pfail[1];
+                const int k0 = pl ? s_pk[0] : 0, gg0 = pl ? s_pg[0] : 0;
+                const int nk = s_pk[0] + s_pk[1];
+                G = s_pg[0] + s_pg[1];
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+                    if (ecnt[r] > 0) went[k0 + ek[r]] = make_int4(ebeg[r], ecnt[r], eleaf[r], gg0 + eg[r]);
+                tc::named_sync(2, 64);
+                if (quit) break;
+                if (TC_TIMED && pl == 0 && lane == 0)
                     atomicAdd(&x.timers[TT_PLAN_WINDOW], (unsigned long long)(clock64() - t0));
-                // tiles of TN8 groups; the entries overlapping a tile are consecutive
+                // tiles of TN8 groups, every second one this planner's; the
+                // entries overlapping a tile are consecutive, and no more than
+                // its groups
                 int cur = 0;
-                for (int g0 = 0; g0 < G; g0 += TN8) {
+                for (int g0 = 0; g0 < G; g0 += TN8, ++otile, ++gtile) {
+                    if ((int)(otile & 1u) != pl || fail) continue;
                     const int g1 = min(g0 + TN8, G);
                     const int op = (int)(otile % NB);
                     const uint32_t use = otile / NB;
@@ -632,66 +664,65 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
                                                     tc::mbar_wait(&gr_empty[gi], (guse & 1u) ^ 1u, x.spin_budget)
                                               : true;
                     if (!__all_sync(0xffffffffu, ok)) {
-                        if (lane == 0) TC_FAIL_SITE(FS_PLAN_SLOT);
+                        if (lane == 0) {
+                            TC_FAIL_SITE(FS_PLAN_SLOT);
+                            s_fail = 1;
+                        }
                         fail = true;
-                        break;
+                        continue;
                     }
                     long long t2 = TC_TIMED ? clock64() : 0;
                     if (lane == 0) tc::mbar_expect_tx(&op_full[op], (uint32_t)(g1 - g0) * S::GB);
                     __syncwarp();
-                    unsigned char* slot = sB + op * TN * S::RB;
-                    int2* grp = sgrp + gi * TN8;
+                    // the first entry that reaches into the tile
+                    int4 e;
+                    int gs, ge;
                     for (;;) {
                         const int i = cur + lane;
-                        const bool valid = i < wn;
-                        const int4 e = valid ? went[i] : make_int4(0, 0, 0, 0x7fffffff);
-                        const int gs = e.w, gg = (e.y + 7) >> 3;
-                        const int lo = max(gs, g0), hi = min(gs + gg, g1);
-                        int real = 0;
-                        const long long tcp = TC_TIMED ? clock64() : 0;
-                        if (valid && hi > lo)
-                            tc::bulk_g2s(slot + (lo - g0) * S::GB,
-                                         rops + ((int64_t)e.z * ls8 + (lo - gs)) * S::GB,
-                                         (uint32_t)(hi - lo) * S::GB, &op_full[op]);
-                        if (TC_TIMED) {
-                            __syncwarp();
-                            if (lane == 0) atomicAdd(&x.timers[TT_PLAN_COPY], (unsigned long long)(clock64() - tcp));
-                        }
-                        if (valid && hi > lo) {
-                            for (int q = lo; q < hi; ++q) {
-                                const int r0 = 8 * (q - gs);
-                                grp[q - g0] = make_int2(e.x + r0, min(8, e.y - r0));
-                            }
-                            real = min(e.y, 8 * (hi - gs)) - 8 * (lo - gs);
-                        }
-                        real = __reduce_add_sync(0xffffffffu, real);
-                        if (lane == 0) n_pp += (unsigned long long)real * nq;
-                        // entries that end within this tile are done; they form a prefix
-                        const unsigned fin = __ballot_sync(0xffffffffu, valid && gs + gg <= g1);
-                        const int adv = fin == 0xffffffffu ? 32 : __ffs(~fin) - 1;
+                        e = i < nk ? went[i] : make_int4(0, 0, 0, 0x3fffffff);
+                        gs = e.w;
+                        ge = gs + ((e.y + 7) >> 3);
+                        const int adv = __popc(__ballot_sync(0xffffffffu, ge <= g0));
+                        if (adv == 0) break;
                         cur += adv;
-                        if (adv < 32) break;
                     }
+                    const int lo = max(gs, g0), hi = min(ge, g1);
+                    const bool over = hi > lo;
+                    if (over)
+                        tc::bulk_g2s(sB + op * TN * S::RB + (lo - g0) * S::GB,
+                                     rops + ((int64_t)e.z * ls8 + (lo - gs)) * S::GB, (uint32_t)(hi - lo) * S::GB,
+                                     &op_full[op]);
                     if (lane == 0) ometa[op] = (g1 - g0) * 8;
+                    // the row-group table: lane l describes group g0 + l, of
+                    // the last entry that starts at or before it
+                    const unsigned starts = __reduce_or_sync(0xffffffffu, over ? 1u << (lo - g0) : 0u);
+                    const int from = __popc(starts & ((2u << lane) - 1u)) - 1;
+                    const int fb = __shfl_sync(0xffffffffu, e.x, from & 31);
+                    const int fc = __shfl_sync(0xffffffffu, e.y, from & 31);
+                    const int fg = __shfl_sync(0xffffffffu, gs, from & 31);
+                    if (g0 + lane < g1) {
+                        const int r0 = 8 * (g0 + lane - fg);
+                        sgrp[gi * TN8 + lane] = make_int2(fb + r0, min(8, fc - r0));
+                    }
                     __syncwarp();
                     if (lane == 0) {
                         if (TC_TIMED) s_handoff[op] = clock64();
                         tc::mbar_arrive(&op_full[op], 1);
-                        if (TC_TIMED) {
-                            atomicAdd(&x.timers[TT_TILES], 1ull);
+                        if (TC_TIMED) atomicAdd(&x.timers[TT_TILES], 1ull);
+                        if (TC_TIMED && pl == 0) {
                             atomicAdd(&x.timers[TT_PLAN_WAIT], (unsigned long long)(t2 - t1));
                             atomicAdd(&x.timers[TT_PLAN_STAGE], (unsigned long long)(clock64() - t2));
                         }
                     }
-                    ++otile;
-                    ++gtile;
+                    olast = otile + 1;
                 }
             }
             // a window fetch still in flight (after a failure) lands before the
             // buffers can be reused
             tc::cp_async_wait_all();
             __syncwarp();
-            if (x.stall && !fail) {
+            fail |= quit;
+            if (x.stall && !fail && pl == 0) {
                 // diagnostics: a wait that nothing ends, which must give up
                 // after spin_budget polls and fail the call
                 const bool ok = lane == 0 ? tc::mbar_wait(&never, 0u, x.spin_budget) : true;
@@ -700,8 +731,8 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
                     fail = true;
                 }
             }
-            // the end of the block
-            if (!fail) {
+            // the end of the block, marked by the planner whose turn it is
+            if (!fail && (int)(otile & 1u) == pl) {
                 const int op = (int)(otile % NB);
                 const uint32_t use = otile / NB;
                 const bool ok = lane == 0 ? tc::mbar_wait(&op_empty[op], (use & 1u) ^ 1u, x.spin_budget) : true;
@@ -710,12 +741,13 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
                         ometa[op] = -1;
                         tc::mbar_arrive(&op_full[op], 1);
                     }
-                    ++otile;
+                    olast = otile + 1;
                 } else {
                     if (lane == 0) TC_FAIL_SITE(FS_PLAN_END);
                     fail = true;
                 }
             }
+            ++otile;
             if (fail && lane == 0) s_fail = 1;
         } else if (warp == MW) {
             // ================= MMA issuer (one thread) =================
@@ -1136,11 +1168,13 @@ __global__ void __launch_bounds__(32 * (4 * NG + 2), 1) k_tile_tc(const TileArgs
     }
     if (s_fail) {
         // drain this CTA's own asynchronous work before TMEM and shared
-        // memory are released: the planner's last NB slot fills (their bulk
+        // memory are released: the planners' last NB slot fills (their bulk
         // copies) and the issuer's MMAs
-        if (warp == PW && lane == 0) {
-            const uint32_t i0 = otile > (uint32_t)NB ? otile - NB : 0u;
-            for (uint32_t i = i0; i < otile; ++i) tc::mbar_wait(&op_full[i % NB], (i / NB) & 1u, kDrainPolls);
+        if ((warp == PW || warp == PW + 1) && lane == 0) {
+            // (a planner's slot uses are those of its parity before olast)
+            const uint32_t i0 = olast > (uint32_t)NB ? olast - NB : 0u;
+            for (uint32_t i = i0; i < olast; ++i)
+                if ((int)(i & 1u) == warp - PW) tc::mbar_wait(&op_full[i % NB], (i / NB) & 1u, kDrainPolls);
         }
         if (warp == MW && lane == 0)
             for (int b = 0; b < NACC; ++b)
@@ -1211,7 +1245,7 @@ int launch_tile_tc(const TileArgs& a, int fmt, int kc, int items, int* err, int 
         size_t smem = tc_smem_bytes<FMTV, DP, KCV, NGV>();                                 \
         DT_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                                       (int)smem));                                         \
-        const int nt = 32 * (4 * NGV + 2);                                                 \
+        const int nt = 32 * (4 * NGV + 3);                                                 \
         int g = occupancy_grid((const void*)kern, nt, smem);                               \
         if (items < g) g = items > 0 ? items : 1;                                          \
         DT_LAUNCH(kern, g, nt, smem, s, a, x);                                             \
