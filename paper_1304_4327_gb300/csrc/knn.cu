@@ -950,10 +950,21 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
     a.csr_dmin = csr_dmin;
     a.Bn = Bn;
     a.work_ctr = ctr + 1;
-    if (fmt)
-        DT_TRY(launch_tile_tc<DP>(a, fmt, KC, NI, derr, spin, s));
-    else
+    if (fmt) {
+        // chunks in pairs where most queries sit in blocks of several chunks
+        // and the pairs still fill the GPU
+        int64_t paired = 0, pairs = 0;
+        for (int i = 0; i < np; ++i) {
+            if (pd[i].cpb > 1) paired += hp[i].tq->n;
+            pairs += (int64_t)pd[i].nblocks * ((pd[i].cpb + 1) / 2);
+        }
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        DT_TRY(launch_tile_tc<DP>(a, fmt, KC, NI, 2 * paired >= NQ && pairs >= 2 * sms, derr, spin, s));
+    } else {
         DT_TRY(launch_tile_cc<DP>(a, KC, MODE_MAIN, NI, s));
+    }
     tm.mark();  // 3
     int nfb = 0, herr = 0;
     DT_CHECK(cudaMemcpyAsync(&nfb, ctr + 3, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -175,9 +175,10 @@ int launch_query_cap(const TileArgs& a, int kc, int budget, float* qcap, cudaStr
 template <int DP>
 int launch_query_fb(const TileArgs& a, int kc, int nfbq, bool exact, cudaStream_t s);
 
-// The tensor-core BaseCase pass (main mode): fmt 1 = BF16 (split), 2 = TF32.
+// The tensor-core BaseCase pass (main mode): fmt 1 = BF16 (split), 2 = TF32;
+// wide: a block's chunks are taken two at a time.
 template <int DP>
-int launch_tile_tc(const TileArgs& a, int fmt, int kc, int items, int* err, int spin,
+int launch_tile_tc(const TileArgs& a, int fmt, int kc, int items, bool wide, int* err, int spin,
                    cudaStream_t s);
 
 // Bytes per operand row, and the fill of a reference tree's operand array

@@ -1,8 +1,9 @@
 // knn_tc.cuh -- the kNN BaseCase (Algorithm 2) on the tensor cores.
 //
 // A work item is a chunk of <= 128 queries of a query block (one TMEM lane
-// and one epilogue thread each); the chunks of a block share its candidate
-// leaves.  Every point is centred on one point c, the centre
+// and one epilogue thread each), or two such chunks (QH = 2), whose halves
+// share every operand tile: half the operand bytes, bulk copies and planning
+// per pair.  The chunks of a block share its candidate leaves.  Every point is centred on one point c, the centre
 // of the reference tree's root box, and rounded to the MMA's input type:
 //   - reference points once per tree and format (k_tc_ops), into an operand
 //     array laid out exactly as the tiles sit in shared memory (8-row groups
@@ -90,12 +91,6 @@ struct TcShape {
     static constexpr int GB = 8 * RB;                   // bytes per 8-row group (the SBO)
     static constexpr int KP = NK * kstep;               // MMA depth
     static constexpr int EPC = 16 / TcFmt<FMT>::esize;  // elements per chunk
-    // reference points per tile: 256 (the MMA's widest N) where the operand
-    // slots fit shared memory
-    static constexpr int TN = DP <= 16 ? 256 : 128;
-    static constexpr int TN8 = TN / 8;  // at most 32: a lane per group
-    // accumulators: as many as TMEM's 512 columns hold
-    static constexpr int NACC = 512 / TN;
     __host__ __device__ static constexpr int astep(int m) {
         return !REUSE ? m : m < 2 * H ? m : m < 3 * H ? m - 2 * H : 2 * H;
     }
@@ -104,30 +99,38 @@ struct TcShape {
     }
 };
 
-// Shared memory of the tile kernel (bytes): NG epilogue groups, lists of KC.
-template <int FMT, int DP, int KC, int NG>
+// Shared memory of the tile kernel (bytes): NG epilogue groups, lists of KC,
+// QH x 128 queries per item.
+template <int FMT, int DP, int KC, int NG, int QH>
 struct TcSmem {
     using S = TcShape<FMT, DP>;
-    static constexpr int NB = 4;                                     // operand slots
-    static constexpr int GR = 8;                                     // row-group tables (a ring)
+    // reference points per tile: 256 (the MMA's widest N) where the operand
+    // slots fit shared memory and one half of 128 queries leaves two
+    // accumulators in TMEM's 512 columns; else 128, with four accumulators
+    static constexpr int TN = DP <= 16 && QH == 1 ? 256 : 128;
+    static constexpr int TN8 = TN / 8;                               // at most 32: a lane per group
+    static constexpr int NACC = 512 / TN;
+    // operand slots: about 100 KB of them
+    static constexpr int NB = QH == 1 ? 4 : DP <= 16 ? 8 : DP == 32 ? 4 : 3;
+    static constexpr int GR = 2 * NB;                                // row-group tables (a ring)
     static constexpr int WIN = 256;                                  // candidates per window
     static constexpr int CB = 8;                                     // deferred insertions per thread
-    static constexpr int OFF_A = 0;                                  // 128 x RB
-    static constexpr int OFF_B = OFF_A + kQB * S::RB;                // NB x TN x RB
-    static constexpr int OFF_GRP = OFF_B + NB * S::TN * S::RB;       // GR x TN8 int2 (row groups)
-    static constexpr int OFF_WIN = OFF_GRP + GR * S::TN8 * 8;        // 2 x WIN (leaf int, d_min float)
+    static constexpr int OFF_A = 0;                                  // QH x 128 x RB
+    static constexpr int OFF_B = OFF_A + QH * kQB * S::RB;           // NB x TN x RB
+    static constexpr int OFF_GRP = OFF_B + NB * TN * S::RB;          // GR x TN8 int2 (row groups)
+    static constexpr int OFF_WIN = OFF_GRP + GR * TN8 * 8;           // 2 x WIN (leaf int, d_min float)
     static constexpr int OFF_WENT = OFF_WIN + 2 * WIN * 8;           // WIN int4 (begin, count, leaf, group0)
-    static constexpr int OFF_SCR = OFF_WENT + WIN * 16;              // NG x 32 x 128 float
-    static constexpr int OFF_BUF = OFF_SCR + NG * 32 * kQB * 4;      // NG x CB x 128 (float, int)
+    static constexpr int OFF_BUF = OFF_WENT + WIN * 16;              // NG x CB x 128 (float, int)
     static constexpr int OFF_CEN = OFF_BUF + NG * CB * kQB * 8;      // DP float
     static constexpr int END = OFF_CEN + DP * 4;
     // at a block's end everything above is idle: the merge of two groups'
     // lists (float + int per entry) and the float64 re-rank (double + int per
     // entry) reuse it from offset 0
-    static constexpr int FIN = kQB * KC * 12;
+    static constexpr int FIN = QH * kQB * KC * 12;
     static constexpr int BYTES = END > FIN ? END : FIN;
     static_assert(BYTES <= 225 * 1024, "tensor-core tile shared memory over budget");
-    static_assert(S::TN8 * 8 == S::TN && S::TN8 <= 32, "tiles hold whole 8-row groups, one per lane");
+    static_assert(TN8 * 8 == TN && TN8 <= 32, "tiles hold whole 8-row groups, one per lane");
+    static_assert(QH == 1 || (QH == NG && NACC == 4), "a group per half, two accumulators each");
 };
 
 // An upper bound on sqrt(x), x >= 0, in three instructions: the approximate
@@ -388,12 +391,13 @@ static_assert(TT_N <= 32, "the diagnostic timer buffer holds 32 counters");
 // row-group table is read).  Every wait is bounded; after a
 // failed wait the item's work is abandoned, the kernel drains its own copies
 // and MMAs, releases TMEM and reports through x.err.
-template <int FMT, int DP, int KC, int NG>
+template <int FMT, int DP, int KC, int NG, int QH>
 __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs a, const TcExtra x) {
     using S = TcShape<FMT, DP>;
-    using L = TcSmem<FMT, DP, KC, NG>;
+    using L = TcSmem<FMT, DP, KC, NG, QH>;
     using Bd = TcBound<FMT, DP>;
-    constexpr int TN = S::TN, TN8 = S::TN8, NACC = S::NACC, NB = L::NB, GR = L::GR, CB = L::CB, WIN = L::WIN;
+    constexpr int TN = L::TN, TN8 = L::TN8, NACC = L::NACC, NB = L::NB, GR = L::GR, CB = L::CB, WIN = L::WIN;
+    constexpr bool WIDE = NG == 1 || KC <= 24;  // 64-column reads
     constexpr int PW = 4 * NG, MW = 4 * NG + 2;  // the first planner's and the MMA issuer's warps
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* sA = smem + L::OFF_A;
@@ -402,7 +406,6 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
     int32_t* swleaf = reinterpret_cast<int32_t*>(smem + L::OFF_WIN);
     float* swdmin = reinterpret_cast<float*>(smem + L::OFF_WIN + 2 * WIN * 4);
     int4* went = reinterpret_cast<int4*>(smem + L::OFF_WENT);
-    float* sscr = reinterpret_cast<float*>(smem + L::OFF_SCR);
     float* sbuf = reinterpret_cast<float*>(smem + L::OFF_BUF);
     float* scen = reinterpret_cast<float*>(smem + L::OFF_CEN);
     __shared__ uint64_t op_full[NB], op_empty[NB], gr_empty[GR], acc_full[NACC], acc_empty[NACC], never;
@@ -421,6 +424,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
     const bool epi = warp < 4 * NG;
     const int grp_id = warp >> 2;  // an epilogue thread's group
     const int qt = tid & 127;  // query row of an epilogue thread
+    const int half = QH == 2 ? grp_id : 0;  // and its half of the item's queries
     const int nitems = a.nitems;
     unsigned long long n_skip = 0, n_eval = 0, n_pp = 0, n_re = 0, n_ins = 0;
 
@@ -429,7 +433,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
             tc::mbar_init(&op_full[i], 1);   // the planner's arrival (+ copied bytes)
             tc::mbar_init(&op_empty[i], 1);  // tcgen05.commit
         }
-        for (int i = 0; i < GR; ++i) tc::mbar_init(&gr_empty[i], 4);  // the four epilogue warps
+        for (int i = 0; i < GR; ++i) tc::mbar_init(&gr_empty[i], 4 * QH);  // the epilogue warps that read a tile
         for (int i = 0; i < NACC; ++i) {
             tc::mbar_init(&acc_full[i], 2);   // tcgen05.commit + the issuer's arrival
             tc::mbar_init(&acc_empty[i], 4);  // the four epilogue warps
@@ -454,8 +458,10 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
     // array: a dynamically indexed array would live in local memory)
     uint32_t aph = 0u, aused = 0u;
     // MMA issuer / each epilogue warp: the next accumulator; tiles (and the
-    // markers that end a block) take them in turn, group g every NG-th
+    // markers that end a block) take them in turn, group g every NG-th.  With
+    // QH = 2 a tile takes one of each group's, and the issuer keeps both turns
     uint32_t acur = epi ? (uint32_t)grp_id : 0u;
+    uint32_t acur1 = 1u;                 // MMA issuer, QH = 2: the next one of group 1
 
     const ProbDev& P = s_prob;
     for (;;) {
@@ -469,17 +475,20 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
         const int2 wi = a.items[item];
         const int blk = wi.x, chunk = wi.y;  // global block, chunk of its queries
         const int64_t qnode = P.qblock0 + (blk - P.block0);
-        const int nq = min(kQB, P.qcnt[qnode] - chunk * kQB);
+        // (work items are numbered by chunks of 128: with QH = 2 the even ones
+        // stand for themselves and the next)
+        const int nq = QH == 2 && (chunk & 1) ? 0 : min(QH * kQB, P.qcnt[qnode] - chunk * kQB);
         if (nq <= 0) {
             __syncthreads();
             continue;
         }
+        const bool both = QH == 2 && nq > kQB;  // the second half holds queries
         long long tm0 = TC_TIMED ? clock64() : 0;
         // the centring point: the reference root box's centre, as k_tc_ops used it
         if (tid < DP) scen[tid] = 0.5f * (P.rbox[tid] + P.rbox[DP + tid]);
         __syncthreads();
-        const bool act = epi && qt < nq;
-        const int myq = P.qbeg[qnode] + chunk * kQB + qt;
+        const bool act = epi && half * kQB + qt < nq;
+        const int myq = P.qbeg[qnode] + (chunk + half) * kQB + qt;
         const int kq = P.k;  // read once: stores below could alias P
         const bool mono = P.mono != 0;
         const float lam2 = 2.f * P.qlam[qnode];
@@ -507,10 +516,10 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                 qa2 = __fmaf_ru(h[j], h[j], qa2);
             }
             qn = tc_norm<FMT, DP>(h);
-            if (grp_id == 0) {
+            if (QH == 2 || grp_id == 0) {
 #pragma unroll
                 for (int c = 0; c < S::NCH; ++c)
-                    *reinterpret_cast<uint4*>(sA + tc::core_offset(qt, c, S::GB)) =
+                    *reinterpret_cast<uint4*>(sA + half * kQB * S::RB + tc::core_offset(qt, c, S::GB)) =
                         tc_row_chunk<FMT, DP, true>(c, h, 1.f, 1.f);
             }
             qa = __fsqrt_ru(qa2);
@@ -577,16 +586,21 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                 __syncwarp();
                 if (w0 + WIN < ntot) fetch(w0 + WIN, wbuf ^ 1);
                 // the block's bound from the epilogue warps' published values
-                float b = Bq;
+                // (two groups of one half each keep a list per query: their
+                // queries' bounds join; two groups of the same queries keep two
+                // lists per query, and either's bounds hold for all of them)
+                float b = Bq, mx = -INFINITY, mn = INFINITY;
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
-                    float mx = -INFINITY, mn = INFINITY;
 #pragma unroll
                     for (int w = 0; w < 4; ++w) {
                         mx = fmaxf(mx, s_wmax[4 * g + w]);
                         mn = fminf(mn, s_wmin[4 * g + w]);
                     }
+                    if (QH == 2 && g + 1 < NG) continue;
                     b = fminf(b, fminf(mx, __fadd_ru(mn, lam2)));
+                    mx = -INFINITY;
+                    mn = INFINITY;
                 }
                 // the window's kept leaves (Algorithm 3: a leaf whose d_min
                 // exceeds the bound is pruned), their ranges, and where each
@@ -752,11 +766,12 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
         } else if (warp == MW) {
             // ================= MMA issuer (one thread) =================
             if (lane == 0) {
+                bool seen = false;  // the next slot was seen filled while MMAs were under way
                 for (;;) {
                     const int op = (int)(otile % NB);
                     const uint32_t use = otile / NB;
                     long long t0 = TC_TIMED ? clock64() : 0;
-                    if (!tc::mbar_wait(&op_full[op], use & 1u, x.spin_budget)) {
+                    if (!seen && !tc::mbar_wait(&op_full[op], use & 1u, x.spin_budget)) {
                         TC_FAIL_SITE(FS_MMA_OP);
                         s_fail = 1;
                         break;
@@ -771,14 +786,15 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                         tc::mbar_arrive(&op_empty[op], 1);
                         bool ok = true;
                         for (int e = 0; e < NG && ok; ++e) {
-                            const int b = (int)acur;
+                            uint32_t& turn = QH == 2 && e == 1 ? acur1 : acur;
+                            const int b = (int)turn;
                             ok = tc::mbar_wait(&acc_empty[b], ((aph >> b) & 1u) ^ 1u, x.spin_budget);
                             if (ok) {
                                 amet[b] = make_int2(op, -1);
                                 tc::mbar_arrive(&acc_full[b], 2);
                                 aph ^= 1u << b;
                                 aused |= 1u << b;
-                                acur = (acur + 1) % NACC;
+                                turn = (turn + QH) % NACC;
                             }
                         }
                         if (!ok) {
@@ -787,41 +803,53 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                         }
                         break;
                     }
-                    const int b = (int)acur;
-                    const long long ta = TC_TIMED ? clock64() : 0;
-                    if (!tc::mbar_wait(&acc_empty[b], ((aph >> b) & 1u) ^ 1u, x.spin_budget)) {
+                    bool ok = true;
+#pragma unroll
+                    for (int h = 0; h < QH; ++h) {
+                        if (h == 1 && !both) break;
+                        uint32_t& turn = h == 1 ? acur1 : acur;
+                        const int b = (int)turn;
+                        const long long ta = TC_TIMED ? clock64() : 0;
+                        ok = tc::mbar_wait(&acc_empty[b], ((aph >> b) & 1u) ^ 1u, x.spin_budget);
+                        if (!ok) break;
+                        if (TC_TIMED) {
+                            const long long tb = clock64();
+                            atomicAdd(&x.timers[TT_MMA_WAIT], (unsigned long long)(tb - (h == 0 ? t0 : ta)));
+                            atomicAdd(&x.timers[TT_MMA_WAIT_ACC], (unsigned long long)(tb - ta));
+                        }
+                        tc::fence_after_sync();
+                        const uint32_t a0 = tc::smem_u32(sA + h * kQB * S::RB), b0 = tc::smem_u32(sB + op * TN * S::RB);
+#pragma unroll
+                        for (int m = 0; m < S::NK; ++m) {
+                            // the tensor pipe queues an MMA or two: the next
+                            // slot's barrier is polled behind the queued ones
+                            if (m == S::NK - 1 && (h == QH - 1 || !both))
+                                seen = tc::mbar_test(&op_full[otile % NB], (otile / NB) & 1u);
+                            tc::mma<TcFmt<FMT>::hw>(tmem + (uint32_t)(b * TN),
+                                                    tc::sdesc(a0 + 256u * S::astep(m), 128u, S::GB),
+                                                    tc::sdesc(b0 + 256u * S::bstep(m), 128u, S::GB), idesc,
+                                                    m > 0 ? 1u : 0u);
+                        }
+                        tc::mma_commit(&acc_full[b]);
+                        amet[b] = make_int2((int)(gtile % GR), nst);
+                        tc::mbar_arrive(&acc_full[b], 1);
+                        aph ^= 1u << b;
+                        aused |= 1u << b;
+                        turn = (turn + QH) % NACC;
+                    }
+                    if (!ok) {
                         TC_FAIL_SITE(FS_MMA_ACC);
                         s_fail = 1;
                         break;
                     }
-                    if (TC_TIMED) {
-                        const long long tb = clock64();
-                        atomicAdd(&x.timers[TT_MMA_WAIT], (unsigned long long)(tb - t0));
-                        atomicAdd(&x.timers[TT_MMA_WAIT_ACC], (unsigned long long)(tb - ta));
-                    }
-                    tc::fence_after_sync();
-                    const uint32_t a0 = tc::smem_u32(sA), b0 = tc::smem_u32(sB + op * TN * S::RB);
-#pragma unroll
-                    for (int m = 0; m < S::NK; ++m)
-                        tc::mma<TcFmt<FMT>::hw>(tmem + (uint32_t)(b * TN),
-                                                tc::sdesc(a0 + 256u * S::astep(m), 128u, S::GB),
-                                                tc::sdesc(b0 + 256u * S::bstep(m), 128u, S::GB), idesc,
-                                                m > 0 ? 1u : 0u);
-                    tc::mma_commit(&acc_full[b]);
                     tc::mma_commit(&op_empty[op]);  // the slot is free once the MMAs are done
-                    amet[b] = make_int2((int)(gtile % GR), nst);
                     ++gtile;
-                    tc::mbar_arrive(&acc_full[b], 1);
-                    aph ^= 1u << b;
-                    aused |= 1u << b;
-                    acur = (acur + 1) % NACC;
                 }
             }
             __syncwarp();
         } else {
             // ================= epilogue warp =================
             const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);  // this warp's lanes
-            float* scr = sscr + grp_id * 32 * kQB + qt;
             float* bw = sbuf + grp_id * CB * kQB + qt;
             int32_t* bi = reinterpret_cast<int32_t*>(sbuf + NG * CB * kQB) + grp_id * CB * kQB + qt;
             // insertion threshold in w units: below the list's last key and
@@ -903,12 +931,13 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                     take(__ffs(m) - 1, mm);
                     return;
                 }
-#pragma unroll
-                for (int i = 0; i < 32; ++i) scr[i * kQB] = __uint_as_float(v[i]);
                 while (m) {
                     const int i = __ffs(m) - 1;
                     m &= m - 1;
-                    const float w = scr[i * kQB];
+                    uint32_t wv = v[0];
+#pragma unroll
+                    for (int j = 1; j < 32; ++j) wv = i == j ? v[j] : wv;
+                    const float w = __uint_as_float(wv);
                     if (!(w <= t)) continue;
                     if (nb == CB) {
                         flush();
@@ -957,11 +986,12 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                 // examine path keeps the kernel's code within the instruction
                 // cache).  A 64-column read past the tile's columns stays
                 // within the accumulator (TN is a multiple of 64); its stale
-                // columns only lower the minimum.  With two epilogue groups
-                // (registers capped lower) the columns are read 32 at a time;
+                // columns only lower the minimum.  With two epilogue groups and
+                // lists of 32 (registers capped lower) the columns are read 32
+                // at a time;
                 // every 8th tile of a warp checks the load's minimum against
                 // the computed one (diagnostics).
-                if constexpr (NG == 1) {
+                if constexpr (WIDE) {
 #pragma unroll 1
                     for (int c2 = 0; c2 < nch; c2 += 2) {
                         const long long l0 = TC_TIMED ? clock64() : 0;
@@ -995,7 +1025,8 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                 __syncwarp();
                 if (lane == 0) {
                     tc::mbar_arrive(&acc_empty[b], 1);
-                    tc::mbar_arrive(&gr_empty[am.x], 1);
+                    // (an idle second half's arrivals are the first's to make)
+                    tc::mbar_arrive(&gr_empty[am.x], QH == 2 && !both ? 2u : 1u);
                 }
                 // the whole warp inserts its buffered candidates together, once
                 // enough lanes hold some (one pass of the insertion code then
@@ -1045,7 +1076,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
         // the buffers the re-rank would reuse)
         __syncthreads();
         if (s_fail) break;
-        if (epi && NG == 2) {
+        if (epi && NG == 2 && QH == 1) {
             // merge group 1's lists into group 0's
             float* smd = reinterpret_cast<float*>(smem);
             int32_t* smi = reinterpret_cast<int32_t*>(smem + kQB * KC * 4);
@@ -1068,7 +1099,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
             // the re-rank below reuses the merge buffers: group 0 has read them
             tc::named_sync(1, 256);
         }
-        if (epi && grp_id == 0) {
+        if (epi && (QH == 2 || grp_id == 0)) {
             // ---- finish the work item
             long long tf0 = TC_TIMED ? clock64() : 0;
             const float ubk = fminf(Bd::ub(list_at(ld, kq - 1), qa), qc);
@@ -1079,9 +1110,10 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
             } else if (act) {
                 // exact order of the band's candidates, in shared memory:
                 // entry j is rk / rd[j kQB + qt] with its position ri[...]
-                uint64_t* rk = reinterpret_cast<uint64_t*>(smem);
-                double* rd = reinterpret_cast<double*>(smem);
-                int32_t* ri = reinterpret_cast<int32_t*>(smem + kQB * KC * 8);
+                unsigned char* fin = smem + half * kQB * KC * 12;
+                uint64_t* rk = reinterpret_cast<uint64_t*>(fin);
+                double* rd = reinterpret_cast<double*>(fin);
+                int32_t* ri = reinterpret_cast<int32_t*>(fin + kQB * KC * 8);
                 const float* qp = P.qpts + (int64_t)myq * DP;
                 int nr = 0;
 #pragma unroll
@@ -1194,14 +1226,14 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
 
 // The kernel allocates all of TMEM; at most one CTA may be resident per
 // SM: the request is raised above half the SM's shared memory.
-template <int FMT, int DP, int KC, int NG>
+template <int FMT, int DP, int KC, int NG, int QH>
 inline size_t tc_smem_bytes() {
     int dev = 0, sm_total = 233472;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sm_total, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     cudaGetLastError();
     size_t guard = (size_t)sm_total / 2 + 1024;
-    size_t need = (size_t)TcSmem<FMT, DP, KC, NG>::BYTES;
+    size_t need = (size_t)TcSmem<FMT, DP, KC, NG, QH>::BYTES;
     return need > guard ? need : guard;
 }
 
@@ -1231,25 +1263,31 @@ int launch_tc_ops(const dtree_t* t, int fmt, int ls, void* out, cudaStream_t s) 
     return DTREE_OK;
 }
 
+template <int FMT, int DP, int KC, int NG, int QH>
+int launch_tile_tc_as(const TileArgs& a, const TcExtra& x, int items, cudaStream_t s) {
+    auto kern = k_tile_tc<FMT, DP, KC, NG, QH>;
+    const size_t smem = tc_smem_bytes<FMT, DP, KC, NG, QH>();
+    DT_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int nt = 32 * (4 * NG + 3);
+    int g = occupancy_grid((const void*)kern, nt, smem);
+    if (items < g) g = items > 0 ? items : 1;
+    DT_LAUNCH(kern, g, nt, smem, s, a, x);
+    return DTREE_OK;
+}
+
 template <int DP>
-int launch_tile_tc(const TileArgs& a, int fmt, int kc, int items, int* err, int spin, cudaStream_t s) {
+int launch_tile_tc(const TileArgs& a, int fmt, int kc, int items, bool wide, int* err, int spin, cudaStream_t s) {
     TcExtra x{err, spin, g_tc_timers, g_tc_stall};
     const int F = tc_format(fmt);
     // two epilogue groups where their lists leave room for a second group's
-    // registers (ten warps put three on a sub-partition: 168 registers a
-    // thread) and their scratch fits shared memory; else one group
-#define DT_TC_CASE(FMTV, KCV)                                                              \
-    if (F == FMTV && kc == KCV) {                                                          \
-        constexpr int NGV = (KCV <= 32 && DP <= 32) ? 2 : 1;                               \
-        auto kern = k_tile_tc<FMTV, DP, KCV, NGV>;                                         \
-        size_t smem = tc_smem_bytes<FMTV, DP, KCV, NGV>();                                 \
-        DT_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                                      (int)smem));                                         \
-        const int nt = 32 * (4 * NGV + 3);                                                 \
-        int g = occupancy_grid((const void*)kern, nt, smem);                               \
-        if (items < g) g = items > 0 ? items : 1;                                          \
-        DT_LAUNCH(kern, g, nt, smem, s, a, x);                                             \
-        return DTREE_OK;                                                                   \
+    // registers (eleven warps put three on a sub-partition: 168 registers a
+    // thread); else one group.  Items of two halves where the caller's blocks
+    // hold them (wide), a group per half
+#define DT_TC_CASE(FMTV, KCV)                                                                     \
+    if (F == FMTV && kc == KCV) {                                                                 \
+        if constexpr (KCV <= 32)                                                                  \
+            if (wide) return launch_tile_tc_as<FMTV, DP, KCV, 2, 2>(a, x, items, s);              \
+        return launch_tile_tc_as<FMTV, DP, KCV, (KCV <= 32 && DP <= 32) ? 2 : 1, 1>(a, x, items, s); \
     }
     DT_TC_CASE(2, 16)
     DT_TC_CASE(2, 24)
