@@ -1,6 +1,7 @@
 // kfn.cu -- dtree_kfn: exact k-furthest-neighbour search, host side (the
 // kernels and their reading of Section 5 are in kfn.cuh).
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "kfn.cuh"
@@ -16,6 +17,41 @@ int kfn_launch(int dp, const KfnArgs& a, int kc, bool exact, int grid, cudaStrea
         case 32: return launch_kfn<32>(a, kc, exact, grid, s);
         default: return launch_kfn<64>(a, kc, exact, grid, s);
     }
+}
+
+// Whether the block search serves a problem: enough work that its passes pay
+// (d > 8 and 1e9 pairs), and extents (the reference points' radius R about their box centre, the
+// queries' largest distance from it) that keep the squares and the bounds
+// relative to them inside float32's range.  Reads both roots back.
+//
+// A walk per query visits few leaves where the box bound prunes well (d <= 8:
+// 1M x 100k uniform points in d = 3 3.6 ms against 5.4; 1M x 30k in d = 8 5.9
+// against 9.6) and has no passes to pay for (2k queries of 5k points, d = 16:
+// 1.1 against 1.7 ms).  Above, blocks of queries share the visits and the
+// tensor cores do the distances: 1M x 20k points of the mixture, d = 12, 16,
+// 32: 26.5 -> 11.3, 40.8 -> 11.6, 195 -> 19.6 ms; 50k x 20k, d = 16: 5.5 ->
+// 3.9; 300k x 5k, d = 10 and 20: 5.4 -> 4.9, 14.7 -> 6.5.
+int kfn_tiles_fit(const dtree_t* tq, const dtree_t* tr, cudaStream_t s, bool* fit) {
+    *fit = false;
+    int major = 0, minor = 0;
+    cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, tr->device);
+    cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, tr->device);
+    if (major != 10 || minor != 3) return DTREE_OK;  // the tiles are tcgen05 code
+    if (tr->dp < 16 || (double)tq->n * (double)tr->n < 1e9) return DTREE_OK;
+    float qb[128], rb[128], ql = 0.f, rl = 0.f;
+    const size_t row = (size_t)2 * tr->dp * sizeof(float);
+    DT_CHECK(cudaMemcpyAsync(qb, tq->box, row, cudaMemcpyDeviceToHost, s));
+    DT_CHECK(cudaMemcpyAsync(rb, tr->box, row, cudaMemcpyDeviceToHost, s));
+    DT_CHECK(cudaMemcpyAsync(&ql, tq->lam, sizeof(float), cudaMemcpyDeviceToHost, s));
+    DT_CHECK(cudaMemcpyAsync(&rl, tr->lam, sizeof(float), cudaMemcpyDeviceToHost, s));
+    DT_CHECK(cudaStreamSynchronize(s));
+    double c2 = 0.0;
+    for (int j = 0; j < tr->dp; ++j) {
+        const double t = 0.5 * ((double)qb[j] + qb[tr->dp + j]) - 0.5 * ((double)rb[j] + rb[tr->dp + j]);
+        c2 += t * t;
+    }
+    *fit = rl >= 1e-12f && rl <= 1e15f && std::sqrt(c2) + ql <= 1e15;
+    return DTREE_OK;
 }
 
 }  // namespace
@@ -44,6 +80,18 @@ extern "C" int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, in
     const int kc = k + 1 <= 16 ? 16 : k + 1 <= 32 ? 32 : 64;
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t launches0 = g_launches.load();
+    bool tiles = false;
+    int rt = kfn_tiles_fit(tq, ref, s, &tiles);
+    if (rt != DTREE_OK) return rt;
+    if (tiles) {
+        rt = kfn_by_tiles(tq, ref, mono, k, out_idx, out_dist, s, st);
+        if (rt == DTREE_OK && st) st->point_pairs += st->seed_point_pairs;
+        if (rt == DTREE_OK) return rt;
+        // (its operand rows or candidate pairs may not fit where the search
+        // below, which needs 4 bytes a query, does)
+        if (rt != DTREE_ERR_OOM) return rt;
+        if (st) memset(st, 0, sizeof(*st));
+    }
 
     // scratch: three counters, the fallback count, and the fallback list
     unsigned char* scratch = nullptr;
@@ -67,6 +115,7 @@ extern "C" int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, in
     a.stats = reinterpret_cast<unsigned long long*>(scratch);
     a.fb_count = reinterpret_cast<int*>(scratch + 32);
     a.fb_list = reinterpret_cast<int*>(scratch + 48);
+    a.fb_stride = 1;
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaEvent_t ev[2] = {};

@@ -9,6 +9,10 @@
 // unique: the first k of the list sorted by (distance descending, index
 // ascending).
 //
+// Large problems in d > 8 go through the block search of knn.cu with every
+// distance negated (kfn.cu's kfn_tiles_fit says which); this file's kernels
+// serve the others, and the queries whose band overflowed there.
+//
 // One warp serves one query (a query node of one point, so the traversal is
 // Algorithm 1's depth-first recursion on the reference tree alone):
 //
@@ -42,27 +46,6 @@
 
 namespace dt {
 
-struct KfnArgs {
-    // query points in query-tree order (DP floats each) and their caller rows
-    const float* qpts;
-    const int32_t* qidx;
-    int64_t nq;
-    // reference tree
-    const float* rpts;
-    const int32_t* ridx;
-    const int32_t* rbeg;
-    const int32_t* rcnt;
-    const float* rbox;
-    int hr;
-    int k;
-    int mono;
-    int64_t* out_idx;   // (rows in the caller's query order) x k
-    float* out_dist;
-    int* fb_list;       // float pass: appends queries whose band overflowed; double pass: its input
-    int* fb_count;
-    unsigned long long* stats;  // [0] point distances, [1] leaves visited, [2] nodes pruned
-};
-
 constexpr int kKfnEmpty = 0x7fffffff;  // the index of an empty list entry
 
 template <int DP, int KC, typename T>
@@ -82,7 +65,7 @@ __global__ void __launch_bounds__(128) k_kfn(const KfnArgs a) {
     unsigned long long n_pts = 0, n_leaves = 0, n_pruned = 0;
 
     for (int64_t wi = w0; wi < count; wi += nw) {
-        const int64_t qpos = EXACT ? (int64_t)a.fb_list[wi] : wi;
+        const int64_t qpos = EXACT ? (int64_t)a.fb_list[wi * a.fb_stride] : wi;
         const float* qp = a.qpts + qpos * DP;
         float q[DP];
 #pragma unroll

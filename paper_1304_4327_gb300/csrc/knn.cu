@@ -111,6 +111,17 @@ __device__ __forceinline__ float box_dmin_centre(const float* a, const float* b,
 }
 
 template <int DP>
+__device__ __forceinline__ float point_box_far2(const float* c, const float* bx) {
+    float s = 0.f;
+#pragma unroll
+    for (int j = 0; j < DP; ++j) {
+        const float g = fmaxf(c[j] - bx[j], bx[DP + j] - c[j]);
+        s = fmaf(g, g, s);
+    }
+    return s;
+}
+
+template <int DP, int OP>
 __global__ void k_seed(const ProbDev* probs, const int32_t* blk_prob, int nblocks, int slots,
                        int32_t* seed_leaf0, int32_t* seed_nleaf) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
@@ -125,7 +136,10 @@ __global__ void k_seed(const ProbDev* probs, const int32_t* blk_prob, int nblock
     for (int L = 0; L < P.Ls; ++L) {
         int64_t l = 2 * n + 1, r = l + 1;
         float dl, dr;
-        if (P.bound == DTREE_BOUND_BOX) {
+        if (OP == OP_FAR) {  // towards the farther corner
+            dl = -point_box_far2<DP>(c, rbox + l * 2 * DP);
+            dr = -point_box_far2<DP>(c, rbox + r * 2 * DP);
+        } else if (P.bound == DTREE_BOUND_BOX) {
             dl = point_box_d2<DP>(c, rbox + l * 2 * DP);
             dr = point_box_d2<DP>(c, rbox + r * 2 * DP);
         } else {  // nearer by the search's bound (an order only: any choice is exact)
@@ -171,7 +185,7 @@ __global__ void k_seed_proposal(const ProbDev* probs, const int32_t* blk_prob, i
 
 constexpr int kExpandProbs = 64;
 
-template <int DP>
+template <int DP, int OP>
 __global__ void __launch_bounds__(256, 2) k_expand(const ProbDev* __restrict__ probs,
                                                 const int32_t* __restrict__ node_prob,
                                                 const float* __restrict__ Bn, const int2* fin,
@@ -237,10 +251,11 @@ __global__ void __launch_bounds__(256, 2) k_expand(const ProbDev* __restrict__ p
                 // order among the candidates), from the same box loads
                 const bool leaves = qbot && rbot;
                 float o = -1.f;
-                float dmin = bound == DTREE_BOUND_BALL ? 0.f
-                             : leaves                  ? box_dmin_centre<DP>(qbx, rbx, o)
-                                                       : box_dmin_down<DP>(qbx, rbx);
-                if (bound != DTREE_BOUND_BOX)
+                float dmin = OP == OP_FAR                ? box_dmax_neg<DP>(qbx, rbx)
+                             : bound == DTREE_BOUND_BALL ? 0.f
+                             : leaves                    ? box_dmin_centre<DP>(qbx, rbx, o)
+                                                         : box_dmin_down<DP>(qbx, rbx);
+                if (OP == OP_NEAR && bound != DTREE_BOUND_BOX)
                     dmin = fmaxf(dmin, ball_dmin_down<DP>(qbx, qlam[qc], rbx, rlam[rc]));
                 ++sc;
                 if (dmin > Bn[node0 + qc]) {  // Score() = infinity: prune every descendant pair
@@ -257,6 +272,7 @@ __global__ void __launch_bounds__(256, 2) k_expand(const ProbDev* __restrict__ p
                                 float t = 0.5f * (qbx[j] + qbx[DP + j]) - 0.5f * (rbx[j] + rbx[DP + j]);
                                 o = fmaf(t, t, o);
                             }
+                            if (OP == OP_FAR) o = -o;  // the farthest first
                         }
                         e4 = make_int4(blk, leaf, __float_as_int(dmin), __float_as_int(o));
                         do_emit = true;
@@ -306,23 +322,18 @@ __global__ void __launch_bounds__(256, 2) k_expand(const ProbDev* __restrict__ p
     }
 }
 
-__global__ void k_fill(float* p, int64_t n, float v) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) p[i] = v;
-}
-
 // One warp per block: B_1 / A of the block from its queries' upper bounds on
-// their k-th distances, then pushed to every ancestor with monotone atomics
-// (non-negative floats order like their bit patterns).
+// their k-th distances, then pushed to every ancestor with monotone atomics on
+// order-preserving codes (f2o; negated distances are negative).
 __global__ void k_block_bounds(const ProbDev* probs, const int32_t* blk_prob, int nblocks,
-                               const float* qub, float* B1n, float* An) {
+                               const float* qub, uint32_t* B1n, uint32_t* An) {
     const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (w >= nblocks) return;
     const ProbDev& P = probs[blk_prob[w]];
     const int64_t node = P.qblock0 + (w - P.block0);
     const int b = P.qbeg[node], c = P.qcnt[node];
-    float mx = 0.f, mn = INFINITY;
+    float mx = -INFINITY, mn = INFINITY;
     for (int i = lane; i < c; i += 32) {
         const float ub = qub[P.q0 + b + i];
         mx = fmaxf(mx, ub);
@@ -334,25 +345,25 @@ __global__ void k_block_bounds(const ProbDev* probs, const int32_t* blk_prob, in
         mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
     }
     if (lane == 0) {
-        B1n[P.node0 + node] = mx;
-        An[P.node0 + node] = mn;
+        B1n[P.node0 + node] = f2o(mx);
+        An[P.node0 + node] = f2o(mn);
         for (int64_t p = node; p > 0;) {
             p = (p - 1) / 2;
-            atomicMax(reinterpret_cast<int*>(&B1n[P.node0 + p]), __float_as_int(mx));
-            atomicMin(reinterpret_cast<int*>(&An[P.node0 + p]), __float_as_int(mn));
+            atomicMax(&B1n[P.node0 + p], f2o(mx));
+            atomicMin(&An[P.node0 + p], f2o(mn));
         }
     }
 }
 
 // B(N) = min over N and its ancestors a of min(B_1(a), A(a) + 2 lambda(a)).
-__global__ void k_node_bounds(const ProbDev* probs, const int32_t* node_prob, const float* B1n,
-                              const float* An, int64_t nn, float* Bn) {
+__global__ void k_node_bounds(const ProbDev* probs, const int32_t* node_prob, const uint32_t* B1n,
+                              const uint32_t* An, int64_t nn, float* Bn) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= nn) return;
     const ProbDev& P = probs[node_prob[i]];
     float B = INFINITY;
     for (int64_t a = i - P.node0;; a = (a - 1) / 2) {
-        B = fminf(B, fminf(B1n[P.node0 + a], __fadd_ru(An[P.node0 + a], 2.f * P.qlam[a])));
+        B = fminf(B, fminf(o2f(B1n[P.node0 + a]), __fadd_ru(o2f(An[P.node0 + a]), 2.f * P.qlam[a])));
         if (a == 0) break;
     }
     Bn[i] = B;
@@ -454,20 +465,22 @@ __global__ void __launch_bounds__(256) k_csr_sort(const int64_t* off, int nb, in
 }  // namespace
 
 template <int DP>
-int launch_expand(const ProbDev* probs, const int32_t* node_prob, const float* Bn, const int2* fin,
+int launch_expand(int op, const ProbDev* probs, const int32_t* node_prob, const float* Bn, const int2* fin,
                   const int* nin, int2* fout, int* nout, int64_t cap, int4* outp, int* noutp,
                   int64_t capp, int* bcount, const int32_t* sl0, const int32_t* sn, int slots,
                   int* overflow, unsigned long long* stats, int np, int grid, cudaStream_t s) {
     const size_t smem = (size_t)std::min(np, kExpandProbs) * sizeof(ProbDev);
-    DT_LAUNCH(k_expand<DP>, grid, 256, smem, s, probs, node_prob, Bn, fin, nin, fout, nout, cap,
+    auto kern = op == OP_FAR ? k_expand<DP, OP_FAR> : k_expand<DP, OP_NEAR>;
+    DT_LAUNCH(kern, grid, 256, smem, s, probs, node_prob, Bn, fin, nin, fout, nout, cap,
               outp, noutp, capp, bcount, sl0, sn, slots, overflow, stats, np);
     return DTREE_OK;
 }
 
 template <int DP>
-int launch_seed(const ProbDev* probs, const int32_t* blk_prob, int nblocks, int slots,
+int launch_seed(int op, const ProbDev* probs, const int32_t* blk_prob, int nblocks, int slots,
                 int32_t* seed_leaf0, int32_t* seed_nleaf, cudaStream_t s) {
-    DT_LAUNCH(k_seed<DP>, (nblocks + 127) / 128, 128, 0, s, probs, blk_prob, nblocks, slots,
+    auto kern = op == OP_FAR ? k_seed<DP, OP_FAR> : k_seed<DP, OP_NEAR>;
+    DT_LAUNCH(kern, (nblocks + 127) / 128, 128, 0, s, probs, blk_prob, nblocks, slots,
               seed_leaf0, seed_nleaf);
     return DTREE_OK;
 }
@@ -610,7 +623,7 @@ inline int kc_bucket(int need) {
 // The search for a batch of problems whose points share the padded dimension
 // DP: every phase is one launch (or one per traversal level) over all the
 // problems' blocks, pairs and queries.
-template <int DP>
+template <int DP, int OP = OP_NEAR>
 int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap_leaves, int prec, int spin,
                    int nprop, int bound, cudaStream_t s, dtree_stats* st, const ScratchArena* arena) {
     const int64_t launches0 = g_launches.load();
@@ -624,7 +637,7 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
     // lists hold up to 64 entries (k <= 63; a band wider than the list sends
     // its queries to the fallback)
     if (kmax + 1 > 64) return DTREE_ERR_UNSUPPORTED;
-    const int KC = std::min(kc_bucket(kc_need), 64);
+    const int KC = OP == OP_FAR ? (kc_need <= 24 ? 24 : kc_need <= 32 ? 32 : 64) : std::min(kc_bucket(kc_need), 64);
 
     // the problems' layout in the batch-wide arrays
     ProbDev one[1];
@@ -725,7 +738,8 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
     int32_t *blk_prob, *node_prob, *sl0, *sn, *cand_i, *csr_leaf = nullptr;
     int2 *items, *roots;
     int4 *fbq_list, *fbq2_list;
-    float *cand_d, *B1n, *An, *Bn, *csr_dmin = nullptr, *csr_key = nullptr, *qub;
+    uint32_t *B1n, *An;
+    float *cand_d, *Bn, *csr_dmin = nullptr, *csr_key = nullptr, *qub;
     int *ctr, *bcount, *bcur, *derr;
     int64_t* off;
     unsigned long long* dstats;
@@ -767,7 +781,7 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
     tm.mark();  // 0
 
     // 1. seed: the greedy subtree of each block, plus its proposed cells
-    DT_TRY(launch_seed<DP>(probs, blk_prob, NB, slots, sl0, sn, s));
+    DT_TRY(launch_seed<DP>(OP, probs, blk_prob, NB, slots, sl0, sn, s));
     if (nprop > 0) {
         int32_t* cells;
         float* centres;
@@ -812,16 +826,22 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
     // them.  It keeps lists of bucket(k + 1) entries (the float32 band needs
     // no more); the main pass's other rows start empty.
     a.kc_rows = KC;
-    DT_TRY(launch_tile_cc<DP>(a, kc_bucket(kmax + 1), MODE_SEED, NI, s));
+    if constexpr (OP == OP_FAR)
+        DT_TRY(launch_far_seed<DP>(a, kmax + 1 <= 16 ? 16 : kmax + 1 <= 32 ? 32 : 64, NI, s));
+    else
+        DT_TRY(launch_tile_cc<DP>(a, kc_bucket(kmax + 1), MODE_SEED, NI, s));
     if (qcap) {
-        DT_TRY(launch_query_cap<DP>(a, KC, cap_leaves, qcap, s));
+        if constexpr (OP == OP_FAR)
+            DT_TRY(launch_far_cap<DP>(a, KC, cap_leaves, qcap, s));
+        else
+            DT_TRY(launch_query_cap<DP>(a, KC, cap_leaves, qcap, s));
         a.qcap = qcap;
     }
     tm.mark();  // 1
 
     // 2. bounds of every query node down to the blocks
-    DT_LAUNCH(k_fill, (int)((NN + 255) / 256), 256, 0, s, B1n, NN, 0.f);
-    DT_LAUNCH(k_fill, (int)((NN + 255) / 256), 256, 0, s, An, NN, INFINITY);
+    DT_CHECK(cudaMemsetAsync(B1n, 0, (size_t)NN * sizeof(uint32_t), s));    // below every code
+    DT_CHECK(cudaMemsetAsync(An, 0xff, (size_t)NN * sizeof(uint32_t), s));  // above every code
     DT_LAUNCH(k_block_bounds, (NB * 32 + 255) / 256, 256, 0, s, probs, blk_prob, NB, qub, B1n, An);
     DT_LAUNCH(k_node_bounds, (int)((NN + 255) / 256), 256, 0, s, probs, node_prob, B1n, An, NN, Bn);
 
@@ -836,7 +856,7 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
         cap = room > 1024 ? (int64_t)std::min<size_t>((room - 1024) / per, (size_t)1 << 30) : 0;
         if (cap < np) return DTREE_ERR_TOO_LARGE;
     }
-    const int egrid = occupancy_grid((const void*)k_expand<DP>, 256,
+    const int egrid = occupancy_grid((const void*)k_expand<DP, OP>, 256,
                                      (size_t)std::min(np, kExpandProbs) * sizeof(ProbDev));
     int npairs = 0;
     int4* outp = nullptr;
@@ -897,7 +917,7 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
                 ocap = oc2;
             }
             DT_CHECK(cudaMemsetAsync(nc[nx], 0, sizeof(int), s));
-            DT_TRY(launch_expand<DP>(probs, node_prob, Bn, F[cur], nc[cur], F[nx], nc[nx], fcap[nx],
+            DT_TRY(launch_expand<DP>(OP, probs, node_prob, Bn, F[cur], nc[cur], F[nx], nc[nx], fcap[nx],
                                      outp, ctr + 7, ocap, bcount, sl0, sn, slots, ctr + 4, dstats,
                                      np, egrid, s));
             int hv[4];
@@ -929,7 +949,7 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
         int *ni = ctr + 5, *no = ctr + 6;
         for (int t = 0; t < steps; ++t) {
             DT_CHECK(cudaMemsetAsync(no, 0, sizeof(int), s));
-            DT_TRY(launch_expand<DP>(probs, node_prob, Bn, fi, ni, fo, no, cap, outp, ctr + 7, cap,
+            DT_TRY(launch_expand<DP>(OP, probs, node_prob, Bn, fi, ni, fo, no, cap, outp, ctr + 7, cap,
                                      bcount, sl0, sn, slots, ctr + 4, dstats, np, egrid, s));
             std::swap(fi, fo);
             std::swap(ni, no);
@@ -961,7 +981,11 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        DT_TRY(launch_tile_tc<DP>(a, fmt, KC, NI, 2 * paired >= NQ && pairs >= 2 * sms, derr, spin, s));
+        const bool wide = 2 * paired >= NQ && pairs >= 2 * sms;
+        if constexpr (OP == OP_FAR)
+            DT_TRY(launch_far_tile<DP>(a, KC, NI, wide, derr, spin, s));
+        else
+            DT_TRY(launch_tile_tc<DP>(a, fmt, KC, NI, wide, derr, spin, s));
     } else {
         DT_TRY(launch_tile_cc<DP>(a, KC, MODE_MAIN, NI, s));
     }
@@ -976,7 +1000,34 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
     //    with a float64 re-rank of their band, and exact float64 for those
     //    whose float32 band overflows too
     int nfb2 = 0;
-    if (nfb > 0) {
+    if constexpr (OP == OP_FAR) {
+        if (nfb > 0) {
+            // the float64 search, a warp per query
+            KfnArgs ka{};
+            ka.qpts = hp[0].tq->pts;
+            ka.qidx = hp[0].tq->idx;
+            ka.nq = NQ;
+            ka.rpts = hp[0].tr->pts;
+            ka.ridx = hp[0].tr->idx;
+            ka.rbeg = hp[0].tr->nbeg;
+            ka.rcnt = hp[0].tr->ncnt;
+            ka.rbox = hp[0].tr->box;
+            ka.hr = hp[0].tr->height;
+            ka.k = kmax;
+            ka.mono = hp[0].mono ? 1 : 0;
+            ka.out_idx = hp[0].out_idx;
+            ka.out_dist = hp[0].out_dist;
+            ka.fb_list = reinterpret_cast<int*>(fbq_list);
+            ka.fb_stride = 4;
+            ka.fb_count = ctr + 3;
+            int dev = 0, sms = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            DT_TRY(launch_kfn<DP>(ka, kmax + 1 <= 16 ? 16 : kmax + 1 <= 32 ? 32 : 64, true,
+                                  (int)std::max(1, std::min((nfb + 3) / 4, sms * 16)), s));
+            nfb2 = nfb;
+        }
+    } else if (nfb > 0) {
         // few such queries: each one's candidates are split over up to 64
         // CTAs (about two per SM in all), whose lists are then merged
         int dev = 0, sms = 0;
@@ -1109,6 +1160,24 @@ int device_checks(int prec, bool arena, const HostProb* hp, int np, int* dev_out
 }
 
 }  // namespace
+
+int kfn_by_tiles(const dtree_t* tq, const dtree_t* tr, bool mono, int k, int64_t* out_idx, float* out_dist,
+                 cudaStream_t s, dtree_stats* st) {
+    const HostProb hp{tq, tr, mono, k, out_idx, out_dist, 0, nullptr};
+    // blocks of 256 queries (pairs of chunks), the library's default seed and
+    // cap sizes
+    constexpr int qb = 256, seed = 64, cap = 8, prec = DTREE_PREC_BF16, spin = 1 << 20;
+    int rc;
+    switch (tr->dp) {
+        case 4: rc = knn_batch_impl<4, OP_FAR>(&hp, 1, qb, seed, cap, prec, spin, 0, DTREE_BOUND_BOX, s, st, nullptr); break;
+        case 8: rc = knn_batch_impl<8, OP_FAR>(&hp, 1, qb, seed, cap, prec, spin, 0, DTREE_BOUND_BOX, s, st, nullptr); break;
+        case 16: rc = knn_batch_impl<16, OP_FAR>(&hp, 1, qb, seed, cap, prec, spin, 0, DTREE_BOUND_BOX, s, st, nullptr); break;
+        case 32: rc = knn_batch_impl<32, OP_FAR>(&hp, 1, qb, seed, cap, prec, spin, 0, DTREE_BOUND_BOX, s, st, nullptr); break;
+        default: rc = knn_batch_impl<64, OP_FAR>(&hp, 1, qb, seed, cap, prec, spin, 0, DTREE_BOUND_BOX, s, st, nullptr); break;
+    }
+    if (rc != DTREE_OK) cudaStreamSynchronize(s);
+    return rc;
+}
 
 int knn_entry(const dtree_t* query, const dtree_t* ref, int32_t k, int64_t* out_idx,
               float* out_dist, const dtree_opts* o, void* stream, dtree_stats* st,

@@ -25,6 +25,14 @@ enum TileMode {
     MODE_MAIN = 1   // traversal candidates, lists in, exact re-rank + output out
 };
 
+// Which neighbours a search finds.  The furthest ones are found by the same
+// passes with every distance negated: keys are -d^2, node bounds -d_max (a
+// lower bound on the negated distances), B's terms negated k-th distances, so
+// that "smaller is better" holds throughout and B_1, A + 2 lambda and Score keep
+// their form (Section 5's paragraph on k-furthest neighbours inverts the rules;
+// this inverts the distances).
+enum SearchOp { OP_NEAR = 0, OP_FAR = 1 };
+
 constexpr int kQB = 128;           // queries of one work item (one thread each)
 constexpr int kEmptyIdx = 0x7fffffff;
 
@@ -127,6 +135,51 @@ __device__ __forceinline__ float point_dmin_down(int bound, const float* q, cons
     return bound == DTREE_BOUND_BALL ? b : fmaxf(b, point_box_dmin_down<DP>(q, bx));
 }
 
+// Largest distance between the points of two boxes, rounded up and negated: a
+// lower bound on every negated distance.
+template <int DP>
+__device__ __forceinline__ float box_dmax_neg(const float* a, const float* b) {
+    const float4* al = reinterpret_cast<const float4*>(a);
+    const float4* ah = reinterpret_cast<const float4*>(a + DP);
+    const float4* bl = reinterpret_cast<const float4*>(b);
+    const float4* bh = reinterpret_cast<const float4*>(b + DP);
+    float s = 0.f;
+#pragma unroll 4
+    for (int j = 0; j < DP / 4; ++j) {
+        const float4 x = al[j], y = ah[j], u = bl[j], v = bh[j];
+        const float g0 = fmaxf(y.x - u.x, v.x - x.x), g1 = fmaxf(y.y - u.y, v.y - x.y);
+        const float g2 = fmaxf(y.z - u.z, v.z - x.z), g3 = fmaxf(y.w - u.w, v.w - x.w);
+        s = fmaf(g0, g0, s);
+        s = fmaf(g1, g1, s);
+        s = fmaf(g2, g2, s);
+        s = fmaf(g3, g3, s);
+    }
+    return -__fmul_ru(__fsqrt_ru(s), 1.f + rel_eps<DP>());
+}
+
+// What the one-warp-per-query furthest-neighbour kernels read and write.
+struct KfnArgs {
+    // query points in query-tree order (DP floats each) and their caller rows
+    const float* qpts;
+    const int32_t* qidx;
+    int64_t nq;
+    // reference tree
+    const float* rpts;
+    const int32_t* ridx;
+    const int32_t* rbeg;
+    const int32_t* rcnt;
+    const float* rbox;
+    int hr;
+    int k;
+    int mono;
+    int64_t* out_idx;   // (rows in the caller's query order) x k
+    float* out_dist;
+    int* fb_list;       // float pass: appends queries whose band overflowed; double pass: its input,
+    int fb_stride;      //   every fb_stride-th entry
+    int* fb_count;
+    unsigned long long* stats;  // [0] point distances, [1] leaves visited, [2] nodes pruned
+};
+
 struct TileArgs {
     const ProbDev* probs;       // the batch's problems
     const int32_t* blk_prob;    // per block: its problem
@@ -181,6 +234,23 @@ template <int DP>
 int launch_tile_tc(const TileArgs& a, int fmt, int kc, int items, bool wide, int* err, int spin,
                    cudaStream_t s);
 
+// The furthest-neighbour search's seed tile, cap and tensor-core passes (BF16),
+// with lists of 16, 32 or 64 (seed) and 24, 32 or 64 entries.
+template <int DP>
+int launch_far_seed(const TileArgs& a, int kc, int items, cudaStream_t s);
+template <int DP>
+int launch_far_cap(const TileArgs& a, int kc, int budget, float* qcap, cudaStream_t s);
+template <int DP>
+int launch_far_tile(const TileArgs& a, int kc, int items, bool wide, int* err, int spin, cudaStream_t s);
+// ... and the float64 search of the queries listed in a.fb_list (kfn.cuh).
+template <int DP>
+int launch_kfn(const KfnArgs& a, int kc, bool exact, int grid, cudaStream_t s);
+
+// dtree_kfn by these passes: one problem whose extents keep every squared
+// distance inside float32's range (kfn.cu checks).  Adds to st when given.
+int kfn_by_tiles(const dtree_t* tq, const dtree_t* tr, bool mono, int k, int64_t* out_idx, float* out_dist,
+                 cudaStream_t s, dtree_stats* st);
+
 // Bytes per operand row, and the fill of a reference tree's operand array
 // (nleaves x ls rows, ls a multiple of 8) for the tensor-core pass.
 template <int DP>
@@ -226,14 +296,14 @@ __device__ __forceinline__ bool in_seed(const int32_t* sl0, const int32_t* sn, i
 // The traversal's frontier holds (global query node, reference node) pairs;
 // node_prob gives each global query node's problem.
 template <int DP>
-int launch_expand(const ProbDev* probs, const int32_t* node_prob, const float* Bn, const int2* fin,
+int launch_expand(int op, const ProbDev* probs, const int32_t* node_prob, const float* Bn, const int2* fin,
                   const int* nin, int2* fout, int* nout, int64_t cap, int4* outp, int* nout_p,
                   int64_t cap_p, int* bcount, const int32_t* seed_leaf0,
                   const int32_t* seed_nleaf, int seed_slots, int* overflow,
                   unsigned long long* stats, int np, int grid, cudaStream_t s);
 
 template <int DP>
-int launch_seed(const ProbDev* probs, const int32_t* blk_prob, int nblocks, int seed_slots,
+int launch_seed(int op, const ProbDev* probs, const int32_t* blk_prob, int nblocks, int seed_slots,
                 int32_t* seed_leaf0, int32_t* seed_nleaf, cudaStream_t s);
 
 int occupancy_grid(const void* kernel, int threads, size_t smem);

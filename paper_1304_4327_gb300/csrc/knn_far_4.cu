@@ -1,0 +1,8 @@
+// knn_far_4.cu -- furthest-neighbour passes of the block search for dimension bucket DP = 4.
+#include "knn_tc.cuh"
+
+namespace dt {
+template int launch_far_seed<4>(const TileArgs&, int, int, cudaStream_t);
+template int launch_far_cap<4>(const TileArgs&, int, int, float*, cudaStream_t);
+template int launch_far_tile<4>(const TileArgs&, int, int, bool, int*, int, cudaStream_t);
+}  // namespace dt

@@ -67,15 +67,17 @@ struct TcFmt<3> {  // split BF16
     static constexpr float cross = 4.6e-05f;
 };
 
-// Operand rows.  A row (query) carries -2 x the centred coordinates and two
-// ones; a B row (reference) carries the centred coordinates and the float32
-// norm of its represented values split as hi + lo, so the accumulator holds
-// w = |r~|^2 - 2 q~.r~ directly.  Rows are NKS K steps of 32 bytes; MMA m
+// Operand rows.  A row (query) carries -2 x the centred coordinates and three
+// ones; a B row (reference) carries the centred coordinates, the float32 norm
+// of its represented values split as hi + lo, and a zero (+inf in a padding
+// row), so the accumulator holds w = |r~|^2 - 2 q~.r~ directly, +inf for
+// padding.  For the furthest neighbours the A row's signs are the opposite but
+// for the last one: w = -|r~|^2 + 2 q~.r~ from the same B rows.  Rows are NKS K steps of 32 bytes; MMA m
 // reads A step astep(m) and B step bstep(m).
-//   TF32:                     A: -2x, 1, 1      B: x, nhi, nlo          (one pass)
-//   split BF16, DP <= 8:      A: -2hi, -2lo, -2hi, 1, 1
-//                             B:  hi,   hi,   lo, nhi, nlo              (one pass)
-//   split BF16, DP >= 16:     A: [-2hi] [-2lo] [1, 1]  B: [hi] [lo] [nhi, nlo]
+//   TF32:                     A: -2x, 1, 1, 1   B: x, nhi, nlo, 0       (one pass)
+//   split BF16, DP <= 8:      A: -2hi, -2lo, -2hi, 1, 1, 1
+//                             B:  hi,   hi,   lo, nhi, nlo, 0           (one pass)
+//   split BF16, DP >= 16:     A: [-2hi] [-2lo] [1, 1, 1]  B: [hi] [lo] [nhi, nlo, 0]
 //     (each bracket padded to whole K steps; the MMAs pair A hi/B hi,
 //      A lo/B hi, A hi/B lo and the norm steps, so a row stores each copy
 //      of the coordinates once)
@@ -84,7 +86,7 @@ struct TcShape {
     static constexpr int kstep = TcFmt<FMT>::kstep;  // elements per 32-byte K step
     static constexpr bool REUSE = FMT == 3 && DP >= 16;
     static constexpr int H = (DP + kstep - 1) / kstep;  // K steps of one copy of the coordinates
-    static constexpr int NKS = REUSE ? 2 * H + 1 : (DP * TcFmt<FMT>::split + 2 + kstep - 1) / kstep;
+    static constexpr int NKS = REUSE ? 2 * H + 1 : (DP * TcFmt<FMT>::split + 3 + kstep - 1) / kstep;
     static constexpr int NK = REUSE ? 3 * H + 1 : NKS;  // MMAs per tile
     static constexpr int RB = NKS * 32;                 // bytes per operand row
     static constexpr int NCH = RB / 16;                 // 16-byte chunks per row
@@ -143,7 +145,22 @@ __device__ __forceinline__ float sqrt_up(float x) {
     return __fmaf_ru(r, 1.f + 4.7683716e-07f, 1.2e-19f);
 }
 
-template <int FMT, int DP>
+// A lower bound on sqrt(x), as sqrt_up.
+__device__ __forceinline__ float sqrt_down(float x) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return fmaxf(__fmul_rd(r, 1.f - 4.7683716e-07f), 0.f);
+}
+
+// ub(S, a, R) and band(ub, a, R): see the head of the file; R bounds |r - c|
+// over the reference points (only OP_FAR needs it: the root's lambda).  For
+// OP_FAR keys are -s and values -distance; with b <= R,
+//     D >= sqrt(s - alpha (a^2 + R^2)) - e1 (a + R)
+// for each of the k points with a key up to S, so the k-th furthest distance is
+// at least L = that with s = -S, and every true k-furthest point has
+//     s >= (L - e1 (a + R))^2 - alpha (a^2 + R^2).
+// Nothing cancels: the furthest distances are of the size of a + R.
+template <int FMT, int DP, int OP>
 struct TcBound {
     static constexpr float u = 5.9604645e-08f;
     static constexpr float e1 = TcFmt<FMT>::u + 2.f * u;
@@ -152,8 +169,13 @@ struct TcBound {
     static constexpr float alpha =
         ((4.f * TcShape<FMT, DP>::KP + 16.f) * u + TcFmt<FMT>::cross) * 1.01f;
     // upper bound on the true k-th distance of a query with k-th key S
-    __device__ static float ub(float S, float a) {
+    __device__ static float ub(float S, float a, float R) {
         if (!(S < INFINITY)) return INFINITY;
+        if (OP == OP_FAR) {
+            const float n2 = __fmaf_ru(a, a, __fmul_ru(R, R));
+            const float x = fmaxf(__fsub_rd(-S, __fmul_ru(alpha, n2)), 0.f);
+            return -fmaxf(__fsub_rd(sqrt_down(x), __fmul_ru(e1, __fadd_ru(a, R))), 0.f);
+        }
         float sq = sqrt_up(fmaxf(S, 0.f));
         float bb = __fmul_ru(1.03f, __fadd_ru(a, sq));
         float n2 = __fmaf_ru(a, a, __fmul_ru(bb, bb));
@@ -161,8 +183,13 @@ struct TcBound {
         return __fmaf_ru(e1, __fadd_ru(a, bb), r);
     }
     // band: every true k-nearest neighbour has a key <= band(ub, a)
-    __device__ static float band(float ubk, float a) {
+    __device__ static float band(float ubk, float a, float R) {
         if (!(ubk < INFINITY)) return INFINITY;
+        if (OP == OP_FAR) {
+            const float n2 = __fmaf_ru(a, a, __fmul_ru(R, R));
+            const float x = fmaxf(__fsub_rd(fmaxf(-ubk, 0.f), __fmul_ru(e1, __fadd_ru(a, R))), 0.f);
+            return -__fsub_rd(__fmul_rd(x, x), __fmul_ru(alpha, n2));
+        }
         float bu = __fmul_ru(1.01f, __fadd_ru(a, ubk));
         float x = __fmaf_ru(e1, __fadd_ru(a, bu), ubk);
         float n2 = __fmaf_ru(a, a, __fmul_ru(bu, bu));
@@ -197,11 +224,12 @@ __device__ __forceinline__ float tc_norm(const float (&h)[DP]) {
 }
 
 // Element e of an operand row built from the centred coordinates h (A rows:
-// the query side, scaled by -2, with ones in the norm columns).
-template <int FMT, int DP, bool AROW>
-__device__ __forceinline__ float tc_elem(int e, const float (&h)[DP], float nhi, float nlo) {
+// the query side, scaled by -2, with ones in the norm columns, or the opposite
+// for OP_FAR).  pad: the last column.
+template <int FMT, int DP, bool AROW, int OP>
+__device__ __forceinline__ float tc_elem(int e, const float (&h)[DP], float nhi, float nlo, float pad) {
     using S = TcShape<FMT, DP>;
-    const float sc = AROW ? -2.f : 1.f;
+    const float sc = !AROW ? 1.f : OP == OP_FAR ? 2.f : -2.f;
     if constexpr (S::REUSE) {
         constexpr int W = S::H * S::kstep;
         if (e < W) return e < DP ? sc * tc_round<FMT>(h[e < DP ? e : 0]) : 0.f;
@@ -219,34 +247,35 @@ __device__ __forceinline__ float tc_elem(int e, const float (&h)[DP], float nhi,
         if (e < DP) return sc * tc_round<FMT>(h[e]);
         e -= DP;
     }
-    if (e == 0) return AROW ? 1.f : nhi;
-    if (e == 1) return AROW ? 1.f : nlo;
+    if (e == 0) return AROW ? -0.5f * sc : nhi;
+    if (e == 1) return AROW ? -0.5f * sc : nlo;
+    if (e == 2) return AROW ? 1.f : pad;
     return 0.f;
 }
 
 // The 16 bytes of chunk c of an operand row.
-template <int FMT, int DP, bool AROW>
-__device__ __forceinline__ uint4 tc_row_chunk(int c, const float (&h)[DP], float nhi, float nlo) {
+template <int FMT, int DP, bool AROW, int OP = OP_NEAR>
+__device__ __forceinline__ uint4 tc_row_chunk(int c, const float (&h)[DP], float nhi, float nlo, float pad) {
     uint4 w;
     uint32_t* p = reinterpret_cast<uint32_t*>(&w);
     if (TcFmt<FMT>::esize == 2) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            __nv_bfloat162 b = __floats2bfloat162_rn(tc_elem<FMT, DP, AROW>(8 * c + 2 * i, h, nhi, nlo),
-                                                     tc_elem<FMT, DP, AROW>(8 * c + 2 * i + 1, h, nhi, nlo));
+            __nv_bfloat162 b = __floats2bfloat162_rn(tc_elem<FMT, DP, AROW, OP>(8 * c + 2 * i, h, nhi, nlo, pad),
+                                                     tc_elem<FMT, DP, AROW, OP>(8 * c + 2 * i + 1, h, nhi, nlo, pad));
             p[i] = *reinterpret_cast<uint32_t*>(&b);
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) p[i] = __float_as_uint(tc_elem<FMT, DP, AROW>(4 * c + i, h, nhi, nlo));
+        for (int i = 0; i < 4; ++i) p[i] = __float_as_uint(tc_elem<FMT, DP, AROW, OP>(4 * c + i, h, nhi, nlo, pad));
     }
     return w;
 }
 
 // The reference operand array of a tree: leaf l occupies rows [l ls, (l + 1) ls)
 // (ls a multiple of 8); row i < count(l) is the leaf's i-th point centred on
-// the root box centre, the rest are padding rows (zero coordinates, norm
-// +inf, so that their key is +inf).  Row r sits at byte (r / 8) GB +
+// the root box centre, the rest are padding rows (zero coordinates and norm,
+// +inf in the last column, so that their key is +inf).  Row r sits at byte (r / 8) GB +
 // (r % 8) 16 + chunk 128, the shared-memory layout of a tile.
 template <int FMT, int DP>
 __global__ void __launch_bounds__(128) k_tc_ops(const float* __restrict__ pts,
@@ -263,7 +292,7 @@ __global__ void __launch_bounds__(128) k_tc_ops(const float* __restrict__ pts,
         const int i = (int)(r - l * ls);
         const int cnt = ncnt[leaf0 + l];
         float h[DP];
-        float nhi = INFINITY, nlo = 0.f;
+        float nhi = 0.f, nlo = 0.f, pad = INFINITY;
         if (i < cnt) {
             const float4* p4 = reinterpret_cast<const float4*>(pts + ((int64_t)nbeg[leaf0 + l] + i) * DP);
 #pragma unroll
@@ -277,6 +306,7 @@ __global__ void __launch_bounds__(128) k_tc_ops(const float* __restrict__ pts,
             const float rn = tc_norm<FMT, DP>(h);
             nhi = tc_round<FMT>(rn);
             nlo = tc_round<FMT>(rn - nhi);
+            pad = 0.f;
         } else {
 #pragma unroll
             for (int j = 0; j < DP; ++j) h[j] = 0.f;
@@ -284,7 +314,7 @@ __global__ void __launch_bounds__(128) k_tc_ops(const float* __restrict__ pts,
         unsigned char* base = out + (r >> 3) * S::GB + (r & 7) * 16;
 #pragma unroll
         for (int c = 0; c < S::NCH; ++c)
-            *reinterpret_cast<uint4*>(base + c * 128) = tc_row_chunk<FMT, DP, false>(c, h, nhi, nlo);
+            *reinterpret_cast<uint4*>(base + c * 128) = tc_row_chunk<FMT, DP, false>(c, h, nhi, nlo, pad);
     }
 }
 
@@ -391,11 +421,11 @@ static_assert(TT_N <= 32, "the diagnostic timer buffer holds 32 counters");
 // row-group table is read).  Every wait is bounded; after a
 // failed wait the item's work is abandoned, the kernel drains its own copies
 // and MMAs, releases TMEM and reports through x.err.
-template <int FMT, int DP, int KC, int NG, int QH>
+template <int FMT, int DP, int KC, int NG, int QH, int OP>
 __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs a, const TcExtra x) {
     using S = TcShape<FMT, DP>;
     using L = TcSmem<FMT, DP, KC, NG, QH>;
-    using Bd = TcBound<FMT, DP>;
+    using Bd = TcBound<FMT, DP, OP>;
     constexpr int TN = L::TN, TN8 = L::TN8, NACC = L::NACC, NB = L::NB, GR = L::GR, CB = L::CB, WIN = L::WIN;
     constexpr bool WIDE = NG == 1 || KC <= 24;  // 64-column reads
     constexpr int PW = 4 * NG, MW = 4 * NG + 2;  // the first planner's and the MMA issuer's warps
@@ -492,6 +522,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
         const int kq = P.k;  // read once: stores below could alias P
         const bool mono = P.mono != 0;
         const float lam2 = 2.f * P.qlam[qnode];
+        const float rad = OP == OP_FAR ? P.rlam[0] : 0.f;
         float qa = 0.f, qn = 0.f;
         // the cap pass's bound on the query's k-th distance
         const float qc = act && a.qcap ? a.qcap[P.q0 + myq] : INFINITY;
@@ -515,12 +546,12 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                 h[j] = act ? h[j] - scen[j] : 0.f;
                 qa2 = __fmaf_ru(h[j], h[j], qa2);
             }
-            qn = tc_norm<FMT, DP>(h);
+            qn = (OP == OP_FAR ? -1.f : 1.f) * tc_norm<FMT, DP>(h);
             if (QH == 2 || grp_id == 0) {
 #pragma unroll
                 for (int c = 0; c < S::NCH; ++c)
                     *reinterpret_cast<uint4*>(sA + half * kQB * S::RB + tc::core_offset(qt, c, S::GB)) =
-                        tc_row_chunk<FMT, DP, true>(c, h, 1.f, 1.f);
+                        tc_row_chunk<FMT, DP, true, OP>(c, h, 0.f, 0.f, 0.f);
             }
             qa = __fsqrt_ru(qa2);
 #pragma unroll
@@ -528,7 +559,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                 ld[j] = act ? a.cand_d[(int64_t)j * a.nq_all + (P.q0 + myq)] : INFINITY;
                 li[j] = act ? a.cand_i[(int64_t)j * a.nq_all + (P.q0 + myq)] : kEmptyIdx;
             }
-            float ub = fminf(Bd::ub(list_at(ld, kq - 1), qa), qc);
+            float ub = fminf(Bd::ub(list_at(ld, kq - 1), qa, rad), qc);
             float vmax = act ? ub : -INFINITY, vmin = act ? ub : INFINITY;
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) {
@@ -860,7 +891,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
             // insertion lands before it
             float kd = list_at(ld, kq - 1);
             auto threshold = [&]() {
-                const float bnd = Bd::band(fminf(Bd::ub(kd, qa), qc), qa);
+                const float bnd = Bd::band(fminf(Bd::ub(kd, qa, rad), qc), qa, rad);
                 return __fsub_ru(fminf(ld[KC - 1], bnd), qn);
             };
             float t = threshold();
@@ -1046,7 +1077,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                 // later publication only prunes later; any is valid)
                 dirty |= __any_sync(0xffffffffu, changed);
                 if (dirty && ++since_pub >= 4) {
-                    float ub = fminf(Bd::ub(kd, qa), qc);
+                    float ub = fminf(Bd::ub(kd, qa, rad), qc);
                     float vmax = act ? ub : -INFINITY, vmin = act ? ub : INFINITY;
 #pragma unroll
                     for (int off = 16; off > 0; off >>= 1) {
@@ -1102,8 +1133,8 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
         if (epi && (QH == 2 || grp_id == 0)) {
             // ---- finish the work item
             long long tf0 = TC_TIMED ? clock64() : 0;
-            const float ubk = fminf(Bd::ub(list_at(ld, kq - 1), qa), qc);
-            const float band = Bd::band(ubk, qa);
+            const float ubk = fminf(Bd::ub(list_at(ld, kq - 1), qa, rad), qc);
+            const float band = Bd::band(ubk, qa, rad);
             const bool ovf = act && li[KC - 1] != kEmptyIdx && !(ld[KC - 1] > band);
             if (ovf) {
                 a.fbq_list[atomicAdd(a.fbq_count, 1)] = make_int4(myq, blk, __float_as_int(ubk), 0);
@@ -1140,7 +1171,8 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                         const int pos = ri[c * kQB + qt];
                         float h, l;
                         sure &= pair_d2<DP>(q, P.rpts + (int64_t)pos * DP, h, l);
-                        const uint64_t v = ((uint64_t)f2o(h) << 32) | f2o(l);
+                        // (the furthest first: ascending order of the complement)
+                        const uint64_t up = ((uint64_t)f2o(h) << 32) | f2o(l), v = OP == OP_FAR ? ~up : up;
                         int j = c;
                         for (; j > 0 && rk[(j - 1) * kQB + qt] > v; --j) {
                             rk[j * kQB + qt] = rk[(j - 1) * kQB + qt];
@@ -1153,17 +1185,18 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                 if (sure) {
                     float ph = 0.f, pl = 0.f;
                     for (int j = 0; j < nr && j <= kq; ++j) {
-                        const uint64_t v = rk[j * kQB + qt];
+                        const uint64_t v = OP == OP_FAR ? ~rk[j * kQB + qt] : rk[j * kQB + qt];
                         const float h = o2f((uint32_t)(v >> 32)), l = o2f((uint32_t)v);
+                        const float gap = OP == OP_FAR ? (ph - h) + (pl - l) : (h - ph) + (l - pl);
                         // equal zeros are ties too
-                        if (j > 0 && !((h - ph) + (l - pl) > h * ((DP + 4) * 2.2737368e-13f))) sure = false;  // 2^-42
+                        if (j > 0 && !(gap > fmaxf(h, ph) * ((DP + 4) * 2.2737368e-13f))) sure = false;  // 2^-42
                         ph = h;
                         pl = l;
                     }
                 }
                 if (sure) {
                     for (int j = 0; j < kq; ++j) {
-                        const uint64_t v = rk[j * kQB + qt];
+                        const uint64_t v = OP == OP_FAR ? ~rk[j * kQB + qt] : rk[j * kQB + qt];
                         const int pos = ri[j * kQB + qt];
                         float dist;
                         if (!pair_dist<DP>(o2f((uint32_t)(v >> 32)), o2f((uint32_t)v), dist))
@@ -1176,7 +1209,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
 #pragma unroll 1
                     for (int c = 0; c < nr; ++c) {
                         const int pos = ri[c * kQB + qt];
-                        rd[c * kQB + qt] = exact_d2<DP>(qp, P.rpts + (int64_t)pos * DP);
+                        rd[c * kQB + qt] = (OP == OP_FAR ? -1.0 : 1.0) * exact_d2<DP>(qp, P.rpts + (int64_t)pos * DP);
                         ri[c * kQB + qt] = P.ridx[pos];
                     }
                     for (int j = 0; j < kq; ++j) {
@@ -1189,7 +1222,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                         rd[best * kQB + qt] = rd[j * kQB + qt];
                         ri[best * kQB + qt] = ri[j * kQB + qt];
                         P.out_idx[base + j] = bix;
-                        P.out_dist[base + j] = (float)sqrt(bd);
+                        P.out_dist[base + j] = (float)sqrt(OP == OP_FAR ? -bd : bd);
                     }
                 }
             }
@@ -1263,9 +1296,9 @@ int launch_tc_ops(const dtree_t* t, int fmt, int ls, void* out, cudaStream_t s) 
     return DTREE_OK;
 }
 
-template <int FMT, int DP, int KC, int NG, int QH>
+template <int FMT, int DP, int KC, int NG, int QH, int OP>
 int launch_tile_tc_as(const TileArgs& a, const TcExtra& x, int items, cudaStream_t s) {
-    auto kern = k_tile_tc<FMT, DP, KC, NG, QH>;
+    auto kern = k_tile_tc<FMT, DP, KC, NG, QH, OP>;
     const size_t smem = tc_smem_bytes<FMT, DP, KC, NG, QH>();
     DT_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int nt = 32 * (4 * NG + 3);
@@ -1286,8 +1319,8 @@ int launch_tile_tc(const TileArgs& a, int fmt, int kc, int items, bool wide, int
 #define DT_TC_CASE(FMTV, KCV)                                                                     \
     if (F == FMTV && kc == KCV) {                                                                 \
         if constexpr (KCV <= 32)                                                                  \
-            if (wide) return launch_tile_tc_as<FMTV, DP, KCV, 2, 2>(a, x, items, s);              \
-        return launch_tile_tc_as<FMTV, DP, KCV, (KCV <= 32 && DP <= 32) ? 2 : 1, 1>(a, x, items, s); \
+            if (wide) return launch_tile_tc_as<FMTV, DP, KCV, 2, 2, OP_NEAR>(a, x, items, s);     \
+        return launch_tile_tc_as<FMTV, DP, KCV, (KCV <= 32 && DP <= 32) ? 2 : 1, 1, OP_NEAR>(a, x, items, s); \
     }
     DT_TC_CASE(2, 16)
     DT_TC_CASE(2, 24)
@@ -1300,6 +1333,45 @@ int launch_tile_tc(const TileArgs& a, int fmt, int kc, int items, bool wide, int
     DT_TC_CASE(3, 48)
     DT_TC_CASE(3, 64)
 #undef DT_TC_CASE
+    return DTREE_ERR_UNSUPPORTED;
+}
+
+// ---- the furthest-neighbour search's passes (instantiated in knn_far_*.cu)
+template <int DP>
+int launch_far_seed(const TileArgs& a, int kc, int items, cudaStream_t s) {
+#define DT_FAR_SEED(KCV)                                                  \
+    if (kc == KCV) {                                                      \
+        auto kern = k_tile<DP, KCV, MODE_SEED, OP_FAR>;                   \
+        DT_LAUNCH(kern, tile_grid(kern, items), kQB, 0, s, a);            \
+        return DTREE_OK;                                                  \
+    }
+    DT_FAR_SEED(16)
+    DT_FAR_SEED(32)
+    DT_FAR_SEED(64)
+#undef DT_FAR_SEED
+    return DTREE_ERR_UNSUPPORTED;
+}
+
+template <int DP>
+int launch_far_cap(const TileArgs& a, int kc, int budget, float* qcap, cudaStream_t s) {
+    if (kc != a.kc_rows) return DTREE_ERR_UNSUPPORTED;
+    if (kc == 24) return launch_query_cap_as<DP, 24, OP_FAR>(a, budget, qcap, s);
+    if (kc == 32) return launch_query_cap_as<DP, 32, OP_FAR>(a, budget, qcap, s);
+    if (kc == 64) return launch_query_cap_as<DP, 64, OP_FAR>(a, budget, qcap, s);
+    return DTREE_ERR_UNSUPPORTED;
+}
+
+template <int DP>
+int launch_far_tile(const TileArgs& a, int kc, int items, bool wide, int* err, int spin, cudaStream_t s) {
+    TcExtra x{err, spin, g_tc_timers, g_tc_stall};
+    constexpr int NG = DP <= 32 ? 2 : 1;
+    if (kc == 24)
+        return wide ? launch_tile_tc_as<3, DP, 24, 2, 2, OP_FAR>(a, x, items, s)
+                    : launch_tile_tc_as<3, DP, 24, NG, 1, OP_FAR>(a, x, items, s);
+    if (kc == 32)
+        return wide ? launch_tile_tc_as<3, DP, 32, 2, 2, OP_FAR>(a, x, items, s)
+                    : launch_tile_tc_as<3, DP, 32, NG, 1, OP_FAR>(a, x, items, s);
+    if (kc == 64) return launch_tile_tc_as<3, DP, 64, 1, 1, OP_FAR>(a, x, items, s);
     return DTREE_ERR_UNSUPPORTED;
 }
 

@@ -194,6 +194,12 @@ __device__ __forceinline__ bool pair_dist(float h, float l, float& out) {
            half - fabsf(e) > f * ((DP + 4) * 1.1368684e-13f);  // 2^-43
 }
 
+// Upper bound on the true k-th value (a distance; for OP_FAR a negated one, of
+// the negated key): for the furthest neighbours a lower bound on the k-th
+// distance, negated.
+template <int DP, int OP>
+__device__ __forceinline__ float ub_op(float kth);
+
 template <typename T, int DP>
 __device__ __forceinline__ float ub_of(T kth) {
     if (sizeof(T) == 8) return __double2float_ru(__dsqrt_ru((double)kth));
@@ -201,12 +207,19 @@ __device__ __forceinline__ float ub_of(T kth) {
     return __fsqrt_ru(__fmul_ru((float)kth, 1.f + 2.f * rel_eps<DP>()));
 }
 
+template <int DP, int OP>
+__device__ __forceinline__ float ub_op(float kth) {
+    if (OP == OP_NEAR) return ub_of<float, DP>(kth);
+    if (!(kth < INFINITY)) return INFINITY;
+    return -__fsqrt_rd(fmaxf(__fmul_rd(-kth, 1.f - 2.f * rel_eps<DP>()), 0.f));
+}
+
 // Warp 0 of a tile CTA: take candidate leaves from the current window, in
 // order, skip those whose d_min exceeds the block's bound (Algorithm 3:
 // Score = infinity), and pack the rows of the rest (whole leaves, or the
 // part of a leaf that fits) into a stage of at most TN points.  stab gets one
 // (first row, rows, stage offset) entry per run of rows.
-template <int TN, int MODE>
+template <int TN, int MODE, int OP>
 __device__ __forceinline__ void stage_fill(const TileArgs& a, const ProbDev& P, int64_t w0,
                                            int wn, int nseed, int blk, int64_t c0, int3* stab,
                                            unsigned long long& n_skip, unsigned long long& n_eval,
@@ -218,7 +231,7 @@ __device__ __forceinline__ void stage_fill(const TileArgs& a, const ProbDev& P, 
         int c = cur + lane;
         bool valid = c < wn;
         int leaf = 0;
-        float dmin = 0.f;
+        float dmin = -INFINITY;  // (a seed leaf is never pruned)
         if (valid) {
             if (MODE == MODE_MAIN) {  // the block's candidates, sorted nearest-first
                 const int64_t ci = c0 + w0 + c;
@@ -288,7 +301,7 @@ __device__ __forceinline__ void stage_fill(const TileArgs& a, const ProbDev& P, 
     }
 }
 
-template <int DP, int KC, int MODE>
+template <int DP, int KC, int MODE, int OP = OP_NEAR>
 __global__ void __launch_bounds__(kQB) k_tile(const TileArgs a) {
     constexpr int TN = 4096 / DP;       // staged reference points (16 KB)
     constexpr int WINDOW = 2048;        // candidates per window of the main pass
@@ -300,6 +313,8 @@ __global__ void __launch_bounds__(kQB) k_tile(const TileArgs a) {
     __shared__ float s_rmax[kQB / 32], s_rmin[kQB / 32];
     __shared__ ProbDev s_prob;
 
+    constexpr float sgn = OP == OP_FAR ? -1.f : 1.f;  // keys are negated squared distances for OP_FAR
+    static_assert(OP == OP_NEAR || MODE == MODE_SEED, "the furthest neighbours' main pass is the tensor-core one");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nitems = a.nitems;
     unsigned long long n_skip = 0, n_eval = 0, n_pp = 0, n_re = 0;
@@ -351,7 +366,7 @@ __global__ void __launch_bounds__(kQB) k_tile(const TileArgs a) {
 
             // the block's live bound: min(B from the traversal, B_1, B_2)
             auto refresh_bound = [&]() {
-                float ub = fminf(ub_of<float, DP>(list_at(ld, kq - 1)), qc);
+                float ub = fminf(ub_op<DP, OP>(list_at(ld, kq - 1)), qc);
                 float vmax = act ? ub : -INFINITY, vmin = act ? ub : INFINITY;
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) {
@@ -391,7 +406,7 @@ __global__ void __launch_bounds__(kQB) k_tile(const TileArgs a) {
                 while (s_cur < wn) {
                     // ---- warp 0 fills the stage with whole or partial leaves
                     if (warp == 0)
-                        stage_fill<TN, MODE>(a, P, w0, wn, nseed, blk, c0, stab, n_skip,
+                        stage_fill<TN, MODE, OP>(a, P, w0, wn, nseed, blk, c0, stab, n_skip,
                                              n_eval, s_cur, s_part, s_nst, s_ntab, s_B);
                     __syncthreads();
                     // ---- all warps copy the staged rows
@@ -417,15 +432,15 @@ __global__ void __launch_bounds__(kQB) k_tile(const TileArgs a) {
                             if (nst - e0 >= 32) {
 #pragma unroll (DP <= 8 ? 8 : DP <= 16 ? 4 : 2)
                                 for (int i = 0; i < 32; ++i)
-                                    m |= (packed_d2<DP>(q, rows + i * DP) <= tail ? 1u : 0u) << i;
+                                    m |= (sgn * packed_d2<DP>(q, rows + i * DP) <= tail ? 1u : 0u) << i;
                             } else {
                                 for (int i = 0; i < nst - e0; ++i)
-                                    m |= (packed_d2<DP>(q, rows + i * DP) <= tail ? 1u : 0u) << i;
+                                    m |= (sgn * packed_d2<DP>(q, rows + i * DP) <= tail ? 1u : 0u) << i;
                             }
                             while (m) {
                                 const int i = __ffs(m) - 1;
                                 m &= m - 1;
-                                const float key = packed_d2<DP>(q, rows + i * DP);
+                                const float key = sgn * packed_d2<DP>(q, rows + i * DP);
                                 const int rp = spos[e0 + i];
                                 // (the cap pass may have listed this point already)
                                 if (key_less(key, rp, ld[KC - 1], li[KC - 1]) && !(mono && rp == myq) &&
@@ -453,7 +468,7 @@ __global__ void __launch_bounds__(kQB) k_tile(const TileArgs a) {
                         a.cand_d[(int64_t)j * a.nq_all + row] = INFINITY;
                         a.cand_i[(int64_t)j * a.nq_all + row] = kEmptyIdx;
                     }
-                    a.qub[row] = ub_of<float, DP>(list_at(ld, kq - 1));
+                    a.qub[row] = ub_op<DP, OP>(list_at(ld, kq - 1));
                 }
             } else {
                 const float kth = list_at(ld, kq - 1);
@@ -461,7 +476,7 @@ __global__ void __launch_bounds__(kQB) k_tile(const TileArgs a) {
                 const bool ovf = act && li[KC - 1] != kEmptyIdx && !(ld[KC - 1] > band);
                 if (ovf) {
                     a.fbq_list[atomicAdd(a.fbq_count, 1)] =
-                        make_int4(myq, blk, __float_as_int(ub_of<float, DP>(list_at(ld, kq - 1))), 0);
+                        make_int4(myq, blk, __float_as_int(ub_op<DP, OP>(list_at(ld, kq - 1))), 0);
                 } else if (act) {
                     // float64 distances of the band; the float32 order is
                     // theirs but for near-ties, so that sorting them is mostly
@@ -830,7 +845,7 @@ inline int tile_grid(K kern, int items) {
 // e % DP), whose query coordinate is qd[t]; point rb + lane (+ 32 u) of a leaf.
 constexpr int kCapMaxLeaves = 17;
 
-template <int DP, int KC>
+template <int DP, int KC, int OP = OP_NEAR>
 __global__ void __launch_bounds__(kQB) k_query_cap(const TileArgs a, float* qcap, int budget) {
     constexpr int NE = (KC + 31) / 32;      // list entries per lane
     constexpr int NT = (2 * DP + 31) / 32;  // box elements per lane
@@ -904,7 +919,8 @@ __global__ void __launch_bounds__(kQB) k_query_cap(const TileArgs a, float* qcap
                     if (e < 2 * DP) {
                         const int c = e / DP, d = e % DP;
                         const float lo = bx[c * 2 * DP + d], hi = bx[c * 2 * DP + DP + d];
-                        const float g = fmaxf(fmaxf(lo - qd[t], qd[t] - hi), 0.f);
+                        const float g = OP == OP_FAR ? fmaxf(qd[t] - lo, hi - qd[t])
+                                                     : fmaxf(fmaxf(lo - qd[t], qd[t] - hi), 0.f);
                         const float w = qd[t] - 0.5f * (lo + hi);
                         if (c == 0) {
                             s0 = fmaf(g, g, s0);
@@ -915,7 +931,7 @@ __global__ void __launch_bounds__(kQB) k_query_cap(const TileArgs a, float* qcap
                         }
                     }
                 }
-                const bool ball = P.bound != DTREE_BOUND_BOX;  // uniform over the warp
+                const bool ball = OP == OP_NEAR && P.bound != DTREE_BOUND_BOX;  // uniform over the warp
                 float dl, dr;
                 if (2 * DP <= 32) {
                     // child c's coordinates sit in lanes [c DP, c DP + DP)
@@ -950,6 +966,10 @@ __global__ void __launch_bounds__(kQB) k_query_cap(const TileArgs a, float* qcap
                     dl = both ? fmaxf(dl, gl * gl) : gl * gl;
                     dr = both ? fmaxf(dr, gr * gr) : gr * gr;
                 }
+                if (OP == OP_FAR) {  // negated squared d_max: the farther child is the smaller
+                    dl = -dl;
+                    dr = -dr;
+                }
                 const bool right = dr < dl;
                 const float df = right ? dl : dr;
                 if (df < kth) {
@@ -975,7 +995,7 @@ __global__ void __launch_bounds__(kQB) k_query_cap(const TileArgs a, float* qcap
                 for (int r0 = 0; r0 < rc; r0 += 32) {
                     const int r = rb + r0 + lane;
                     float d = INFINITY;
-                    if (r0 + lane < rc && !(mono && r == myq)) d = approx_d2<DP>(q, P.rpts + (int64_t)r * DP);
+                    if (r0 + lane < rc && !(mono && r == myq)) d = (OP == OP_FAR ? -1.f : 1.f) * approx_d2<DP>(q, P.rpts + (int64_t)r * DP);
                     uint32_t m = __ballot_sync(0xffffffffu, d < INFINITY && key_less(d, r, td, ti));
                     while (m) {
                         const int src = __ffs(m) - 1;
@@ -1035,40 +1055,38 @@ __global__ void __launch_bounds__(kQB) k_query_cap(const TileArgs a, float* qcap
             }
         }
         if (lane == 0) {
-            const float cap = ub_of<float, DP>(kth);
+            const float cap = ub_op<DP, OP>(kth);
             qcap[row] = cap;
             a.qub[row] = fminf(a.qub[row], cap);
         }
     }
 }
 
+// One CTA per work item, or, where the items alone do not fill the GPU, as many
+// as do (a warp then serves a few of the item's queries instead of 32 in a row:
+// 64 items at d = 16, 0.60 -> 0.08 ms).
+template <int DP, int KC, int OP>
+int launch_query_cap_as(const TileArgs& a, int budget, float* qcap, cudaStream_t s) {
+    auto kern = k_query_cap<DP, KC, OP>;
+    const int split = std::max(1, std::min(32, occupancy_grid((const void*)kern, kQB, 0) / a.nitems));
+    DT_LAUNCH(kern, dim3(a.nitems, split), kQB, 0, s, a, qcap, std::min(budget, kCapMaxLeaves));
+    return DTREE_OK;
+}
+
 template <int DP>
 int launch_query_cap(const TileArgs& a, int kc, int budget, float* qcap, cudaStream_t s) {
     if (a.nitems <= 0) return DTREE_OK;
     if (budget < 1 || kc != a.kc_rows) return DTREE_ERR_UNSUPPORTED;
-    budget = std::min(budget, kCapMaxLeaves);
-    // one CTA per work item, or, where the items alone do not fill the GPU, as
-    // many as do (a warp then serves a few of the item's queries instead of 32
-    // in a row: 64 items at d = 16, 0.60 -> 0.08 ms)
-#define DT_CAP_CASE(KCV)                                                   \
-    case KCV: {                                                            \
-        auto kern = k_query_cap<DP, KCV>;                                  \
-        const int split = std::max(1, std::min(32, occupancy_grid((const void*)kern, kQB, 0) / a.nitems)); \
-        DT_LAUNCH(kern, dim3(a.nitems, split), kQB, 0, s, a, qcap, budget); \
-        return DTREE_OK;                                                   \
-    }
     switch (kc) {
-        DT_CAP_CASE(4)
-        DT_CAP_CASE(8)
-        DT_CAP_CASE(16)
-        DT_CAP_CASE(24)
-        DT_CAP_CASE(32)
-        DT_CAP_CASE(48)
-        DT_CAP_CASE(64)
-        default:
-            return DTREE_ERR_UNSUPPORTED;
+        case 4: return launch_query_cap_as<DP, 4, OP_NEAR>(a, budget, qcap, s);
+        case 8: return launch_query_cap_as<DP, 8, OP_NEAR>(a, budget, qcap, s);
+        case 16: return launch_query_cap_as<DP, 16, OP_NEAR>(a, budget, qcap, s);
+        case 24: return launch_query_cap_as<DP, 24, OP_NEAR>(a, budget, qcap, s);
+        case 32: return launch_query_cap_as<DP, 32, OP_NEAR>(a, budget, qcap, s);
+        case 48: return launch_query_cap_as<DP, 48, OP_NEAR>(a, budget, qcap, s);
+        case 64: return launch_query_cap_as<DP, 64, OP_NEAR>(a, budget, qcap, s);
+        default: return DTREE_ERR_UNSUPPORTED;
     }
-#undef DT_CAP_CASE
 }
 
 template <int DP>
