@@ -1,7 +1,6 @@
 // kfn.cu -- dtree_kfn: exact k-furthest-neighbour search, host side (the
 // kernels and their reading of Section 5 are in kfn.cuh).
 #include <algorithm>
-#include <cmath>
 #include <cstring>
 
 #include "kfn.cuh"
@@ -20,9 +19,7 @@ int kfn_launch(int dp, const KfnArgs& a, int kc, bool exact, int grid, cudaStrea
 }
 
 // Whether the block search serves a problem: enough work that its passes pay
-// (d > 8 and 1e9 pairs), and extents (the reference points' radius R about their box centre, the
-// queries' largest distance from it) that keep the squares and the bounds
-// relative to them inside float32's range.  Reads both roots back.
+// (d > 8, 4096 queries and 1e9 pairs), and extents that its float32 bounds cover.
 //
 // A walk per query visits few leaves where the box bound prunes well (d <= 8:
 // 1M x 100k uniform points in d = 3 3.6 ms against 5.4; 1M x 30k in d = 8 5.9
@@ -37,21 +34,9 @@ int kfn_tiles_fit(const dtree_t* tq, const dtree_t* tr, cudaStream_t s, bool* fi
     cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, tr->device);
     cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, tr->device);
     if (major != 10 || minor != 3) return DTREE_OK;  // the tiles are tcgen05 code
-    if (tr->dp < 16 || (double)tq->n * (double)tr->n < 1e9) return DTREE_OK;
-    float qb[128], rb[128], ql = 0.f, rl = 0.f;
-    const size_t row = (size_t)2 * tr->dp * sizeof(float);
-    DT_CHECK(cudaMemcpyAsync(qb, tq->box, row, cudaMemcpyDeviceToHost, s));
-    DT_CHECK(cudaMemcpyAsync(rb, tr->box, row, cudaMemcpyDeviceToHost, s));
-    DT_CHECK(cudaMemcpyAsync(&ql, tq->lam, sizeof(float), cudaMemcpyDeviceToHost, s));
-    DT_CHECK(cudaMemcpyAsync(&rl, tr->lam, sizeof(float), cudaMemcpyDeviceToHost, s));
-    DT_CHECK(cudaStreamSynchronize(s));
-    double c2 = 0.0;
-    for (int j = 0; j < tr->dp; ++j) {
-        const double t = 0.5 * ((double)qb[j] + qb[tr->dp + j]) - 0.5 * ((double)rb[j] + rb[tr->dp + j]);
-        c2 += t * t;
-    }
-    *fit = rl >= 1e-12f && rl <= 1e15f && std::sqrt(c2) + ql <= 1e15;
-    return DTREE_OK;
+    if (tr->dp < 16 || tq->n < 4096 || (double)tq->n * (double)tr->n < 1e9) return DTREE_OK;
+    double radius;
+    return extents_fit(tq, tr, s, fit, &radius);
 }
 
 }  // namespace

@@ -31,7 +31,8 @@ enum TileMode {
 // that "smaller is better" holds throughout and B_1, A + 2 lambda and Score keep
 // their form (Section 5's paragraph on k-furthest neighbours inverts the rules;
 // this inverts the distances).
-enum SearchOp { OP_NEAR = 0, OP_FAR = 1 };
+// A range search visits the leaf pairs within its range and keeps no lists.
+enum SearchOp { OP_NEAR = 0, OP_FAR = 1, OP_RANGE = 2 };
 
 constexpr int kQB = 128;           // queries of one work item (one thread each)
 constexpr int kEmptyIdx = 0x7fffffff;
@@ -77,6 +78,7 @@ struct ProbDev {
     int32_t Lp;       // level of the learned proposal's cells (the proposed seed subtrees)
     int32_t item0;    // first work item of the problem
     int32_t bound;    // dtree_bound of the node and point lower bounds
+    float lo_dn;      // range search: a float below d_lo (0: no lower end)
 };
 
 // ---- lower bounds on distances to a node (Section 3: d_min), rounded down
@@ -157,6 +159,20 @@ __device__ __forceinline__ float box_dmax_neg(const float* a, const float* b) {
     return -__fmul_ru(__fsqrt_ru(s), 1.f + rel_eps<DP>());
 }
 
+// A range search's range, the floats around its squared ends that settle a
+// float32 key (range.cuh), and where its results go.
+struct RangeOut {
+    double d_lo, d_hi;
+    float hi_up;                  // a float above d_hi
+    float lo2_dn, lo2_up;
+    float hi2_dn, hi2_up;
+    int fill;                     // 0: counts per caller row; 1: the segments at offsets
+    int64_t* counts;
+    const int64_t* offsets;
+    int64_t* out_idx;
+    float* out_dist;
+};
+
 // What the one-warp-per-query furthest-neighbour kernels read and write.
 struct KfnArgs {
     // query points in query-tree order (DP floats each) and their caller rows
@@ -214,6 +230,7 @@ struct TileArgs {
     int fb_slices;
     void* fb_part;
     unsigned long long* stats;
+    RangeOut range;    // (OP_RANGE)
 };
 
 template <int DP>
@@ -235,7 +252,7 @@ int launch_tile_tc(const TileArgs& a, int fmt, int kc, int items, bool wide, int
                    cudaStream_t s);
 
 // The furthest-neighbour search's seed tile, cap and tensor-core passes (BF16),
-// with lists of 16, 32 or 64 (seed) and 24, 32 or 64 entries.
+// with lists of 24, 32 or 64 entries.
 template <int DP>
 int launch_far_seed(const TileArgs& a, int kc, int items, cudaStream_t s);
 template <int DP>
@@ -245,6 +262,21 @@ int launch_far_tile(const TileArgs& a, int kc, int items, bool wide, int* err, i
 // ... and the float64 search of the queries listed in a.fb_list (kfn.cuh).
 template <int DP>
 int launch_kfn(const KfnArgs& a, int kc, bool exact, int grid, cudaStream_t s);
+
+// The range search's tensor-core pass (BF16).
+template <int DP>
+int launch_range_tile(const TileArgs& a, int items, int* err, int spin, cudaStream_t s);
+
+// One pass (count or fill) of a range search by block traversal and tensor-core
+// tiles; range.cu checks that it fits.  Adds to st when given.
+int range_by_tiles(const dtree_t* tq, const dtree_t* tr, bool mono, const RangeOut& r, cudaStream_t s,
+                   dtree_stats* st);
+
+// Whether a problem's extents (the reference points' radius R about their box
+// centre, the queries' largest distance from it) keep squared distances, and
+// the tensor-core keys' bounds relative to R^2, inside float32's range; *radius
+// is then the larger of the two.  Reads both roots back.
+int extents_fit(const dtree_t* tq, const dtree_t* tr, cudaStream_t s, bool* fit, double* radius);
 
 // dtree_kfn by these passes: one problem whose extents keep every squared
 // distance inside float32's range (kfn.cu checks).  Adds to st when given.

@@ -426,6 +426,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
     using S = TcShape<FMT, DP>;
     using L = TcSmem<FMT, DP, KC, NG, QH>;
     using Bd = TcBound<FMT, DP, OP>;
+    constexpr bool LISTS = OP != OP_RANGE;
     constexpr int TN = L::TN, TN8 = L::TN8, NACC = L::NACC, NB = L::NB, GR = L::GR, CB = L::CB, WIN = L::WIN;
     constexpr bool WIDE = NG == 1 || KC <= 24;  // 64-column reads
     constexpr int PW = 4 * NG, MW = 4 * NG + 2;  // the first planner's and the MMA issuer's warps
@@ -528,6 +529,8 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
         const float qc = act && a.qcap ? a.qcap[P.q0 + myq] : INFINITY;
         float ld[KC];
         int li[KC];
+        int64_t found = 0;        // OP_RANGE: this thread's results
+        if (OP == OP_RANGE) acur = epi ? (uint32_t)grp_id : 0u;  // (a group's tiles, so the order written, follow from the item)
         if (epi) {
             // the query, centred and rounded, as row qt of the A tile
             float h[DP];
@@ -556,10 +559,10 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
             qa = __fsqrt_ru(qa2);
 #pragma unroll
             for (int j = 0; j < KC; ++j) {
-                ld[j] = act ? a.cand_d[(int64_t)j * a.nq_all + (P.q0 + myq)] : INFINITY;
-                li[j] = act ? a.cand_i[(int64_t)j * a.nq_all + (P.q0 + myq)] : kEmptyIdx;
+                ld[j] = LISTS && act ? a.cand_d[(int64_t)j * a.nq_all + (P.q0 + myq)] : INFINITY;
+                li[j] = LISTS && act ? a.cand_i[(int64_t)j * a.nq_all + (P.q0 + myq)] : kEmptyIdx;
             }
-            float ub = fminf(Bd::ub(list_at(ld, kq - 1), qa, rad), qc);
+            float ub = LISTS ? fminf(Bd::ub(list_at(ld, kq - 1), qa, rad), qc) : INFINITY;
             float vmax = act ? ub : -INFINITY, vmin = act ? ub : INFINITY;
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) {
@@ -889,8 +892,10 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
             // when the list does
             // the list's k-th key, kept at hand: it changes only when an
             // insertion lands before it
-            float kd = list_at(ld, kq - 1);
+            float kd = LISTS ? list_at(ld, kq - 1) : INFINITY;
             auto threshold = [&]() {
+                // every point within the range has a key up to its band
+                if (!LISTS) return __fsub_ru(Bd::band(a.range.hi_up, qa, rad), qn);
                 const float bnd = Bd::band(fminf(Bd::ub(kd, qa, rad), qc), qa, rad);
                 return __fsub_ru(fminf(ld[KC - 1], bnd), qn);
             };
@@ -900,6 +905,39 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
             // candidates under the threshold are buffered per thread and
             // inserted together by the whole warp at the end of the tile
             auto flush = [&]() {
+                if constexpr (!LISTS) {
+                    // decide each candidate as range.cuh does: on a float32 key
+                    // where that settles it, else on its float64 distance.  Group
+                    // 0's results fill a segment from its start, group 1's from
+                    // its end
+                    const float* qp = P.qpts + (int64_t)myq * DP;
+                    const float eps = rel_eps<DP>();
+                    for (int e = 0; e < nb; ++e) {
+                        const int rp = bi[e * kQB];
+                        if (rp == kEmptyIdx || (mono && rp == myq)) continue;
+                        const float* rq = P.rpts + (int64_t)rp * DP;
+                        const float kf = approx_d2<DP>(qp, rq);
+                        const float k_dn = __fmul_rd(kf, 1.f - 2.f * eps), k_up = __fmul_ru(kf, 1.f + 2.f * eps);
+                        if (k_up < a.range.lo2_dn || k_dn > a.range.hi2_up) continue;
+                        if (!a.range.fill && k_dn >= a.range.lo2_up && k_up <= a.range.hi2_dn) {
+                            ++found;
+                            continue;
+                        }
+                        ++n_re;
+                        const double d = sqrt(exact_d2<DP>(qp, rq));
+                        if (!(d >= a.range.d_lo && d <= a.range.d_hi)) continue;
+                        if (a.range.fill) {
+                            const int64_t row = P.qidx[myq];
+                            const int64_t at = grp_id == 0 ? a.range.offsets[row] + found
+                                                           : a.range.offsets[row + 1] - 1 - found;
+                            a.range.out_idx[at] = P.ridx[rp];
+                            a.range.out_dist[at] = (float)d;
+                        }
+                        ++found;
+                    }
+                    nb = 0;
+                    return;
+                }
                 for (int e = 0; e < nb; ++e) {
                     const float sv = qn + bw[e * kQB];
                     const int rp = bi[e * kQB];
@@ -1107,7 +1145,14 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
         // the buffers the re-rank would reuse)
         __syncthreads();
         if (s_fail) break;
-        if (epi && NG == 2 && QH == 1) {
+        if (!LISTS && !a.range.fill) {
+            // the groups' counts of each query
+            int64_t* cnt = reinterpret_cast<int64_t*>(smem);
+            if (epi && grp_id == 1) cnt[qt] = found;
+            __syncthreads();
+            if (epi && grp_id == 0 && act) a.range.counts[P.qidx[myq]] = found + (NG == 2 ? cnt[qt] : 0);
+        }
+        if (LISTS && epi && NG == 2 && QH == 1) {
             // merge group 1's lists into group 0's
             float* smd = reinterpret_cast<float*>(smem);
             int32_t* smi = reinterpret_cast<int32_t*>(smem + kQB * KC * 4);
@@ -1130,7 +1175,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
             // the re-rank below reuses the merge buffers: group 0 has read them
             tc::named_sync(1, 256);
         }
-        if (epi && (QH == 2 || grp_id == 0)) {
+        if (LISTS && epi && (QH == 2 || grp_id == 0)) {
             // ---- finish the work item
             long long tf0 = TC_TIMED ? clock64() : 0;
             const float ubk = fminf(Bd::ub(list_at(ld, kq - 1), qa, rad), qc);
@@ -1345,7 +1390,7 @@ int launch_far_seed(const TileArgs& a, int kc, int items, cudaStream_t s) {
         DT_LAUNCH(kern, tile_grid(kern, items), kQB, 0, s, a);            \
         return DTREE_OK;                                                  \
     }
-    DT_FAR_SEED(16)
+    DT_FAR_SEED(24)
     DT_FAR_SEED(32)
     DT_FAR_SEED(64)
 #undef DT_FAR_SEED
@@ -1373,6 +1418,14 @@ int launch_far_tile(const TileArgs& a, int kc, int items, bool wide, int* err, i
                     : launch_tile_tc_as<3, DP, 32, NG, 1, OP_FAR>(a, x, items, s);
     if (kc == 64) return launch_tile_tc_as<3, DP, 64, 1, 1, OP_FAR>(a, x, items, s);
     return DTREE_ERR_UNSUPPORTED;
+}
+
+// The range search's pass: no lists (KC only sizes buffers), two groups that
+// take every second tile of an item.
+template <int DP>
+int launch_range_tile(const TileArgs& a, int items, int* err, int spin, cudaStream_t s) {
+    TcExtra x{err, spin, g_tc_timers, g_tc_stall};
+    return launch_tile_tc_as<3, DP, 16, 2, 1, OP_RANGE>(a, x, items, s);
 }
 
 }  // namespace dt

@@ -67,6 +67,51 @@ int range_grid(int64_t nq) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((nq + 3) / 4, (int64_t)sms * 16));
 }
 
+RangeOut range_out(const RangeArgs& a, bool fill) {
+    RangeOut r{};
+    r.d_lo = a.d_lo;
+    r.d_hi = a.d_hi;
+    const float hi = (float)(a.d_hi * (1.0 + 1e-12));
+    r.hi_up = std::isinf(hi) ? hi : std::nextafter(hi, INFINITY);
+    r.lo2_dn = a.lo2_dn;
+    r.lo2_up = a.lo2_up;
+    r.hi2_dn = a.hi2_dn;
+    r.hi2_up = a.hi2_up;
+    r.fill = fill ? 1 : 0;
+    r.counts = a.counts;
+    r.offsets = a.offsets;
+    r.out_idx = a.out_idx;
+    r.out_dist = a.out_dist;
+    return r;
+}
+
+// Whether the block search serves a range: enough work that its passes pay
+// (d > 8, 10k queries and 1e9 pairs), a candidate bit per (block, leaf) in at most 1 GB,
+// extents that its float32 bounds cover, and a range whose square is at least
+// 4e-4 of the largest squared extent, so that the tensor-core keys' error
+// (about 1e-4 of it) adds few candidates.  Both passes of a search decide alike.
+//
+// A walk per query visits few leaves where the box bound prunes well (d <= 8),
+// and a few queries make too few blocks for the GPU (mixture, d = 16, radius
+// 2.4: 1M x 2k points 5.3 against 6.9 ms, 300k x 5k 4.4 against 4.6).  Above,
+// blocks share the visits and the tensor cores do the distances: 100k x 20k
+// 4.2 -> 3.9 ms, 1M x 20k 16.5 -> 6.9, 1M x 100k 64 -> 10.3; 300k x 100k in d =
+// 32 91 -> 13; 100k x 20k in d = 64 179 -> 21; points of three latent
+// dimensions 6.3 -> 6.2.
+int range_tiles_fit(const dtree_t* tq, const dtree_t* tr, double d_hi, cudaStream_t s, bool* fit) {
+    *fit = false;
+    int major = 0, minor = 0;
+    cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, tr->device);
+    cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, tr->device);
+    if (major != 10 || minor != 3) return DTREE_OK;  // the tiles are tcgen05 code
+    if (tr->dp < 16 || tq->n < 10000 || (double)tq->n * (double)tr->n < 1e9) return DTREE_OK;
+    if ((double)tq->n / 64.0 * (double)tr->nleaves / 8.0 > 1e9) return DTREE_OK;
+    double radius = 0.0;
+    const int rc = extents_fit(tq, tr, s, fit, &radius);
+    if (!(d_hi * d_hi >= 4e-4 * radius * radius)) *fit = false;
+    return rc;
+}
+
 }  // namespace
 }  // namespace dt
 
@@ -89,6 +134,7 @@ extern "C" int dtree_range_count(const dtree_t* query, const dtree_t* ref, doubl
     a.counts = offsets;
     a.stats = cnt;
     unsigned long long h[4] = {0, 0, 0, 0};
+    dtree_stats tst{};  // the block search's counters
     cudaEvent_t ev[2] = {};
     const bool timed = st && cudaEventCreate(&ev[0]) == cudaSuccess && cudaEventCreate(&ev[1]) == cudaSuccess;
     cudaGetLastError();
@@ -98,7 +144,15 @@ extern "C" int dtree_range_count(const dtree_t* query, const dtree_t* ref, doubl
             break;
         }
         if (timed) cudaEventRecord(ev[0], s);
-        rc = range_launch(ref->dp, a, false, range_grid(a.nq), s);
+        bool tiles = false;
+        rc = range_tiles_fit(query ? query : ref, ref, d_hi, s, &tiles);
+        if (rc != DTREE_OK) break;
+        if (tiles) {
+            rc = range_by_tiles(query ? query : ref, ref, a.mono != 0, range_out(a, false), s, st ? &tst : nullptr);
+            if (rc == DTREE_ERR_OOM) tiles = false;  // (the walk needs no memory)
+            else if (rc != DTREE_OK) break;
+        }
+        if (!tiles) rc = range_launch(ref->dp, a, false, range_grid(a.nq), s);
         if (rc != DTREE_OK) break;
         rc = exclusive_scan(offsets, a.nq, sums, s);
         if (rc != DTREE_OK) break;
@@ -112,10 +166,10 @@ extern "C" int dtree_range_count(const dtree_t* query, const dtree_t* ref, doubl
     cudaFreeAsync(cnt, s);
     if (cudaStreamSynchronize(s) != cudaSuccess && rc == DTREE_OK) rc = cuda_status(cudaGetLastError());
     if (st && rc == DTREE_OK) {
-        st->point_pairs = (int64_t)h[0];
-        st->leaf_pairs_evaluated = (int64_t)h[1];
-        st->node_pairs_pruned = (int64_t)h[2];
-        st->rerank_candidates = (int64_t)h[3];
+        st->point_pairs = (int64_t)h[0] + tst.point_pairs;
+        st->leaf_pairs_evaluated = (int64_t)h[1] + tst.leaf_pairs_evaluated;
+        st->node_pairs_pruned = (int64_t)h[2] + tst.node_pairs_pruned;
+        st->rerank_candidates = (int64_t)h[3] + tst.rerank_candidates;
         float ms = 0.f;
         if (timed && cudaEventElapsedTime(&ms, ev[0], ev[1]) == cudaSuccess) st->ns_basecase = (int64_t)(ms * 1e6);
         st->kernel_launches = g_launches.load() - launches0;
@@ -140,7 +194,14 @@ extern "C" int dtree_range_fill(const dtree_t* query, const dtree_t* ref, double
     a.offsets = offsets;
     a.out_idx = out_idx;
     a.out_dist = out_dist;
-    rc = range_launch(ref->dp, a, true, range_grid(a.nq), s);
+    bool tiles = false;
+    rc = range_tiles_fit(query ? query : ref, ref, d_hi, s, &tiles);
+    if (rc != DTREE_OK) return rc;
+    if (tiles) {
+        rc = range_by_tiles(query ? query : ref, ref, a.mono != 0, range_out(a, true), s, nullptr);
+        if (rc == DTREE_ERR_OOM) tiles = false;
+    }
+    if (!tiles) rc = range_launch(ref->dp, a, true, range_grid(a.nq), s);
     if (cudaStreamSynchronize(s) != cudaSuccess && rc == DTREE_OK) rc = cuda_status(cudaGetLastError());
     return rc;
 }

@@ -32,7 +32,7 @@ def compare(R, Q, k, leaf=32):
     parts = []
     try:
         idx, dist = dtree.dtree_kfn(tq, tr, k)
-        step = 10 ** 9 // R.shape[0] - 1
+        step = min(4_000, 10 ** 9 // R.shape[0] - 1)
         for a in range(0, Q.shape[0], step):
             t = dtree.dtree_build(Q[a:a + step], leaf)
             parts.append(dtree.dtree_kfn(t, tr, k))
