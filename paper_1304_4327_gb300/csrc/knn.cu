@@ -875,14 +875,16 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
     // start empty, so nearly every early candidate is an insertion, which the
     // float32 tile does cheaply; its keys (relative error <= rel_eps) are
     // tighter than any tensor-core key, so the main pass's bounds hold for
-    // them.  It keeps lists of bucket(k + 1) entries (the float32 band needs
-    // no more); the main pass's other rows start empty.
+    // them.  Its lists are as long as the main pass's: a point it drops then has
+    // KC points no farther than it, and if it lies in the final band the list's
+    // last key does too, which the overflow test sees.  (Lists of bucket(k + 1)
+    // lost members of tie groups that lay wholly in the seed subtree.)
     a.kc_rows = KC;
     if (range) a.range = *range;
     if constexpr (OP == OP_FAR)
         DT_TRY(launch_far_seed<DP>(a, KC, NI, s));
     else if constexpr (OP == OP_NEAR)
-        DT_TRY(launch_tile_cc<DP>(a, kc_bucket(kmax + 1), MODE_SEED, NI, s));
+        DT_TRY(launch_tile_cc<DP>(a, KC, MODE_SEED, NI, s));
     if (qcap) {
         if constexpr (OP == OP_FAR)
             DT_TRY(launch_far_cap<DP>(a, KC, cap_leaves, qcap, s));
