@@ -588,17 +588,18 @@ int build_impl(dtree_t* t, const float* in, cudaStream_t s) {
         DT_TRY(sc.get(&sdim, maxnodes));
     }
     struct PingPong {
+        cudaStream_t s;
         float* p = nullptr;
         int32_t* i = nullptr;
         ~PingPong() {
+            if (p || i) cudaStreamSynchronize(s);  // (freeing pool memory waits for nothing)
             cudaFree(p);
             cudaFree(i);
         }
-    } pp;
+    } pp{s};
     if (Ltop > 0) {
-        g_allocs.fetch_add(2, std::memory_order_relaxed);
-        if (cudaMalloc((void**)&pp.p, (size_t)n * DP * 4) != cudaSuccess ||
-            cudaMalloc((void**)&pp.i, (size_t)n * 4) != cudaSuccess) {
+        if (tree_alloc((void**)&pp.p, (size_t)n * DP * 4, t->device, s) != cudaSuccess ||
+            tree_alloc((void**)&pp.i, (size_t)n * 4, t->device, s) != cudaSuccess) {
             cudaGetLastError();
             return DTREE_ERR_OOM;
         }
@@ -707,18 +708,24 @@ extern "C" int dtree_build(const float* pts, int64_t n, int32_t d, const dtree_o
     int rc = DTREE_OK;
     auto alloc = [&](void** p, size_t bytes) {
         if (rc != DTREE_OK) return;
-        dt::g_allocs.fetch_add(1, std::memory_order_relaxed);
-        if (cudaMalloc(p, bytes) != cudaSuccess) {
+        if (dt::tree_alloc(p, bytes, t->device, s) != cudaSuccess) {
             cudaGetLastError();
             rc = DTREE_ERR_OOM;
         }
     };
     alloc((void**)&t->pts, (size_t)n * t->dp * 4);
     alloc((void**)&t->idx, (size_t)n * 4);
-    alloc((void**)&t->box, (size_t)t->nnodes * 2 * t->dp * 4);
-    alloc((void**)&t->lam, (size_t)t->nnodes * 4);
-    alloc((void**)&t->nbeg, (size_t)t->nnodes * 4);
-    alloc((void**)&t->ncnt, (size_t)t->nnodes * 4);
+    // box, lam, nbeg and ncnt in one block
+    const size_t b_box = ((size_t)t->nnodes * 2 * t->dp * 4 + 255) & ~(size_t)255;
+    const size_t b_row = ((size_t)t->nnodes * 4 + 255) & ~(size_t)255;
+    alloc(&t->block, b_box + 3 * b_row);
+    if (rc == DTREE_OK) {
+        unsigned char* m = static_cast<unsigned char*>(t->block);
+        t->box = reinterpret_cast<float*>(m);
+        t->lam = reinterpret_cast<float*>(m + b_box);
+        t->nbeg = reinterpret_cast<int32_t*>(m + b_box + b_row);
+        t->ncnt = reinterpret_cast<int32_t*>(m + b_box + 2 * b_row);
+    }
     if (rc == DTREE_OK) {
         switch (t->dp) {
             case 4: rc = dt::build_impl<4>(t, pts, s); break;

@@ -32,6 +32,7 @@ struct dtree {
     int32_t* nbeg = nullptr;
     int32_t* ncnt = nullptr;
     int device = 0;
+    void* block = nullptr;  // the arrays above but pts and idx
     // frontier capacity that sufficed for the last traversal against this
     // reference tree (a sizing hint only; results never depend on it)
     int64_t cap_hint = 0;
@@ -136,5 +137,10 @@ inline int scratch(T** p, size_t count, cudaStream_t s) {
 }
 
 void prepare_pool(int device);
+
+// A tree's memory (ready when the call returns or, from the pool, in stream
+// order on s; every library call waits for its stream, so it may then be used
+// on any) and its release, which the caller's work must have finished with.
+cudaError_t tree_alloc(void** p, size_t bytes, int device, cudaStream_t s);
 
 }  // namespace dt
