@@ -14,9 +14,9 @@
 //          order-preserving uint32 keys), and a scatter into the children.
 //          Many CTAs work on one node.
 //   bottom one CTA per remaining subtree: the subtree's points are staged in
-//          shared memory and split level by level with a bitonic sort on
-//          (segment, key, slot) composite keys; boxes and the exact lambda of
-//          every node of the subtree are written on the way.
+//          shared memory and split level by level with a bitonic sort of each
+//          segment on (key, slot); boxes and the exact lambda of every node of
+//          the subtree are written on the way.
 // lambda of top-phase nodes is bounded from their children:
 //   lambda(N) <= max_c ( |C_N - C_c| + lambda(c) )   (triangle inequality),
 // rounded upward, which keeps it a valid bound for the B_2 term of Section 5.
@@ -29,7 +29,11 @@ namespace dt {
 namespace {
 
 constexpr int kTPB = 256;            // threads of the top-phase kernels
-constexpr int kChunk = 4096;         // elements per CTA in a top-phase pass
+// Elements per CTA in a top-phase pass: small sets take small chunks, so that a
+// pass has enough CTAs (10k points in chunks of 4096 are 3 CTAs; a scatter of
+// them took 26 us).
+constexpr int kChunkSmall = 512, kChunkLarge = 4096;
+inline int chunk_of(int64_t n) { return n <= (1 << 18) ? kChunkSmall : n <= (1 << 20) ? 1024 : kChunkLarge; }
 constexpr int kBottomFloats = 8192;  // floats of points one bottom CTA stages
 constexpr int kBottomThreads = 256;
 
@@ -78,14 +82,14 @@ __global__ void k_init(const float* in, int64_t n, int d, int dp, float* pts, in
 // order-preserving encodings.
 template <int DP>
 __global__ void __launch_bounds__(kTPB) k_bbox(const float* __restrict__ pts, const int32_t* nbeg,
-                                               const int32_t* ncnt, int64_t node0, int cpn,
+                                               const int32_t* ncnt, int64_t node0, int cpn, int chunk,
                                                uint32_t* blo, uint32_t* bhi) {
     int64_t nl = blockIdx.x / cpn;
     int c = blockIdx.x % cpn;
     int64_t node = node0 + nl;
     int64_t b = nbeg[node], e = b + ncnt[node];
-    int64_t s = b + (int64_t)c * kChunk;
-    int64_t t_end = e < s + kChunk ? e : s + kChunk;
+    int64_t s = b + (int64_t)c * chunk;
+    int64_t t_end = e < s + chunk ? e : s + chunk;
     if (s >= t_end) return;
     constexpr int RPI = kTPB / DP;
     int j = threadIdx.x % DP;
@@ -138,7 +142,7 @@ __global__ void k_box_decode(const uint32_t* blo, const uint32_t* bhi, int64_t n
 template <int DP>
 __global__ void __launch_bounds__(kTPB) k_keys_hist(const float* __restrict__ pts,
                                                     const int32_t* nbeg, const int32_t* ncnt,
-                                                    int64_t node0, int cpn, const uint8_t* sdim,
+                                                    int64_t node0, int cpn, int chunk, const uint8_t* sdim,
                                                     uint32_t* keys, uint32_t* ghist) {
     __shared__ uint32_t h[2048];
     for (int i = threadIdx.x; i < 2048; i += kTPB) h[i] = 0;
@@ -147,8 +151,8 @@ __global__ void __launch_bounds__(kTPB) k_keys_hist(const float* __restrict__ pt
     int c = blockIdx.x % cpn;
     int64_t node = node0 + nl;
     int64_t b = nbeg[node], e = b + ncnt[node];
-    int64_t s = b + (int64_t)c * kChunk;
-    int64_t t_end = e < s + kChunk ? e : s + kChunk;
+    int64_t s = b + (int64_t)c * chunk;
+    int64_t t_end = e < s + chunk ? e : s + chunk;
     int dim = sdim[nl];
     for (int64_t i = s + threadIdx.x; i < t_end; i += kTPB) {
         uint32_t key = f2o(pts[i * DP + dim]);
@@ -163,7 +167,7 @@ __global__ void __launch_bounds__(kTPB) k_keys_hist(const float* __restrict__ pt
 // Histogram pass 1 (bits 20..10 among keys whose top 11 bits match) or
 // pass 2 (bits 9..0 among keys whose top 22 bits match).
 __global__ void __launch_bounds__(kTPB) k_hist(const uint32_t* keys, const int32_t* nbeg,
-                                               const int32_t* ncnt, int64_t node0, int cpn,
+                                               const int32_t* ncnt, int64_t node0, int cpn, int chunk,
                                                int pass, const uint32_t* prefix,
                                                uint32_t* ghist) {
     __shared__ uint32_t h[2048];
@@ -173,8 +177,8 @@ __global__ void __launch_bounds__(kTPB) k_hist(const uint32_t* keys, const int32
     int c = blockIdx.x % cpn;
     int64_t node = node0 + nl;
     int64_t b = nbeg[node], e = b + ncnt[node];
-    int64_t s = b + (int64_t)c * kChunk;
-    int64_t t_end = e < s + kChunk ? e : s + kChunk;
+    int64_t s = b + (int64_t)c * chunk;
+    int64_t t_end = e < s + chunk ? e : s + chunk;
     uint32_t pre = prefix[nl];
     int hi_shift = pass == 1 ? 21 : 10;
     int lo_shift = pass == 1 ? 10 : 0;
@@ -199,39 +203,42 @@ __global__ void __launch_bounds__(kTPB) k_select(const int32_t* ncnt, int64_t no
     int nbins = pass == 2 ? 1024 : 2048;
     int per = nbins / kTPB;
     uint32_t* h = ghist + nl * 2048;
-    __shared__ int32_t ssum[kTPB];
+    __shared__ int32_t wsum[kTPB / 32];
     __shared__ int32_t sres[3];
     if (pass == 0 && threadIdx.x == 0) {
         rank[nl] = ncnt[node0 + nl] / 2 - 1;
         less[nl] = 0;
         prefix[nl] = 0;
     }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // this thread's `per` (8 or 4) consecutive bins
+    int32_t v[8];
+    int32_t sum = 0;
+    const uint4* h4 = reinterpret_cast<const uint4*>(h + threadIdx.x * per);
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u), b0 = h4[0], b1 = per == 8 ? h4[1] : z;
+    v[0] = b0.x, v[1] = b0.y, v[2] = b0.z, v[3] = b0.w, v[4] = b1.x, v[5] = b1.y, v[6] = b1.z, v[7] = b1.w;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) sum += v[q];
+    int32_t incl = sum;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int32_t u = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += u;
+    }
+    if (lane == 31) wsum[warp] = incl;
     __syncthreads();
     int32_t r = rank[nl];
-    int32_t sum = 0;
-    for (int q = 0; q < per; ++q) sum += (int32_t)h[threadIdx.x * per + q];
-    ssum[threadIdx.x] = sum;
-    __syncthreads();
-    // exclusive scan (Hillis-Steele over 256 entries)
-    for (int off = 1; off < kTPB; off <<= 1) {
-        int32_t v = threadIdx.x >= off ? ssum[threadIdx.x - off] : 0;
-        __syncthreads();
-        ssum[threadIdx.x] += v;
-        __syncthreads();
-    }
-    int32_t incl = ssum[threadIdx.x];
+    for (int w = 0; w < warp; ++w) incl += wsum[w];
     int32_t excl = incl - sum;
     if (r >= excl && r < incl) {
         int32_t cum = excl;
         int bin = threadIdx.x * per;
-        for (int q = 0; q < per; ++q) {
-            int32_t v = (int32_t)h[threadIdx.x * per + q];
-            if (r < cum + v) {
-                bin = threadIdx.x * per + q;
-                break;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (r >= cum + v[q] && bin == (int)threadIdx.x * per + q) {
+                cum += v[q];
+                ++bin;
             }
-            cum += v;
-        }
         sres[0] = bin;
         sres[1] = cum;
     }
@@ -255,15 +262,15 @@ __global__ void __launch_bounds__(kTPB) k_scatter(const float* __restrict__ src,
                                                   const int32_t* __restrict__ isrc,
                                                   float* __restrict__ dst, int32_t* __restrict__ idst,
                                                   const uint32_t* keys, const int32_t* nbeg,
-                                                  const int32_t* ncnt, int64_t node0, int cpn,
+                                                  const int32_t* ncnt, int64_t node0, int cpn, int chunk,
                                                   const uint32_t* msplit, const int32_t* eq_left,
                                                   int32_t* eq_ctr, int32_t* cursor, int* bad) {
     int64_t nl = blockIdx.x / cpn;
     int c = blockIdx.x % cpn;
     int64_t node = node0 + nl;
     int64_t b = nbeg[node], cnt = ncnt[node], e = b + cnt;
-    int64_t s = b + (int64_t)c * kChunk;
-    int64_t t_end = e < s + kChunk ? e : s + kChunk;
+    int64_t s = b + (int64_t)c * chunk;
+    int64_t t_end = e < s + chunk ? e : s + chunk;
     int64_t half = cnt / 2;
     uint32_t m = msplit[nl];
     int32_t eql = eq_left[nl];
@@ -394,6 +401,14 @@ __device__ void seg_stats(const float* sp, const uint64_t* sk, int sb, int cnt, 
     __syncwarp();
 }
 
+// A segment of level j keeps to a block of B = S2 >> j slots of its own (S2 the
+// power of two that holds the subtree; a level's segments differ by one point,
+// so none outgrows its block), padded with the largest key.  Sorting within
+// blocks takes log2(B) (log2(B) + 1) / 2 steps instead of those of all S2 slots
+// at every level (266 against 462 for 2048 slots and 7 levels), and a step
+// whose partners lie in one warp's eighth of the slots needs no CTA barrier
+// (all but 10).  Build and release of 10k points, d = 3: 605 -> 304 us; of 10M, d
+// = 8: 9.6 -> 8.8 ms (with the smaller chunks above and the tree pool).
 template <int DP>
 __global__ void __launch_bounds__(kBottomThreads) k_bottom(float* pts, int32_t* idx,
                                                            const int32_t* nbeg,
@@ -401,9 +416,10 @@ __global__ void __launch_bounds__(kBottomThreads) k_bottom(float* pts, int32_t* 
                                                            int d, float* box, float* lam) {
     constexpr int S = bottom_cap<DP>();
     constexpr int NW = kBottomThreads / 32;
+    constexpr int EPT = S > kBottomThreads ? S / kBottomThreads : 1;  // slots per thread, at most
     extern __shared__ __align__(16) unsigned char smem[];
     float* sp = reinterpret_cast<float*>(smem);                // S * DP points
-    uint64_t* sk = reinterpret_cast<uint64_t*>(sp + S * DP);   // S composite keys
+    uint64_t* sk = reinterpret_cast<uint64_t*>(sp + S * DP);   // S keys (key << 16 | slot of the point)
     float* scen = reinterpret_cast<float*>(sk + S);            // NW * DP centres
     int32_t* so = reinterpret_cast<int32_t*>(scen + NW * DP);  // S input rows
     uint16_t* sseg = reinterpret_cast<uint16_t*>(so + S);      // S + 2 segment begins
@@ -411,59 +427,120 @@ __global__ void __launch_bounds__(kBottomThreads) k_bottom(float* pts, int32_t* 
 
     int64_t root = ((int64_t)1 << Ltop) - 1 + blockIdx.x;
     int rb = nbeg[root], rc = ncnt[root];
-    int tid = threadIdx.x, warp = tid >> 5;
+    int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int lg = 6;  // log2(S2)
+    while ((1 << lg) < rc) ++lg;
+    const int S2 = min(1 << lg, S);  // (rc <= S, and S is a power of two)
+    lg = 31 - __clz(S2);
     for (int f = tid; f < rc * DP; f += kBottomThreads) sp[f] = pts[(int64_t)rb * DP + f];
     for (int e = tid; e < rc; e += kBottomThreads) so[e] = idx[rb + e];
-    for (int e = tid; e < S; e += kBottomThreads) sk[e] = e < rc ? (uint64_t)e : ~0ull;
+    for (int e = tid; e < S2; e += kBottomThreads) sk[e] = e < rc ? (uint64_t)e : ~0ull;
     __syncthreads();
     int nsub = h - Ltop;
+    // a warp's own slots: an eighth of them, 64 at least
+    const int C = max(64, S2 / NW);
     for (int j = 0; j <= nsub; ++j) {
         int nseg = 1 << j;
+        const int lb = lg - j, B = 1 << lb;  // slots per segment
         int64_t first = (root + 1) * nseg - 1;
         for (int s = tid; s < nseg; s += kBottomThreads) sseg[s] = (uint16_t)(nbeg[first + s] - rb);
         if (tid == 0) sseg[nseg] = (uint16_t)rc;
         __syncthreads();
         for (int s = warp; s < nseg; s += NW) {
-            int sb = sseg[s], cnt = sseg[s + 1] - sb;
-            seg_stats<DP>(sp, sk, sb, cnt, d, box + (first + s) * 2 * DP, lam + first + s, sdim + s,
+            int cnt = sseg[s + 1] - sseg[s];
+            seg_stats<DP>(sp, sk, s << lb, cnt, d, box + (first + s) * 2 * DP, lam + first + s, sdim + s,
                           scen + warp * DP);
         }
         __syncthreads();
         if (j == nsub) break;
-        for (int e = tid; e < rc; e += kBottomThreads) {
-            int p = (int)(sk[e] & 0xffffu);
-            int lo = 0, hi = nseg - 1;  // last segment whose begin <= e
-            while (lo < hi) {
-                int mid = (lo + hi + 1) >> 1;
-                if (sseg[mid] <= e) lo = mid;
-                else hi = mid - 1;
+        for (int e = tid; e < S2; e += kBottomThreads) {
+            const int s = e >> lb;
+            if ((e & (B - 1)) < sseg[s + 1] - sseg[s]) {
+                const int p = (int)(sk[e] & 0xffffu);
+                sk[e] = ((uint64_t)f2o(sp[p * DP + sdim[s]]) << 16) | (uint64_t)p;
             }
-            uint32_t key = f2o(sp[p * DP + sdim[lo]]);
-            sk[e] = ((uint64_t)lo << 48) | ((uint64_t)key << 16) | (uint64_t)p;
         }
         __syncthreads();
-        for (int kk = 2; kk <= S; kk <<= 1) {
+        auto step = [&](int t, int kk, int jj) {
+            const int i = 2 * t - (t & (jj - 1)), l = i + jj;
+            const bool up = (i & (B - 1) & kk) == 0;  // (a block's last merge ascends)
+            const uint64_t x = sk[i], y = sk[l];
+            if ((x > y) == up) {
+                sk[i] = y;
+                sk[l] = x;
+            }
+        };
+        for (int kk = 2; kk <= B; kk <<= 1) {
             for (int jj = kk >> 1; jj > 0; jj >>= 1) {
-                for (int t = tid; t < S / 2; t += kBottomThreads) {
-                    int i = 2 * t - (t & (jj - 1));
-                    int l = i + jj;
-                    bool up = (i & kk) == 0;
-                    uint64_t a = sk[i], bb = sk[l];
-                    if ((a > bb) == up) {
-                        sk[i] = bb;
-                        sk[l] = a;
+                if (jj >= C) {
+                    __syncthreads();
+                    for (int t = tid; t < S2 / 2; t += kBottomThreads) step(t, kk, jj);
+                    __syncthreads();
+                } else if (warp * C < S2) {
+                    // up to four pairs a lane, all loaded before any is stored
+                    uint64_t x[4], y[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int t = warp * (C / 2) + lane + 32 * q, i = 2 * t - (t & (jj - 1));
+                        if (lane + 32 * q < C / 2) {
+                            x[q] = sk[i];
+                            y[q] = sk[i + jj];
+                        }
                     }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int t = warp * (C / 2) + lane + 32 * q, i = 2 * t - (t & (jj - 1));
+                        if (lane + 32 * q < C / 2 && (x[q] > y[q]) == ((i & (B - 1) & kk) == 0)) {
+                            sk[i] = y[q];
+                            sk[i + jj] = x[q];
+                        }
+                    }
+                    __syncwarp();
                 }
-                __syncthreads();
             }
         }
+        __syncthreads();
+        // a segment's points from floor(cnt / 2) on move to the second half of
+        // its block
+        uint64_t v[EPT];
+#pragma unroll
+        for (int q = 0; q < EPT; ++q) {
+            const int e = tid + q * kBottomThreads;
+            const int s = e >> lb, l = e & (B - 1);
+            v[q] = ~0ull;
+            if (e < S2) {
+                const int cnt = sseg[s + 1] - sseg[s], half = cnt / 2;
+                const int from = l < B / 2 ? (l < half ? l : -1) : (half + l - B / 2 < cnt ? half + l - B / 2 : -1);
+                if (from >= 0) v[q] = sk[(s << lb) + from];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < EPT; ++q) {
+            const int e = tid + q * kBottomThreads;
+            if (e < S2) sk[e] = v[q];
+        }
+        __syncthreads();
     }
-    for (int f = tid; f < rc * DP; f += kBottomThreads) {
-        int e = f / DP, jj = f % DP;
-        int p = (int)(sk[e] & 0xffffu);
-        pts[(int64_t)rb * DP + f] = sp[p * DP + jj];
+    // out, leaf by leaf: tree position e is slot e - begin of its leaf's block
+    const int lb = lg - nsub, nseg = 1 << nsub;
+    auto slot_of = [&](int e) {
+        int lo = 0, hi = nseg - 1;  // last leaf whose begin <= e
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (sseg[mid] <= e) lo = mid;
+            else hi = mid - 1;
+        }
+        return (int)(sk[(lo << lb) + e - sseg[lo]] & 0xffffu);
+    };
+    for (int e = tid; e < rc; e += kBottomThreads) {
+        const int p = slot_of(e);
+        idx[rb + e] = so[p];
     }
-    for (int e = tid; e < rc; e += kBottomThreads) idx[rb + e] = so[sk[e] & 0xffffu];
+    for (int f = tid; f < rc * (DP / 4); f += kBottomThreads) {
+        const int e = f / (DP / 4), q = f % (DP / 4);
+        reinterpret_cast<float4*>(pts + (int64_t)(rb + e) * DP)[q] = reinterpret_cast<const float4*>(sp + slot_of(e) * DP)[q];
+    }
 }
 
 template <int DP>
@@ -562,6 +639,7 @@ template <int DP>
 int build_impl(dtree_t* t, const float* in, cudaStream_t s) {
     const int64_t n = t->n;
     const int h = t->height;
+    const int chunk = chunk_of(n);
     Scratch sc{s};
     int* dbad = nullptr;
     DT_TRY(sc.get(&dbad, 1));
@@ -623,10 +701,10 @@ int build_impl(dtree_t* t, const float* in, cudaStream_t s) {
     auto level_boxes = [&](int L) -> int {
         int64_t node0 = ((int64_t)1 << L) - 1, nn = (int64_t)1 << L;
         int64_t maxc = (n + nn - 1) / nn;
-        int cpn = (int)((maxc + kChunk - 1) / kChunk);
+        int cpn = (int)((maxc + chunk - 1) / chunk);
         DT_CHECK(cudaMemsetAsync(blo, 0xff, nn * DP * 4, s));
         DT_CHECK(cudaMemsetAsync(bhi, 0x00, nn * DP * 4, s));
-        DT_LAUNCH(k_bbox<DP>, (int)(nn * cpn), kTPB, 0, s, src, t->nbeg, t->ncnt, node0, cpn, blo,
+        DT_LAUNCH(k_bbox<DP>, (int)(nn * cpn), kTPB, 0, s, src, t->nbeg, t->ncnt, node0, cpn, chunk, blo,
                   bhi);
         DT_LAUNCH(k_box_decode<DP>, grid_for(nn, 256), 256, 0, s, blo, bhi, node0, nn, t->d,
                   t->box, sdim);
@@ -635,20 +713,20 @@ int build_impl(dtree_t* t, const float* in, cudaStream_t s) {
     for (int L = 0; L < Ltop; ++L) {
         int64_t node0 = ((int64_t)1 << L) - 1, nn = (int64_t)1 << L;
         int64_t maxc = (n + nn - 1) / nn;
-        int cpn = (int)((maxc + kChunk - 1) / kChunk);
+        int cpn = (int)((maxc + chunk - 1) / chunk);
         int grid = (int)(nn * cpn);
         DT_TRY(level_boxes(L));
-        DT_LAUNCH(k_keys_hist<DP>, grid, kTPB, 0, s, src, t->nbeg, t->ncnt, node0, cpn, sdim, keys,
+        DT_LAUNCH(k_keys_hist<DP>, grid, kTPB, 0, s, src, t->nbeg, t->ncnt, node0, cpn, chunk, sdim, keys,
                   ghist);
         DT_LAUNCH(k_select, (int)nn, kTPB, 0, s, t->ncnt, node0, 0, ghist, prefix, rank, less, eql);
-        DT_LAUNCH(k_hist, grid, kTPB, 0, s, keys, t->nbeg, t->ncnt, node0, cpn, 1, prefix, ghist);
+        DT_LAUNCH(k_hist, grid, kTPB, 0, s, keys, t->nbeg, t->ncnt, node0, cpn, chunk, 1, prefix, ghist);
         DT_LAUNCH(k_select, (int)nn, kTPB, 0, s, t->ncnt, node0, 1, ghist, prefix, rank, less, eql);
-        DT_LAUNCH(k_hist, grid, kTPB, 0, s, keys, t->nbeg, t->ncnt, node0, cpn, 2, prefix, ghist);
+        DT_LAUNCH(k_hist, grid, kTPB, 0, s, keys, t->nbeg, t->ncnt, node0, cpn, chunk, 2, prefix, ghist);
         DT_LAUNCH(k_select, (int)nn, kTPB, 0, s, t->ncnt, node0, 2, ghist, prefix, rank, less, eql);
         DT_CHECK(cudaMemsetAsync(eqc, 0, nn * 4, s));
         DT_CHECK(cudaMemsetAsync(cur, 0, 2 * nn * 4, s));
         DT_LAUNCH(k_scatter<DP>, grid, kTPB, 0, s, src, isrc, dst, idst, keys, t->nbeg, t->ncnt,
-                  node0, cpn, prefix, eql, eqc, cur, dbad);
+                  node0, cpn, chunk, prefix, eql, eqc, cur, dbad);
         std::swap(src, dst);
         std::swap(isrc, idst);
     }
