@@ -186,6 +186,11 @@ __global__ void k_seed_proposal(const ProbDev* probs, const int32_t* blk_prob, i
 
 constexpr int kExpandProbs = 64;
 
+// Problems of at most this many (block, leaf) pairs get buffers for all of them
+// (64 MB) and run every traversal level without reading its size back: nine
+// read-backs of about 12 us are a tenth of a 10k-point search.
+constexpr int64_t kSmallPairs = (int64_t)1 << 21;
+
 template <int DP, int OP>
 __global__ void __launch_bounds__(256, 2) k_expand(const ProbDev* __restrict__ probs,
                                                 const int32_t* __restrict__ node_prob,
@@ -948,7 +953,40 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
         P.release(outp);
         return DTREE_OK;
     };
-    if (!arena) {
+    // a level's CTAs: no more than its frontier can use (four times the last
+    // level's, at most)
+    auto level_grid = [&](int64_t nf) { return (int)std::min<int64_t>(egrid, (nf + 255) / 256); };
+    // every (block, leaf) pair of the batch, which no level's frontier exceeds
+    int64_t all_pairs = 0;
+    for (int i = 0; i < np; ++i) all_pairs += (int64_t)pd[i].nblocks * hp[i].tr->nleaves;
+    if (!arena && all_pairs <= kSmallPairs) {
+        // a small problem: room for every pair, all levels without a read-back
+        int2 *F0, *F1;
+        int* lc;  // per level: the frontier's size
+        DT_TRY(P.get(&outp, all_pairs));
+        DT_TRY(P.get(&F0, all_pairs));
+        DT_TRY(P.get(&F1, all_pairs));
+        DT_TRY(P.get(&lc, steps + 1));
+        DT_CHECK(cudaMemsetAsync(bcount, 0, NB * sizeof(int), s));
+        DT_CHECK(cudaMemsetAsync(ctr + 4, 0, 4 * sizeof(int), s));
+        DT_CHECK(cudaMemsetAsync(lc, 0, (steps + 1) * sizeof(int), s));
+        DT_CHECK(cudaMemcpyAsync(F0, roots, np * sizeof(int2), cudaMemcpyDeviceToDevice, s));
+        DT_CHECK(cudaMemcpyAsync(lc, &np, sizeof(int), cudaMemcpyHostToDevice, s));
+        int64_t most = np;
+        for (int t = 0; t < steps; ++t, most = std::min(4 * most, all_pairs)) {
+            DT_TRY(launch_expand<DP>(OP, probs, node_prob, Bn, t & 1 ? F1 : F0, lc + t, t & 1 ? F0 : F1, lc + t + 1,
+                                     all_pairs, outp, ctr + 7, all_pairs, bcount, sl0, sn, slots, ctr + 4, dstats, np,
+                                     level_grid(most), s));
+        }
+        int hv[4];
+        DT_CHECK(cudaMemcpyAsync(hv, ctr + 4, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
+        DT_CHECK(cudaStreamSynchronize(s));
+        if (hv[0]) return DTREE_ERR_CUDA;  // cannot happen: the buffers hold every pair
+        P.release(lc);
+        P.release(F1);
+        P.release(F0);
+        DT_TRY(finish_csr(hv[3]));
+    } else if (!arena) {
         // Buffers sized level by level: a frontier pair has at most four child
         // pairs, so before each level the output frontier and the candidate
         // buffer get room for four times the current frontier (the frontier
@@ -988,7 +1026,7 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
             DT_CHECK(cudaMemsetAsync(nc[nx], 0, sizeof(int), s));
             DT_TRY(launch_expand<DP>(OP, probs, node_prob, Bn, F[cur], nc[cur], F[nx], nc[nx], fcap[nx],
                                      outp, ctr + 7, ocap, bcount, sl0, sn, slots, ctr + 4, dstats,
-                                     np, egrid, s));
+                                     np, level_grid(nf), s));
             int hv[4];
             DT_CHECK(cudaMemcpyAsync(hv, ctr + 4, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
             DT_CHECK(cudaStreamSynchronize(s));
