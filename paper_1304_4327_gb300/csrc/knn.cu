@@ -1089,12 +1089,30 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const bool wide = 2 * paired >= NQ && pairs >= 2 * sms;
+        // fewer items than SMs: each item's windows of 256 candidates are split
+        // over several CTAs, about two per SM in all, and the last one done
+        // merges their lists (4097 queries of 1M points, d = 16: 64 items; the
+        // pass 1.77 -> 0.72 ms)
+        a.slices = 1;
+        if (OP != OP_RANGE && !wide && NI < sms) {
+            const int64_t windows = (npairs / NB + 255) / 256;
+            int S = (int)std::min<int64_t>(std::min<int64_t>(2 * sms / NI, windows), 16);
+            if (S > 1) {
+                const size_t each = (size_t)NI * S * KC * kQB;
+                if (P.get(&a.slice_d, each) == DTREE_OK && P.get(&a.slice_i, each) == DTREE_OK &&
+                    P.get(&a.slice_done, NI) == DTREE_OK) {
+                    DT_CHECK(cudaMemsetAsync(a.slice_done, 0, NI * sizeof(int), s));
+                    a.slices = S;
+                }
+            }
+        }
+        const int ni_tc = NI * a.slices;
         if constexpr (OP == OP_RANGE)
-            DT_TRY(launch_range_tile<DP>(a, NI, derr, spin, s));
+            DT_TRY(launch_range_tile<DP>(a, ni_tc, derr, spin, s));
         else if constexpr (OP == OP_FAR)
-            DT_TRY(launch_far_tile<DP>(a, KC, NI, wide, derr, spin, s));
+            DT_TRY(launch_far_tile<DP>(a, KC, ni_tc, wide, derr, spin, s));
         else
-            DT_TRY(launch_tile_tc<DP>(a, fmt, KC, NI, wide, derr, spin, s));
+            DT_TRY(launch_tile_tc<DP>(a, fmt, KC, ni_tc, wide, derr, spin, s));
     } else {
         DT_TRY(launch_tile_cc<DP>(a, KC, MODE_MAIN, NI, s));
     }

@@ -231,6 +231,13 @@ struct TileArgs {
     void* fb_part;
     unsigned long long* stats;
     RangeOut range;    // (OP_RANGE)
+    // the tensor-core pass's slices per work item (1: one CTA per item), their
+    // lists ([item][slice][entry][query] keys, then as many positions) and, per
+    // item, how many slices are done
+    int slices;
+    float* slice_d;
+    int32_t* slice_i;
+    int* slice_done;
 };
 
 template <int DP>

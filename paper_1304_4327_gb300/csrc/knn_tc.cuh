@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
     __shared__ long long s_handoff[NB];  // diagnostics: when the planner handed each slot over
     __shared__ int2 amet[NACC];  // the tile in each accumulator: (table, columns), columns < 0 ends the block
     __shared__ uint32_t s_tmem;
-    __shared__ int s_item;
+    __shared__ int s_item, s_last;
     __shared__ ProbDev s_prob;
     __shared__ volatile int s_fail;
     __shared__ volatile float s_wmax[4 * NG], s_wmin[4 * NG];
@@ -456,7 +456,8 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
     const int grp_id = warp >> 2;  // an epilogue thread's group
     const int qt = tid & 127;  // query row of an epilogue thread
     const int half = QH == 2 ? grp_id : 0;  // and its half of the item's queries
-    const int nitems = a.nitems;
+    const int nslice = QH == 1 && OP != OP_RANGE ? a.slices : 1;
+    const int nitems = a.nitems * nslice;
     unsigned long long n_skip = 0, n_eval = 0, n_pp = 0, n_re = 0, n_ins = 0;
 
     if (tid == 0) {
@@ -498,12 +499,13 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
     for (;;) {
         if (tid == 0) {
             s_item = atomicAdd(a.work_ctr, 1);
-            if (s_item < nitems) s_prob = a.probs[a.blk_prob[a.items[s_item].x]];
+            if (s_item < nitems) s_prob = a.probs[a.blk_prob[a.items[s_item / nslice].x]];
         }
         __syncthreads();
         const int item = s_item;
         if (item >= nitems || s_fail) break;
-        const int2 wi = a.items[item];
+        const int slice = item % nslice;
+        const int2 wi = a.items[item / nslice];
         const int blk = wi.x, chunk = wi.y;  // global block, chunk of its queries
         const int64_t qnode = P.qblock0 + (blk - P.block0);
         // (work items are numbered by chunks of 128: with QH = 2 the even ones
@@ -611,14 +613,16 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                 }
                 tc::cp_async_commit();
             };
-            if (ntot > 0) fetch(0, 0);
+            // (a slice takes every nslice-th window)
+            const int64_t wstep = (int64_t)nslice * WIN, wfirst = (int64_t)slice * WIN;
+            if (wfirst < ntot) fetch(wfirst, 0);
             int wbuf = 0;
-            for (int64_t w0 = 0; w0 < ntot; w0 += WIN, wbuf ^= 1) {
+            for (int64_t w0 = wfirst; w0 < ntot; w0 += wstep, wbuf ^= 1) {
                 const int wn = (int)(ntot - w0 < WIN ? ntot - w0 : WIN);
                 long long t0 = TC_TIMED ? clock64() : 0;
                 tc::cp_async_wait_all();
                 __syncwarp();
-                if (w0 + WIN < ntot) fetch(w0 + WIN, wbuf ^ 1);
+                if (w0 + wstep < ntot) fetch(w0 + wstep, wbuf ^ 1);
                 // the block's bound from the epilogue warps' published values
                 // (two groups of one half each keep a list per query: their
                 // queries' bounds join; two groups of the same queries keep two
@@ -1175,7 +1179,39 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
             // the re-rank below reuses the merge buffers: group 0 has read them
             tc::named_sync(1, 256);
         }
-        if (LISTS && epi && (QH == 2 || grp_id == 0)) {
+        bool last = true;  // this slice finishes the item
+        if (LISTS && nslice > 1) {
+            // leave the lists in memory; the item's last slice merges them all
+            const int64_t base = (int64_t)(item / nslice) * nslice * KC * kQB;
+            if (epi && grp_id == 0) {
+#pragma unroll
+                for (int j = 0; j < KC; ++j) {
+                    a.slice_d[base + ((int64_t)slice * KC + j) * kQB + qt] = ld[j];
+                    a.slice_i[base + ((int64_t)slice * KC + j) * kQB + qt] = li[j];
+                }
+                __threadfence();
+            }
+            __syncthreads();
+            if (tid == 0) s_last = atomicAdd(&a.slice_done[item / nslice], 1) == nslice - 1;
+            __syncthreads();
+            last = s_last;
+            if (last && epi && grp_id == 0) {
+                __threadfence();
+                for (int o = 0; o < nslice; ++o) {
+                    if (o == slice) continue;
+#pragma unroll 1
+                    for (int j = 0; j < KC; ++j) {
+                        const float d = __ldcg(&a.slice_d[base + ((int64_t)o * KC + j) * kQB + qt]);
+                        const int i = __ldcg(&a.slice_i[base + ((int64_t)o * KC + j) * kQB + qt]);
+                        // (entries come in ascending order; all slices started
+                        // from the same list)
+                        if (!(d < ld[KC - 1])) break;
+                        if (!listed(li, i)) list_insert_key(ld, li, d, i);
+                    }
+                }
+            }
+        }
+        if (LISTS && last && epi && (QH == 2 || grp_id == 0)) {
             // ---- finish the work item
             long long tf0 = TC_TIMED ? clock64() : 0;
             const float ubk = fminf(Bd::ub(list_at(ld, kq - 1), qa, rad), qc);
