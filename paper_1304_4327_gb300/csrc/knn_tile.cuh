@@ -849,6 +849,7 @@ template <int DP, int KC, int OP = OP_NEAR>
 __global__ void __launch_bounds__(kQB) k_query_cap(const TileArgs a, float* qcap, int budget) {
     constexpr int NE = (KC + 31) / 32;      // list entries per lane
     constexpr int NT = (2 * DP + 31) / 32;  // box elements per lane
+    constexpr int LPR = DP / 4;             // lanes per point of a leaf
     const int item = blockIdx.x;
     if (item >= a.nitems) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -863,15 +864,8 @@ __global__ void __launch_bounds__(kQB) k_query_cap(const TileArgs a, float* qcap
         const int myq = P.qbeg[qnode] + wi.y * kQB + qi;
         const int64_t row = P.q0 + myq;
         const float* qp = P.qpts + (int64_t)myq * DP;
-        float q[DP];
-#pragma unroll
-        for (int j = 0; j < DP / 4; ++j) {
-            const float4 v = reinterpret_cast<const float4*>(qp)[j];
-            q[4 * j] = v.x;
-            q[4 * j + 1] = v.y;
-            q[4 * j + 2] = v.z;
-            q[4 * j + 3] = v.w;
-        }
+        // this lane's four coordinates of the query in the leaf evaluation
+        const float4 qv = reinterpret_cast<const float4*>(qp)[lane % LPR];
         float qd[NT];
 #pragma unroll
         for (int t = 0; t < NT; ++t) {
@@ -994,8 +988,26 @@ __global__ void __launch_bounds__(kQB) k_query_cap(const TileArgs a, float* qcap
                 int ti = entry_i(KC - 1);
                 for (int r0 = 0; r0 < rc; r0 += 32) {
                     const int r = rb + r0 + lane;
+                    // 32 points, LPR lanes each, in LPR steps: the group that
+                    // starts at lane g takes points g, g + 1, ..., so that lane l
+                    // ends up with point l's key, and a step's loads are whole
+                    // rows.  (A lane per point touched 32 lines with every load
+                    // and was bound by L1: seed and cap of 500k queries, d = 64,
+                    // 16 leaves 29.2 -> 23.7 ms; of 131k, d = 27 3.6 -> 2.7; d = 16
+                    // 11.0 -> 10.8.)
+                    float key = 0.f;
+#pragma unroll
+                    for (int s = 0; s < LPR; ++s) {
+                        const int row = min(r0 + lane - lane % LPR + s, rc - 1);
+                        const float4 v = reinterpret_cast<const float4*>(P.rpts + (int64_t)(rb + row) * DP)[lane % LPR];
+                        const float t0 = qv.x - v.x, t1 = qv.y - v.y, t2 = qv.z - v.z, t3 = qv.w - v.w;
+                        float f = fmaf(t3, t3, fmaf(t2, t2, fmaf(t1, t1, t0 * t0)));
+#pragma unroll
+                        for (int off = LPR / 2; off > 0; off >>= 1) f += __shfl_xor_sync(0xffffffffu, f, off);
+                        key = lane % LPR == s ? f : key;
+                    }
                     float d = INFINITY;
-                    if (r0 + lane < rc && !(mono && r == myq)) d = (OP == OP_FAR ? -1.f : 1.f) * approx_d2<DP>(q, P.rpts + (int64_t)r * DP);
+                    if (r0 + lane < rc && !(mono && r == myq)) d = (OP == OP_FAR ? -1.f : 1.f) * key;
                     uint32_t m = __ballot_sync(0xffffffffu, d < INFINITY && key_less(d, r, td, ti));
                     while (m) {
                         const int src = __ffs(m) - 1;
