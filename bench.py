@@ -742,8 +742,9 @@ METRIC_RANGE = "exact range-search queries/s (oracle-identical)"
 
 def run_kfn(args, rank, world, local):
     """--op kfn: one step = build the reference tree + build the query tree +
-    dtree_kfn (one warp per query: the single-tree depth-first search with the
-    inverted Score and BaseCase, float32 keys, float64 re-rank and fallback).
+    dtree_kfn (the block search with negated distances at this size; small
+    problems take one warp per query: the single-tree depth-first search with
+    the inverted Score and BaseCase, float32 keys, float64 re-rank and fallback).
     --op range: the same with dtree_range (count, scan, fill) over --range."""
     from oracle import kfn as okfn
     from oracle import rangesearch as orange
@@ -891,7 +892,9 @@ def run_kfn(args, rank, world, local):
                            + ("dtree_range (count, scan, fill)" if is_range else "dtree_kfn"),
                    "l2": "inputs (320 MB) larger than the 129 MB L2; no flush",
                    "parallelism": f"{world} GPU(s), one query shard each, reference replicated"},
-        "roofline": {"bound": "alu",
+        # large problems in d > 8 run the block search: tensor-core tiles
+        "roofline": roofline("bf16", d, pairs, ns, sms, None) if s0["query_blocks"] > 0 else
+                    {"bound": "alu",
                      "kernel": ("k_range count launch" if is_range else "k_kfn")
                      + " (one warp per query, float32 keys)",
                      "achieved": achieved, "peak": peak, "unit": "TFLOP/s",

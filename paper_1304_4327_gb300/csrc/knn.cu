@@ -19,14 +19,18 @@
 //                is scored with the box distance d_min and pruned when
 //                d_min > B(N_q); surviving (block, reference leaf) pairs form
 //                each block's candidate list;
-//   4. basecase  one CTA per block streams its candidate leaves nearest-first,
-//                keeps each query's candidate list, tightens the block's B as
-//                the lists improve and skips leaves whose d_min exceeds it,
-//                then re-ranks the candidates near the k-th distance in float64
-//                and writes the outputs;
+//   4. basecase  one CTA per work item (128 or 256 queries of a block; several
+//                per item where items are few) streams its candidate leaves
+//                nearest-first, keeps each query's candidate list, tightens the
+//                item's B as the lists improve and skips leaves whose d_min
+//                exceeds it, then re-ranks the candidates near the k-th
+//                distance exactly and writes the outputs;
 //   5. fallback  a query whose band of near-k-th candidates overflowed its
 //                list is recomputed exactly in float64 over its block's
 //                candidate leaves (one CTA per such query).
+//
+// The same passes serve k-furthest neighbours (OP_FAR) and range searches
+// (OP_RANGE) of large problems.
 #include <algorithm>
 #include <cmath>
 #include <vector>

@@ -170,6 +170,7 @@ extern "C" int dtree_range_count(const dtree_t* query, const dtree_t* ref, doubl
         st->leaf_pairs_evaluated = (int64_t)h[1] + tst.leaf_pairs_evaluated;
         st->node_pairs_pruned = (int64_t)h[2] + tst.node_pairs_pruned;
         st->rerank_candidates = (int64_t)h[3] + tst.rerank_candidates;
+        st->query_blocks = tst.query_blocks;
         float ms = 0.f;
         if (timed && cudaEventElapsedTime(&ms, ev[0], ev[1]) == cudaSuccess) st->ns_basecase = (int64_t)(ms * 1e6);
         st->kernel_launches = g_launches.load() - launches0;
