@@ -214,9 +214,9 @@ __global__ void k_f32_to_f16(const float* in, int64_t n, __half* out) {
 }
 
 // Softmax cross-entropy per row against a target distribution T (rows sum to
-// 1): loss += -sum_c T[r, c] log p[r, c]; dZ = (p - T) / B (FP32 and FP16).
+// 1): row_loss[r] = -sum_c T[r, c] log p[r, c]; dZ = (p - T) / B (FP32 and FP16).
 __global__ void __launch_bounds__(256) k_softmax_xent(const float* Z, const float* T, int B, int Cc,
-                                                      float* dZ, __half* dZh, int ldh, float* loss) {
+                                                      float* dZ, __half* dZh, int ldh, float* row_loss) {
     const int r = blockIdx.x;
     const float* z = Z + (int64_t)r * Cc;
     const float* t = T + (int64_t)r * Cc;
@@ -254,8 +254,26 @@ __global__ void __launch_bounds__(256) k_softmax_xent(const float* Z, const floa
     if (threadIdx.x == 0) {
         float s = 0.f;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        atomicAdd(loss, s / (float)B);
+        row_loss[r] = s;
     }
+}
+
+constexpr int kLossThreads = 256;
+
+// loss = the mean of the rows' losses, summed in float64 in an order that
+// depends on B alone.  (float32 atomics in the order the rows' CTAs ended gave
+// another loss in every call and rounded at each of the B additions: 4,096
+// equal rows came out up to 6e-5 of their value off.)
+__global__ void __launch_bounds__(kLossThreads) k_mean_loss(const float* row_loss, int B, float* loss) {
+    __shared__ double part[kLossThreads];
+    double s = 0.0;
+    for (int r = threadIdx.x; r < B; r += kLossThreads) s += (double)row_loss[r];
+    part[threadIdx.x] = s;
+    for (int o = kLossThreads / 2; o > 0; o >>= 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < o) part[threadIdx.x] += part[threadIdx.x + o];
+    }
+    if (threadIdx.x == 0) *loss = (float)(part[0] / B);
 }
 
 // g[r, c] *= (h[r, c] > 0) (the ReLU's derivative), also writing an FP16 copy.
@@ -470,7 +488,7 @@ struct Work {
     DevBuf<__half> X, XT, H1h, H1T, H2h, H2T, dZh, dZT, dH2h, dH2T, dH1h, dH1T, W3T, W2T;
     DevBuf<float> H1, H2, Z, dZ, dH2, dH1, g[6], part;
     int Bp = 0, Cp = 0;  // rows and classes rounded up to 16-byte FP16 rows
-    DevBuf<float> loss;
+    DevBuf<float> loss, row_loss;
     DevBuf<int> err;
     int alloc(const dtree_model& md, int B_, cudaStream_t s, bool train) {
         B = B_;
@@ -489,6 +507,7 @@ struct Work {
         MT(XT.get((int64_t)dp * Bp, s));
         MT(H1T.get((int64_t)H * Bp, s));
         MT(H2T.get((int64_t)H * Bp, s));
+        MT(row_loss.get(B, s));
         MT(dZ.get((int64_t)B * C, s));
         MT(dZh.get((int64_t)B * Cp, s));
         MT(dZT.get((int64_t)C * Bp, s));
@@ -522,10 +541,10 @@ int forward(const dtree_model& md, Work& w, int B, cudaStream_t s) {
 // Loss against the targets T (B x C) and every parameter's gradient in w.g.
 int backward(const dtree_model& md, Work& w, int B, const float* T, cudaStream_t s) {
     const int H = md.H, C = md.C, dp = md.dpad;
-    DT_CHECK(cudaMemsetAsync(w.loss.p, 0, sizeof(float), s));
     const int Bp = w.Bp, Cp = w.Cp;
     float* part = w.part.p;
-    DT_LAUNCH(k_softmax_xent, B, 256, 0, s, w.Z.p, T, B, C, w.dZ.p, w.dZh.p, Cp, w.loss.p);
+    DT_LAUNCH(k_softmax_xent, B, 256, 0, s, w.Z.p, T, B, C, w.dZ.p, w.dZh.p, Cp, w.row_loss.p);
+    DT_LAUNCH(k_mean_loss, 1, kLossThreads, 0, s, w.row_loss.p, B, w.loss.p);
     // layer 3: dW3 = dZ^T H2, db3 = colsum dZ, dH2 = dZ W3
     MT(transpose(s, w.dZh.p, Cp, B, C, w.dZT.p, Bp));
     MT(transpose(s, w.H2h.p, H, B, H, w.H2T.p, Bp));
