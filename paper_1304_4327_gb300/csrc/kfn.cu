@@ -19,7 +19,8 @@ int kfn_launch(int dp, const KfnArgs& a, int kc, bool exact, int grid, cudaStrea
 }
 
 // Whether the block search serves a problem: enough work that its passes pay
-// (d > 8, 4096 queries and 1e9 pairs), and extents that its float32 bounds cover.
+// (d > 8, 4096 queries and 1e9 pairs), lists of at most 64 that hold the 14
+// entries beyond k its band wants, and extents that its float32 bounds cover.
 //
 // A walk per query visits few leaves where the box bound prunes well (d <= 8:
 // 1M x 100k uniform points in d = 3 3.6 ms against 5.4; 1M x 30k in d = 8 5.9
@@ -28,13 +29,16 @@ int kfn_launch(int dp, const KfnArgs& a, int kc, bool exact, int grid, cudaStrea
 // tensor cores do the distances: 1M x 20k points of the mixture, d = 12, 16,
 // 32: 26.5 -> 11.3, 40.8 -> 11.6, 195 -> 19.6 ms; 50k x 20k, d = 16: 5.5 ->
 // 3.9; 300k x 5k, d = 10 and 20: 5.4 -> 4.9, 14.7 -> 6.5.
-int kfn_tiles_fit(const dtree_t* tq, const dtree_t* tr, cudaStream_t s, bool* fit) {
+// A band that overflows costs the walk on top: 300k x 50k Gaussian points in d =
+// 16, k = 63 took 3608 ms by tiles (nearly all bands overflow a list of 64) and
+// take 276 by walks; k = 50 on 20k queries 8.5 by tiles, 93 by walks.
+int kfn_tiles_fit(const dtree_t* tq, const dtree_t* tr, int k, cudaStream_t s, bool* fit) {
     *fit = false;
     int major = 0, minor = 0;
     cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, tr->device);
     cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, tr->device);
     if (major != 10 || minor != 3) return DTREE_OK;  // the tiles are tcgen05 code
-    if (tr->dp < 16 || tq->n < 4096 || (double)tq->n * (double)tr->n < 1e9) return DTREE_OK;
+    if (tr->dp < 16 || k + 14 > 64 || tq->n < 4096 || (double)tq->n * (double)tr->n < 1e9) return DTREE_OK;
     double radius;
     return extents_fit(tq, tr, s, fit, &radius);
 }
@@ -66,7 +70,7 @@ extern "C" int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, in
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t launches0 = g_launches.load();
     bool tiles = false;
-    int rt = kfn_tiles_fit(tq, ref, s, &tiles);
+    int rt = kfn_tiles_fit(tq, ref, k, s, &tiles);
     if (rt != DTREE_OK) return rt;
     if (tiles) {
         rt = kfn_by_tiles(tq, ref, mono, k, out_idx, out_dist, s, st);
@@ -100,7 +104,6 @@ extern "C" int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, in
     a.stats = reinterpret_cast<unsigned long long*>(scratch);
     a.fb_count = reinterpret_cast<int*>(scratch + 32);
     a.fb_list = reinterpret_cast<int*>(scratch + 48);
-    a.fb_stride = 1;
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaEvent_t ev[2] = {};
@@ -123,6 +126,9 @@ extern "C" int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, in
             break;
         }
         if (nfb > 0) {
+            a.in_list = a.fb_list;
+            a.in_count = a.fb_count;
+            a.in_stride = 1;
             const int g2 = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)nfb + 3) / 4, (int64_t)sms * 16));
             rc = kfn_launch(ref->dp, a, kc, true, g2, s);
             if (rc != DTREE_OK) break;

@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(128) k_kfn(const KfnArgs a) {
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t count = EXACT ? (int64_t)*a.fb_count : a.nq;
+    const int64_t count = a.in_list ? (int64_t)*a.in_count : a.nq;
     const int k = a.k;
     const bool mono = a.mono != 0;
     // squared-distance rounding: d_max up, list keys down (float keys only)
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(128) k_kfn(const KfnArgs a) {
     unsigned long long n_pts = 0, n_leaves = 0, n_pruned = 0;
 
     for (int64_t wi = w0; wi < count; wi += nw) {
-        const int64_t qpos = EXACT ? (int64_t)a.fb_list[wi * a.fb_stride] : wi;
+        const int64_t qpos = a.in_list ? (int64_t)a.in_list[wi * a.in_stride] : wi;
         const float* qp = a.qpts + qpos * DP;
         float q[DP];
 #pragma unroll

@@ -1133,7 +1133,11 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
     int nfb2 = 0;
     if constexpr (OP == OP_FAR) {
         if (nfb > 0) {
-            // the float64 search, a warp per query
+            // the search of kfn.cuh, a warp per query: float32 keys, then
+            // float64 for those whose float32 band overflows too (whose walks
+            // are some ten times as long: 20k queries at the centre of a sphere
+            // of 50k points in d = 16, all of which overflow, took 220 ms with
+            // float64 alone and take 16.8 so; by walks from the start 14.2)
             KfnArgs ka{};
             ka.qpts = hp[0].tq->pts;
             ka.qidx = hp[0].tq->idx;
@@ -1148,15 +1152,25 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
             ka.mono = hp[0].mono ? 1 : 0;
             ka.out_idx = hp[0].out_idx;
             ka.out_dist = hp[0].out_dist;
-            ka.fb_list = reinterpret_cast<int*>(fbq_list);
-            ka.fb_stride = 4;
-            ka.fb_count = ctr + 3;
+            ka.in_list = reinterpret_cast<int*>(fbq_list);
+            ka.in_count = ctr + 3;
+            ka.in_stride = 4;
+            ka.fb_list = reinterpret_cast<int*>(fbq2_list);
+            ka.fb_count = ctr + 8;
             int dev = 0, sms = 0;
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            DT_TRY(launch_kfn<DP>(ka, kmax + 1 <= 16 ? 16 : kmax + 1 <= 32 ? 32 : 64, true,
-                                  (int)std::max(1, std::min((nfb + 3) / 4, sms * 16)), s));
-            nfb2 = nfb;
+            const int kc = kmax + 1 <= 16 ? 16 : kmax + 1 <= 32 ? 32 : 64;
+            auto grid = [&](int n) { return (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)n + 3) / 4, (int64_t)sms * 16)); };
+            DT_TRY(launch_kfn<DP>(ka, kc, false, grid(nfb), s));
+            DT_CHECK(cudaMemcpyAsync(&nfb2, ctr + 8, sizeof(int), cudaMemcpyDeviceToHost, s));
+            DT_CHECK(cudaStreamSynchronize(s));
+            if (nfb2 > 0) {
+                ka.in_list = ka.fb_list;
+                ka.in_count = ka.fb_count;
+                ka.in_stride = 1;
+                DT_TRY(launch_kfn<DP>(ka, kc, true, grid(nfb2), s));
+            }
         }
     } else if (OP == OP_NEAR && nfb > 0) {
         // few such queries: each one's candidates are split over up to 64

@@ -190,8 +190,10 @@ struct KfnArgs {
     int mono;
     int64_t* out_idx;   // (rows in the caller's query order) x k
     float* out_dist;
-    int* fb_list;       // float pass: appends queries whose band overflowed; double pass: its input,
-    int fb_stride;      //   every fb_stride-th entry
+    const int* in_list;   // the queries to serve: every in_stride-th entry, *in_count of them
+    const int* in_count;  //   (null: all nq)
+    int in_stride;
+    int* fb_list;         // float pass: appends the queries whose band overflowed
     int* fb_count;
     unsigned long long* stats;  // [0] point distances, [1] leaves visited, [2] nodes pruned
 };
