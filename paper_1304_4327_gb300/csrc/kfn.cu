@@ -8,13 +8,13 @@
 namespace dt {
 namespace {
 
-int kfn_launch(int dp, const KfnArgs& a, int kc, bool exact, int grid, cudaStream_t s) {
+int kfn_launch(int dp, const KfnArgs& a, int kc, KfnPass pass, int grid, cudaStream_t s) {
     switch (dp) {
-        case 4: return launch_kfn<4>(a, kc, exact, grid, s);
-        case 8: return launch_kfn<8>(a, kc, exact, grid, s);
-        case 16: return launch_kfn<16>(a, kc, exact, grid, s);
-        case 32: return launch_kfn<32>(a, kc, exact, grid, s);
-        default: return launch_kfn<64>(a, kc, exact, grid, s);
+        case 4: return launch_kfn<4>(a, kc, pass, grid, s);
+        case 8: return launch_kfn<8>(a, kc, pass, grid, s);
+        case 16: return launch_kfn<16>(a, kc, pass, grid, s);
+        case 32: return launch_kfn<32>(a, kc, pass, grid, s);
+        default: return launch_kfn<64>(a, kc, pass, grid, s);
     }
 }
 
@@ -118,7 +118,7 @@ extern "C" int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, in
         // one warp per query, four per CTA; a grid of whole waves of CTAs
         const int64_t want = (nq + 3) / 4;
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * 16));
-        rc = kfn_launch(ref->dp, a, kc, false, grid, s);
+        rc = kfn_launch(ref->dp, a, kc, KFN_ALL, grid, s);
         if (rc != DTREE_OK) break;
         if (cudaMemcpyAsync(&nfb, a.fb_count, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) {
@@ -128,9 +128,8 @@ extern "C" int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, in
         if (nfb > 0) {
             a.in_list = a.fb_list;
             a.in_count = a.fb_count;
-            a.in_stride = 1;
             const int g2 = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)nfb + 3) / 4, (int64_t)sms * 16));
-            rc = kfn_launch(ref->dp, a, kc, true, g2, s);
+            rc = kfn_launch(ref->dp, a, kc, KFN_EXACT, g2, s);
             if (rc != DTREE_OK) break;
         }
         if (timed) cudaEventRecord(ev[1], s);

@@ -48,15 +48,18 @@ namespace dt {
 
 constexpr int kKfnEmpty = 0x7fffffff;  // the index of an empty list entry
 
-template <int DP, int KC, typename T>
+// (the pass is a template argument: with a list read where all queries are
+// served, too, the float kernels took up to eight registers more and 5% longer)
+template <int DP, int KC, int PASS>
 __global__ void __launch_bounds__(128) k_kfn(const KfnArgs a) {
-    constexpr bool EXACT = std::is_same<T, double>::value;
+    constexpr bool EXACT = PASS == KFN_EXACT;
+    using T = std::conditional_t<EXACT, double, float>;
     constexpr int NE = (KC + 31) / 32;      // list entries per lane
     constexpr int NT = (2 * DP + 31) / 32;  // box elements per lane
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t count = a.in_list ? (int64_t)*a.in_count : a.nq;
+    const int64_t count = PASS == KFN_ALL ? a.nq : (int64_t)*a.in_count;
     const int k = a.k;
     const bool mono = a.mono != 0;
     // squared-distance rounding: d_max up, list keys down (float keys only)
@@ -65,7 +68,7 @@ __global__ void __launch_bounds__(128) k_kfn(const KfnArgs a) {
     unsigned long long n_pts = 0, n_leaves = 0, n_pruned = 0;
 
     for (int64_t wi = w0; wi < count; wi += nw) {
-        const int64_t qpos = a.in_list ? (int64_t)a.in_list[wi * a.in_stride] : wi;
+        const int64_t qpos = PASS == KFN_ALL ? wi : (int64_t)a.in_list[wi * PASS];
         const float* qp = a.qpts + qpos * DP;
         float q[DP];
 #pragma unroll
@@ -307,26 +310,23 @@ __global__ void __launch_bounds__(128) k_kfn(const KfnArgs a) {
     }
 }
 
+template <int DP, int KC>
+int launch_kfn_as(const KfnArgs& a, KfnPass pass, int grid, cudaStream_t s) {
+    auto kern = pass == KFN_EXACT ? k_kfn<DP, KC, KFN_EXACT> : k_kfn<DP, KC, KFN_ALL>;
+    if constexpr (DP >= 16)  // (only the block search lists queries for the float pass)
+        if (pass == KFN_LIST) kern = k_kfn<DP, KC, KFN_LIST>;
+    DT_LAUNCH(kern, grid, 128, 0, s, a);
+    return DTREE_OK;
+}
+
 template <int DP>
-int launch_kfn(const KfnArgs& a, int kc, bool exact, int grid, cudaStream_t s) {
-#define DT_KFN_CASE(KCV)                                                        \
-    case KCV:                                                                   \
-        if (exact) {                                                            \
-            auto kern = k_kfn<DP, KCV, double>;                                 \
-            DT_LAUNCH(kern, grid, 128, 0, s, a);                                \
-        } else {                                                                \
-            auto kern = k_kfn<DP, KCV, float>;                                  \
-            DT_LAUNCH(kern, grid, 128, 0, s, a);                                \
-        }                                                                       \
-        return DTREE_OK;
+int launch_kfn(const KfnArgs& a, int kc, KfnPass pass, int grid, cudaStream_t s) {
     switch (kc) {
-        DT_KFN_CASE(16)
-        DT_KFN_CASE(32)
-        DT_KFN_CASE(64)
-        default:
-            return DTREE_ERR_UNSUPPORTED;
+        case 16: return launch_kfn_as<DP, 16>(a, pass, grid, s);
+        case 32: return launch_kfn_as<DP, 32>(a, pass, grid, s);
+        case 64: return launch_kfn_as<DP, 64>(a, pass, grid, s);
+        default: return DTREE_ERR_UNSUPPORTED;
     }
-#undef DT_KFN_CASE
 }
 
 }  // namespace dt

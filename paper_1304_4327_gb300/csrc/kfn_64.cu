@@ -2,5 +2,5 @@
 #include "kfn.cuh"
 
 namespace dt {
-template int launch_kfn<64>(const KfnArgs&, int, bool, int, cudaStream_t);
+template int launch_kfn<64>(const KfnArgs&, int, KfnPass, int, cudaStream_t);
 }  // namespace dt

@@ -1154,7 +1154,6 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
             ka.out_dist = hp[0].out_dist;
             ka.in_list = reinterpret_cast<int*>(fbq_list);
             ka.in_count = ctr + 3;
-            ka.in_stride = 4;
             ka.fb_list = reinterpret_cast<int*>(fbq2_list);
             ka.fb_count = ctr + 8;
             int dev = 0, sms = 0;
@@ -1162,14 +1161,13 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             const int kc = kmax + 1 <= 16 ? 16 : kmax + 1 <= 32 ? 32 : 64;
             auto grid = [&](int n) { return (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)n + 3) / 4, (int64_t)sms * 16)); };
-            DT_TRY(launch_kfn<DP>(ka, kc, false, grid(nfb), s));
+            DT_TRY(launch_kfn<DP>(ka, kc, KFN_LIST, grid(nfb), s));
             DT_CHECK(cudaMemcpyAsync(&nfb2, ctr + 8, sizeof(int), cudaMemcpyDeviceToHost, s));
             DT_CHECK(cudaStreamSynchronize(s));
             if (nfb2 > 0) {
                 ka.in_list = ka.fb_list;
                 ka.in_count = ka.fb_count;
-                ka.in_stride = 1;
-                DT_TRY(launch_kfn<DP>(ka, kc, true, grid(nfb2), s));
+                DT_TRY(launch_kfn<DP>(ka, kc, KFN_EXACT, grid(nfb2), s));
             }
         }
     } else if (OP == OP_NEAR && nfb > 0) {

@@ -190,9 +190,8 @@ struct KfnArgs {
     int mono;
     int64_t* out_idx;   // (rows in the caller's query order) x k
     float* out_dist;
-    const int* in_list;   // the queries to serve: every in_stride-th entry, *in_count of them
-    const int* in_count;  //   (null: all nq)
-    int in_stride;
+    const int* in_list;   // a list pass: the queries to serve, *in_count of them
+    const int* in_count;
     int* fb_list;         // float pass: appends the queries whose band overflowed
     int* fb_count;
     unsigned long long* stats;  // [0] point distances, [1] leaves visited, [2] nodes pruned
@@ -268,9 +267,12 @@ template <int DP>
 int launch_far_cap(const TileArgs& a, int kc, int budget, float* qcap, cudaStream_t s);
 template <int DP>
 int launch_far_tile(const TileArgs& a, int kc, int items, bool wide, int* err, int spin, cudaStream_t s);
-// ... and the float64 search of the queries listed in a.fb_list (kfn.cuh).
+// ... and the one-warp-per-query search (kfn.cuh): of all queries with float32
+// keys, of the first words of the 16-byte entries of a.in_list with float32 keys,
+// or of its words in float64.
+enum KfnPass { KFN_ALL = 0, KFN_LIST = 4, KFN_EXACT = 1 };  // (words per entry)
 template <int DP>
-int launch_kfn(const KfnArgs& a, int kc, bool exact, int grid, cudaStream_t s);
+int launch_kfn(const KfnArgs& a, int kc, KfnPass pass, int grid, cudaStream_t s);
 
 // The range search's tensor-core pass (BF16).
 template <int DP>
