@@ -18,9 +18,10 @@ int kfn_launch(int dp, const KfnArgs& a, int kc, KfnPass pass, int grid, cudaStr
     }
 }
 
-// Whether the block search serves a problem: enough work that its passes pay
-// (d > 8, 4096 queries and 1e9 pairs), lists of at most 64 that hold the 14
-// entries beyond k its band wants, and extents that its float32 bounds cover.
+// Whether the block search may serve a problem: enough work that its passes pay
+// (d > 8, 4096 queries and 1e9 pairs) and lists of at most 64 that hold the 14
+// entries beyond k its band wants.  A look at the points then decides
+// (probe.cuh: their extents, and what a walk per query would visit).
 //
 // A walk per query visits few leaves where the box bound prunes well (d <= 8:
 // 1M x 100k uniform points in d = 3 3.6 ms against 5.4; 1M x 30k in d = 8 5.9
@@ -32,15 +33,22 @@ int kfn_launch(int dp, const KfnArgs& a, int kc, KfnPass pass, int grid, cudaStr
 // A band that overflows costs the walk on top: 300k x 50k Gaussian points in d =
 // 16, k = 63 took 3608 ms by tiles (nearly all bands overflow a list of 64) and
 // take 276 by walks; k = 50 on 20k queries 8.5 by tiles, 93 by walks.
-int kfn_tiles_fit(const dtree_t* tq, const dtree_t* tr, int k, cudaStream_t s, bool* fit) {
-    *fit = false;
+bool kfn_tiles_fit(const dtree_t* tq, const dtree_t* tr, int k) {
+    if (tr->dp < 16 || k + 14 > 64 || tq->n < 4096 || (double)tq->n * (double)tr->n < 1e9) return false;
     int major = 0, minor = 0;
     cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, tr->device);
     cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, tr->device);
-    if (major != 10 || minor != 3) return DTREE_OK;  // the tiles are tcgen05 code
-    if (tr->dp < 16 || k + 14 > 64 || tq->n < 4096 || (double)tq->n * (double)tr->n < 1e9) return DTREE_OK;
-    double radius;
-    return extents_fit(tq, tr, s, fit, &radius);
+    return major == 10 && minor == 3;  // the tiles are tcgen05 code
+}
+
+int kfn_look(const dtree_t* tq, const dtree_t* tr, int k, ProbeOut* out, cudaStream_t s) {
+    ProbeArgs a = probe_args(tq, tr, out);
+    a.k = k;
+    switch (tr->dp) {
+        case 16: return launch_probe_far<16>(a, s);
+        case 32: return launch_probe_far<32>(a, s);
+        default: return launch_probe_far<64>(a, s);
+    }
 }
 
 }  // namespace
@@ -69,24 +77,13 @@ extern "C" int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, in
     const int kc = k + 1 <= 16 ? 16 : k + 1 <= 32 ? 32 : 64;
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t launches0 = g_launches.load();
-    bool tiles = false;
-    int rt = kfn_tiles_fit(tq, ref, k, s, &tiles);
-    if (rt != DTREE_OK) return rt;
-    if (tiles) {
-        rt = kfn_by_tiles(tq, ref, mono, k, out_idx, out_dist, s, st);
-        if (rt == DTREE_OK && st) st->point_pairs += st->seed_point_pairs;
-        if (rt == DTREE_OK) return rt;
-        // (its operand rows or candidate pairs may not fit where the search
-        // below, which needs 4 bytes a query, does)
-        if (rt != DTREE_ERR_OOM) return rt;
-        if (st) memset(st, 0, sizeof(*st));
-    }
-
-    // scratch: three counters, the fallback count, and the fallback list
+    // scratch: three counters, the fallback count, the look's result, and the
+    // fallback list
     unsigned char* scratch = nullptr;
-    const size_t bytes = 32 + 16 + (size_t)nq * sizeof(int);
-    DT_CHECK(cudaMallocAsync((void**)&scratch, bytes, s));
+    constexpr size_t o_count = 32, o_look = 36, o_list = (o_look + sizeof(ProbeOut) + 15) & ~(size_t)15;
+    DT_CHECK(cudaMallocAsync((void**)&scratch, o_list + (size_t)nq * sizeof(int), s));
     g_allocs.fetch_add(1, std::memory_order_relaxed);
+    ProbeOut* look = reinterpret_cast<ProbeOut*>(scratch + o_look);
     KfnArgs a{};
     a.qpts = tq->pts;
     a.qidx = tq->idx;
@@ -102,28 +99,42 @@ extern "C" int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, in
     a.out_idx = out_idx;
     a.out_dist = out_dist;
     a.stats = reinterpret_cast<unsigned long long*>(scratch);
-    a.fb_count = reinterpret_cast<int*>(scratch + 32);
-    a.fb_list = reinterpret_cast<int*>(scratch + 48);
+    a.fb_count = reinterpret_cast<int*>(scratch + o_count);
+    a.fb_list = reinterpret_cast<int*>(scratch + o_list);
+    bool ask = kfn_tiles_fit(tq, ref, k);
+    a.gate = ask ? &look->gate : nullptr;
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaEvent_t ev[2] = {};
     const bool timed = st && cudaEventCreate(&ev[0]) == cudaSuccess && cudaEventCreate(&ev[1]) == cudaSuccess;
     cudaGetLastError();
     int rc = DTREE_OK;
-    int nfb = 0;
+    int hv[2] = {0, 0};  // the fallback count, and whether the block search serves the call
+    int& nfb = hv[0];
     unsigned long long cnt[3] = {0, 0, 0};
-    do {
-        if (cudaMemsetAsync(scratch, 0, 48, s) != cudaSuccess) { rc = cuda_status(cudaGetLastError()); break; }
+    bool tiles = false;
+    for (;; ask = false, a.gate = nullptr) {
+        if (cudaMemsetAsync(scratch, 0, o_look + 8, s) != cudaSuccess) { rc = cuda_status(cudaGetLastError()); break; }
         if (timed) cudaEventRecord(ev[0], s);
+        if (ask && (rc = kfn_look(tq, ref, k, look, s)) != DTREE_OK) break;
         // one warp per query, four per CTA; a grid of whole waves of CTAs
         const int64_t want = (nq + 3) / 4;
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * 16));
         rc = kfn_launch(ref->dp, a, kc, KFN_ALL, grid, s);
         if (rc != DTREE_OK) break;
-        if (cudaMemcpyAsync(&nfb, a.fb_count, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        if (cudaMemcpyAsync(hv, a.fb_count, sizeof(hv), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) {
             rc = cuda_status(cudaGetLastError());
             break;
+        }
+        if (ask && hv[1]) {
+            rc = kfn_by_tiles(tq, ref, mono, k, out_idx, out_dist, s, st);
+            tiles = rc == DTREE_OK;
+            // (its operand rows or candidate pairs may not fit where the walks,
+            // which need 4 bytes a query, do)
+            if (rc != DTREE_ERR_OOM) break;
+            if (st) memset(st, 0, sizeof(*st));
+            continue;
         }
         if (nfb > 0) {
             a.in_list = a.fb_list;
@@ -138,10 +149,14 @@ extern "C" int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, in
             break;
         }
         if (cudaStreamSynchronize(s) != cudaSuccess) rc = cuda_status(cudaGetLastError());
-    } while (false);
+        break;
+    }
     cudaFreeAsync(scratch, s);
     if (rc == DTREE_OK && cudaStreamSynchronize(s) != cudaSuccess) rc = cuda_status(cudaGetLastError());
-    if (st && rc == DTREE_OK) {
+    if (st && tiles) {
+        st->point_pairs += st->seed_point_pairs;
+        st->kernel_launches = g_launches.load() - launches0;
+    } else if (st && rc == DTREE_OK) {
         st->point_pairs = (int64_t)cnt[0];
         st->leaf_pairs_evaluated = (int64_t)cnt[1];
         st->node_pairs_pruned = (int64_t)cnt[2];

@@ -10,8 +10,8 @@
 // ascending).
 //
 // Large problems in d > 8 go through the block search of knn.cu with every
-// distance negated (kfn.cu's kfn_tiles_fit says which); this file's kernels
-// serve the others, and the queries whose band overflowed there.
+// distance negated (kfn.cu's kfn_tiles_fit and probe.cuh say which); this file's
+// kernels serve the others, and the queries whose band overflowed there.
 //
 // One warp serves one query (a query node of one point, so the traversal is
 // Algorithm 1's depth-first recursion on the reference tree alone):
@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(128) k_kfn(const KfnArgs a) {
     using T = std::conditional_t<EXACT, double, float>;
     constexpr int NE = (KC + 31) / 32;      // list entries per lane
     constexpr int NT = (2 * DP + 31) / 32;  // box elements per lane
+    if (PASS == KFN_ALL && a.gate && *a.gate) return;  // (set by an earlier kernel)
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;

@@ -195,6 +195,7 @@ struct KfnArgs {
     int* fb_list;         // float pass: appends the queries whose band overflowed
     int* fb_count;
     unsigned long long* stats;  // [0] point distances, [1] leaves visited, [2] nodes pruned
+    const int* gate;      // (all queries) set on the device: the block search serves them; or null
 };
 
 struct TileArgs {
@@ -283,6 +284,56 @@ int launch_range_tile(const TileArgs& a, int items, int* err, int spin, cudaStre
 int range_by_tiles(const dtree_t* tq, const dtree_t* tr, bool mono, const RangeOut& r, cudaStream_t s,
                    dtree_stats* st);
 
+// A look at a problem before it is searched (probe.cuh), made on the device: the
+// walk that follows it on the stream returns at once where gate is set, and the
+// host, which waits for the walk anyway, then runs the block search.
+constexpr int kProbeQueries = 64, kProbeLeaves = 1024;
+
+struct ProbeOut {
+    int gate;  // 1: the block search should serve the problem (zero before the look)
+    int done;  // CTAs that have counted (zero before the look)
+    int kept[kProbeQueries];  // per sampled query: the sampled leaves a walk would visit
+    int near[kProbeQueries];  // and the evaluated points that the tiles would settle exactly
+};
+
+struct ProbeArgs {
+    const float* qpts;
+    int64_t nq;
+    const float* rpts;
+    const int32_t* rbeg;
+    const int32_t* rcnt;
+    const float* rbox;
+    const float* rlam;
+    const float* qbox;
+    const float* qlam;
+    int64_t rleaf0, nleaves;
+    int leaves;  // how many of them are scored
+    int k;
+    ProbeOut* out;
+};
+
+inline ProbeArgs probe_args(const dtree_t* tq, const dtree_t* tr, ProbeOut* out) {
+    ProbeArgs a{};
+    a.qpts = tq->pts;
+    a.nq = tq->n;
+    a.rpts = tr->pts;
+    a.rbeg = tr->nbeg;
+    a.rcnt = tr->ncnt;
+    a.rbox = tr->box;
+    a.rlam = tr->lam;
+    a.qbox = tq->box;
+    a.qlam = tq->lam;
+    a.nleaves = tr->nleaves;
+    a.rleaf0 = tr->nleaves - 1;
+    a.leaves = (int)(tr->nleaves < kProbeLeaves ? tr->nleaves : kProbeLeaves);
+    a.out = out;
+    return a;
+}
+
+// DP = 16, 32 and 64 only.
+template <int DP>
+int launch_probe_far(const ProbeArgs& a, cudaStream_t s);
+
 // Whether a problem's extents (the reference points' radius R about their box
 // centre, the queries' largest distance from it) keep squared distances, and
 // the tensor-core keys' bounds relative to R^2, inside float32's range; *radius
@@ -290,7 +341,7 @@ int range_by_tiles(const dtree_t* tq, const dtree_t* tr, bool mono, const RangeO
 int extents_fit(const dtree_t* tq, const dtree_t* tr, cudaStream_t s, bool* fit, double* radius);
 
 // dtree_kfn by these passes: one problem whose extents keep every squared
-// distance inside float32's range (kfn.cu checks).  Adds to st when given.
+// distance inside float32's range (kfn.cu's look checks).  Adds to st when given.
 int kfn_by_tiles(const dtree_t* tq, const dtree_t* tr, bool mono, int k, int64_t* out_idx, float* out_dist,
                  cudaStream_t s, dtree_stats* st);
 

@@ -1,9 +1,10 @@
 // knn_far_16.cu -- furthest-neighbour and range passes of the block search for dimension bucket DP = 16.
-#include "knn_tc.cuh"
+#include "probe.cuh"
 
 namespace dt {
 template int launch_far_seed<16>(const TileArgs&, int, int, cudaStream_t);
 template int launch_far_cap<16>(const TileArgs&, int, int, float*, cudaStream_t);
 template int launch_far_tile<16>(const TileArgs&, int, int, bool, int*, int, cudaStream_t);
 template int launch_range_tile<16>(const TileArgs&, int, int*, int, cudaStream_t);
+template int launch_probe_far<16>(const ProbeArgs&, cudaStream_t);
 }  // namespace dt
