@@ -1304,25 +1304,6 @@ int device_checks(int prec, bool arena, const HostProb* hp, int np, int* dev_out
 
 }  // namespace
 
-int extents_fit(const dtree_t* tq, const dtree_t* tr, cudaStream_t s, bool* fit, double* radius) {
-    float qb[128], rb[128], ql = 0.f, rl = 0.f;
-    const size_t row = (size_t)2 * tr->dp * sizeof(float);
-    DT_CHECK(cudaMemcpyAsync(qb, tq->box, row, cudaMemcpyDeviceToHost, s));
-    DT_CHECK(cudaMemcpyAsync(rb, tr->box, row, cudaMemcpyDeviceToHost, s));
-    DT_CHECK(cudaMemcpyAsync(&ql, tq->lam, sizeof(float), cudaMemcpyDeviceToHost, s));
-    DT_CHECK(cudaMemcpyAsync(&rl, tr->lam, sizeof(float), cudaMemcpyDeviceToHost, s));
-    DT_CHECK(cudaStreamSynchronize(s));
-    double c2 = 0.0;
-    for (int j = 0; j < tr->dp; ++j) {
-        const double t = 0.5 * ((double)qb[j] + qb[tr->dp + j]) - 0.5 * ((double)rb[j] + rb[tr->dp + j]);
-        c2 += t * t;
-    }
-    const double qr = std::sqrt(c2) + ql;
-    *radius = std::max(qr, (double)rl);
-    *fit = rl >= 1e-12f && rl <= 1e15f && qr <= 1e15;
-    return DTREE_OK;
-}
-
 int range_by_tiles(const dtree_t* tq, const dtree_t* tr, bool mono, const RangeOut& r, cudaStream_t s,
                    dtree_stats* st) {
     const HostProb hp{tq, tr, mono, 1, nullptr, nullptr, 0, nullptr};

@@ -280,20 +280,21 @@ template <int DP>
 int launch_range_tile(const TileArgs& a, int items, int* err, int spin, cudaStream_t s);
 
 // One pass (count or fill) of a range search by block traversal and tensor-core
-// tiles; range.cu checks that it fits.  Adds to st when given.
+// tiles; range.cu's look checks that it fits.  Adds to st when given.
 int range_by_tiles(const dtree_t* tq, const dtree_t* tr, bool mono, const RangeOut& r, cudaStream_t s,
                    dtree_stats* st);
 
 // A look at a problem before it is searched (probe.cuh), made on the device: the
 // walk that follows it on the stream returns at once where gate is set, and the
 // host, which waits for the walk anyway, then runs the block search.
-constexpr int kProbeQueries = 64, kProbeLeaves = 1024;
+constexpr int kProbeQueries = 128, kProbeLeaves = 1024;
 
 struct ProbeOut {
     int gate;  // 1: the block search should serve the problem (zero before the look)
     int done;  // CTAs that have counted (zero before the look)
     int kept[kProbeQueries];  // per sampled query: the sampled leaves a walk would visit
-    int near[kProbeQueries];  // and the evaluated points that the tiles would settle exactly
+    int near[kProbeQueries];  // and the evaluated points that the tiles would settle exactly,
+    int pts[kProbeQueries];   // of this many
 };
 
 struct ProbeArgs {
@@ -306,9 +307,10 @@ struct ProbeArgs {
     const float* rlam;
     const float* qbox;
     const float* qlam;
-    int64_t rleaf0, nleaves;
+    int64_t nr, rleaf0, nleaves;
     int leaves;  // how many of them are scored
-    int k;
+    int k;                         // furthest neighbours
+    float lo2_dn, hi2_up, hi_up;   // range search: the ends, as in RangeOut
     ProbeOut* out;
 };
 
@@ -323,6 +325,7 @@ inline ProbeArgs probe_args(const dtree_t* tq, const dtree_t* tr, ProbeOut* out)
     a.rlam = tr->lam;
     a.qbox = tq->box;
     a.qlam = tq->lam;
+    a.nr = tr->n;
     a.nleaves = tr->nleaves;
     a.rleaf0 = tr->nleaves - 1;
     a.leaves = (int)(tr->nleaves < kProbeLeaves ? tr->nleaves : kProbeLeaves);
@@ -333,12 +336,8 @@ inline ProbeArgs probe_args(const dtree_t* tq, const dtree_t* tr, ProbeOut* out)
 // DP = 16, 32 and 64 only.
 template <int DP>
 int launch_probe_far(const ProbeArgs& a, cudaStream_t s);
-
-// Whether a problem's extents (the reference points' radius R about their box
-// centre, the queries' largest distance from it) keep squared distances, and
-// the tensor-core keys' bounds relative to R^2, inside float32's range; *radius
-// is then the larger of the two.  Reads both roots back.
-int extents_fit(const dtree_t* tq, const dtree_t* tr, cudaStream_t s, bool* fit, double* radius);
+template <int DP>
+int launch_probe_range(const ProbeArgs& a, cudaStream_t s);
 
 // dtree_kfn by these passes: one problem whose extents keep every squared
 // distance inside float32's range (kfn.cu's look checks).  Adds to st when given.

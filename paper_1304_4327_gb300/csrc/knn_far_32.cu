@@ -7,4 +7,5 @@ template int launch_far_cap<32>(const TileArgs&, int, int, float*, cudaStream_t)
 template int launch_far_tile<32>(const TileArgs&, int, int, bool, int*, int, cudaStream_t);
 template int launch_range_tile<32>(const TileArgs&, int, int*, int, cudaStream_t);
 template int launch_probe_far<32>(const ProbeArgs&, cudaStream_t);
+template int launch_probe_range<32>(const ProbeArgs&, cudaStream_t);
 }  // namespace dt

@@ -1,7 +1,7 @@
 // probe.cuh -- a look at a problem before it is searched: what a walk per query
 // would visit, and what the block search's tiles would have to settle exactly.
 //
-// A CTA per sampled query scores up to 1024 leaves, evenly spaced in the tree,
+// A CTA per sampled query scores up to 1024 leaves, spread over the tree,
 // and evaluates the points of a few of them; counts go out (the same in every
 // call).  No chain of loads is longer than a few, so that the whole look costs
 // little more than its read-back; a sample of walks would take as long as its
@@ -12,7 +12,14 @@
 
 namespace dt {
 
-constexpr int kProbeThreads = 128, kProbeTop = 8, kProbeRows = 64;
+constexpr int kProbeThreads = 128, kProbeTop = 8, kProbeRangeTop = 16, kProbeRows = 64;
+
+// The i-th of S strata of [0, n), at a place of its own in each (the first point or leaf
+// of a subtree is in a corner of it).
+__device__ __forceinline__ int64_t probe_pick(int i, int64_t n, int S) {
+    const uint32_t width = (uint32_t)(n / S);
+    return i * n / S + (width > 1 ? ((uint32_t)(i + 1) * 0x9e3779b1u >> 8) % width : 0u);
+}
 
 template <int DP>
 __device__ __forceinline__ float probe_load(float (&q)[DP], const float* qp, const float* rbox) {
@@ -34,9 +41,10 @@ __device__ __forceinline__ float probe_load(float (&q)[DP], const float* qp, con
     return sqrtf(a2);
 }
 
-// The CTA's two counts; true for the first warp of the last CTA, which gets the
-// totals.
-__device__ __forceinline__ bool probe_total(const ProbeArgs& a, int kept, int near, int& all_kept, int& all_near) {
+// The CTA's counts (kept and near summed over its threads, pts the same in all);
+// true for the first warp of the last CTA, which gets the totals.
+__device__ __forceinline__ bool probe_total(const ProbeArgs& a, int kept, int near, int pts, int& all_kept,
+                                            int& all_near, int& all_pts) {
     __shared__ int part[2][kProbeThreads / 32];
     __shared__ bool s_last;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -55,19 +63,22 @@ __device__ __forceinline__ bool probe_total(const ProbeArgs& a, int kept, int ne
         }
         a.out->kept[blockIdx.x] = kept;
         a.out->near[blockIdx.x] = near;
+        a.out->pts[blockIdx.x] = pts;
         __threadfence();
         s_last = atomicAdd(&a.out->done, 1) == (int)gridDim.x - 1;
     }
     __syncthreads();
     if (!s_last || tid >= 32) return false;
     __threadfence();
-    int k = 0, n = 0;  // (at most 1024 per CTA, of 64)
+    int k = 0, n = 0, m = 0;  // (at most 1024 x 1024 per CTA, of 128)
     for (int q = lane; q < (int)gridDim.x; q += 32) {
         k += __ldcg(&a.out->kept[q]);
         n += __ldcg(&a.out->near[q]);
+        m += __ldcg(&a.out->pts[q]);
     }
     all_kept = __reduce_add_sync(0xffffffffu, k);
     all_near = __reduce_add_sync(0xffffffffu, n);
+    all_pts = __reduce_add_sync(0xffffffffu, m);
     return true;
 }
 
@@ -127,10 +138,10 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_far(const ProbeArgs a) 
     __shared__ uint32_t s_kth;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float q[DP];
-    const float qa = probe_load<DP>(q, a.qpts + (blockIdx.x * a.nq / gridDim.x) * DP, a.rbox);
+    const float qa = probe_load<DP>(q, a.qpts + probe_pick(blockIdx.x, a.nq, gridDim.x) * DP, a.rbox);
     const int S = a.leaves;
     for (int i = tid; i < S; i += kProbeThreads) {
-        const float4* lo4 = reinterpret_cast<const float4*>(a.rbox + (a.rleaf0 + i * a.nleaves / S) * 2 * DP);
+        const float4* lo4 = reinterpret_cast<const float4*>(a.rbox + (a.rleaf0 + probe_pick(i, a.nleaves, S)) * 2 * DP);
         float s = 0.f;
 #pragma unroll
         for (int j = 0; j < DP / 4; ++j) {
@@ -162,7 +173,7 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_far(const ProbeArgs a) 
         if (best == 0) break;  // (fewer than eight leaves)
         last = best;
         if (tid == 0) {
-            const int64_t nd = a.rleaf0 + ((int64_t)(uint32_t)best - 1) * a.nleaves / S;
+            const int64_t nd = a.rleaf0 + probe_pick((int)(uint32_t)best - 1, a.nleaves, S);
             tbeg[nt] = a.rbeg[nd];
             tcnt[nt] = a.rcnt[nd];
         }
@@ -193,8 +204,8 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_far(const ProbeArgs a) 
     int kept = 0, near = 0;
     for (int i = tid; i < S; i += kProbeThreads) kept += dm[i] >= kth;
     for (int v = tid; v < np; v += kProbeThreads) near += pv[v] >= band;
-    int all_kept, all_near;
-    if (!probe_total(a, kept, near, all_kept, all_near)) return;
+    int all_kept, all_near, all_pts;
+    if (!probe_total(a, kept, near, np, all_kept, all_near, all_pts)) return;
     float radius;
     const bool extents = probe_extents<DP>(a, radius);
     if (lane == 0) {
@@ -202,6 +213,99 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_far(const ProbeArgs a) 
         const float kept_q = (float)all_kept / (float)gridDim.x, near_q = (float)all_near / (float)gridDim.x;
         a.out->gate = extents && far_by_tiles(a.k, a.nq, kept_q / (float)S, kept_q * scale, near_q * scale, scale);
     }
+}
+
+// Range searches, from a walk's share of the leaves, the points in them, and the
+// share of those that lie within the upper end (which the tiles evaluate one by
+// one, and in float64 when they write them).
+//
+// The tiles win where many leaves are visited for few results (the mixture, d = 16,
+// 1M x 50k points: radius 2.0 1.3% of the leaves, 22.9 -> 2.8 ms; 2.5 2.0% and 0.03%
+// of the points, 32.9 -> 5.2; 3.0 2.6% and 0.3%, 42.6 -> 20.4; 10k x 150k at 2.0, 260
+// points, 2.1 -> 1.0; eight latent dimensions, 300k x 50k, 1.1% and 0.4%, 15.5 -> 7.9;
+// d = 32 at 5.5 3.2% and 0.5%, 50 -> 16) and lose where the results are many or the
+// leaves few, most of all at low intrinsic dimension (the mixture at 3.5 2.9% and
+// 1.4%, 77 -> 103; d = 10 at 1.9 1.2% and 0.6%, 12.2 -> 14.1; 300k x 50k points of
+// three latent dimensions at 0.4 1.1% and 45%, 40 -> 243; 1M x 20k of six in d = 32 at
+// 0.6 0.2% and 0.5%, 6.5 -> 8.6; at 1.0 0.8% and 2.2%, 24 -> 72; distances of 9 to 20
+// among Gaussian points, where nearly all points lie within the upper end, 64 -> 207).
+template <int DP>
+__device__ __forceinline__ bool range_by_tiles_pays(float share, float points, float within) {
+    return share >= 0.0025f && points >= 150.f && within <= (DP <= 16 ? 0.0045f : 0.008f);
+}
+
+// Range searches: kept counts the sampled leaves that meet the range, near the
+// points within its upper end of up to sixteen of them, evenly chosen.
+template <int DP>
+__global__ void __launch_bounds__(kProbeThreads) k_probe_range(const ProbeArgs a) {
+    __shared__ int list[kProbeLeaves], wcnt[kProbeThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float q[DP];
+    probe_load<DP>(q, a.qpts + probe_pick(blockIdx.x, a.nq, gridDim.x) * DP, a.rbox);
+    const int S = a.leaves;
+    const float dn = 1.f - 2.f * rel_eps<DP>(), up = 1.f + 2.f * rel_eps<DP>();
+    int kept = 0, found = 0;  // this thread's, the CTA's so far
+    for (int i0 = 0; i0 < S; i0 += kProbeThreads) {
+        const int i = i0 + tid;
+        bool keep = false;
+        if (i < S) {
+            const float4* lo4 = reinterpret_cast<const float4*>(a.rbox + (a.rleaf0 + probe_pick(i, a.nleaves, S)) * 2 * DP);
+            float mn = 0.f, mx = 0.f;
+#pragma unroll
+            for (int j = 0; j < DP / 4; ++j) {
+                const float4 lo = lo4[j], hi = lo4[DP / 4 + j];
+                const float l[4] = {lo.x, lo.y, lo.z, lo.w}, h[4] = {hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const float below = l[t] - q[4 * j + t], above = q[4 * j + t] - h[t];
+                    const float g = fmaxf(fmaxf(below, above), 0.f), f = fmaxf(-below, -above);
+                    mn = fmaf(g, g, mn);
+                    mx = fmaf(f, f, mx);
+                }
+            }
+            keep = !(mn * dn > a.hi2_up) && !(mx * up < a.lo2_dn);
+        }
+        kept += keep;
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        if (lane == 0) wcnt[warp] = __popc(m);
+        __syncthreads();
+        int at = found + __popc(m & ((1u << lane) - 1u));
+        for (int w = 0; w < kProbeThreads / 32; ++w) {
+            if (w < warp) at += wcnt[w];
+            found += wcnt[w];
+        }
+        if (keep) list[at] = i;
+        __syncthreads();
+    }
+    int near = 0, pts = 0;
+    const int nt = min(found, kProbeRangeTop);
+    for (int t = 0; t < nt; ++t) {
+        const int64_t nd = a.rleaf0 + probe_pick(list[probe_pick(t, found, nt)], a.nleaves, S);
+        const int rows = min(a.rcnt[nd], kProbeRows);
+        pts += rows;
+        if (t % (kProbeThreads / 32) != warp) continue;
+        for (int r = lane; r < rows; r += 32)
+            near += approx_d2<DP>(q, a.rpts + ((int64_t)a.rbeg[nd] + r) * DP) <= a.hi2_up;
+    }
+    // (each query by the leaves it stands for: sixteen times found / nt)
+    const int weight = nt == kProbeRangeTop ? found : kProbeRangeTop;
+    int all_kept, all_near, all_pts;
+    if (!probe_total(a, kept, near * weight, pts * weight, all_kept, all_near, all_pts)) return;
+    float radius;
+    const bool extents = probe_extents<DP>(a, radius);
+    if (lane == 0) {
+        const float share = (float)all_kept / ((float)gridDim.x * (float)S);
+        // (a range far below the extents: the tensor-core keys' error, about 1e-4
+        // of their square, would add too many candidates)
+        a.out->gate = extents && a.hi_up * a.hi_up >= 4e-4f * radius * radius &&
+                      range_by_tiles_pays<DP>(share, share * (float)a.nr, (float)all_near / fmaxf((float)all_pts, 1.f));
+    }
+}
+
+template <int DP>
+int launch_probe_range(const ProbeArgs& a, cudaStream_t s) {
+    DT_LAUNCH(k_probe_range<DP>, (int)(a.nq < kProbeQueries ? a.nq : kProbeQueries), kProbeThreads, 0, s, a);
+    return DTREE_OK;
 }
 
 template <int DP>

@@ -85,31 +85,38 @@ RangeOut range_out(const RangeArgs& a, bool fill) {
     return r;
 }
 
-// Whether the block search serves a range: enough work that its passes pay
-// (d > 8, 10k queries and 1e9 pairs), a candidate bit per (block, leaf) in at most 1 GB,
-// extents that its float32 bounds cover, and a range whose square is at least
-// 4e-4 of the largest squared extent, so that the tensor-core keys' error
-// (about 1e-4 of it) adds few candidates.  Both passes of a search decide alike.
+// Whether the block search may serve a range: enough work that its passes pay
+// (d > 8, 10k queries and 1e9 pairs) and a candidate bit per (block, leaf) in at
+// most 1 GB.  A look at the points then decides (probe.cuh: their extents, what a
+// walk would visit, and how many of the points it evaluates are results).  Both
+// passes of a search decide alike.
 //
 // A walk per query visits few leaves where the box bound prunes well (d <= 8),
 // and a few queries make too few blocks for the GPU (mixture, d = 16, radius
 // 2.4: 1M x 2k points 5.3 against 6.9 ms, 300k x 5k 4.4 against 4.6).  Above,
 // blocks share the visits and the tensor cores do the distances: 100k x 20k
 // 4.2 -> 3.9 ms, 1M x 20k 16.5 -> 6.9, 1M x 100k 64 -> 10.3; 300k x 100k in d =
-// 32 91 -> 13; 100k x 20k in d = 64 179 -> 21; points of three latent
-// dimensions 6.3 -> 6.2.
-int range_tiles_fit(const dtree_t* tq, const dtree_t* tr, double d_hi, cudaStream_t s, bool* fit) {
-    *fit = false;
+// 32 91 -> 13; 100k x 20k in d = 64 179 -> 21.
+bool range_tiles_fit(const dtree_t* tq, const dtree_t* tr) {
+    if (tr->dp < 16 || tq->n < 10000 || (double)tq->n * (double)tr->n < 1e9) return false;
+    if ((double)tq->n / 64.0 * (double)tr->nleaves / 8.0 > 1e9) return false;
     int major = 0, minor = 0;
     cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, tr->device);
     cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, tr->device);
-    if (major != 10 || minor != 3) return DTREE_OK;  // the tiles are tcgen05 code
-    if (tr->dp < 16 || tq->n < 10000 || (double)tq->n * (double)tr->n < 1e9) return DTREE_OK;
-    if ((double)tq->n / 64.0 * (double)tr->nleaves / 8.0 > 1e9) return DTREE_OK;
-    double radius = 0.0;
-    const int rc = extents_fit(tq, tr, s, fit, &radius);
-    if (!(d_hi * d_hi >= 4e-4 * radius * radius)) *fit = false;
-    return rc;
+    return major == 10 && minor == 3;  // the tiles are tcgen05 code
+}
+
+int range_look(const dtree_t* tq, const dtree_t* tr, const RangeArgs& r, ProbeOut* out, cudaStream_t s) {
+    ProbeArgs a = probe_args(tq, tr, out);
+    a.lo2_dn = r.lo2_dn;
+    a.hi2_up = r.hi2_up;
+    a.hi_up = range_out(r, false).hi_up;
+    if (cudaMemsetAsync(out, 0, 8, s) != cudaSuccess) return cuda_status(cudaGetLastError());
+    switch (tr->dp) {
+        case 16: return launch_probe_range<16>(a, s);
+        case 32: return launch_probe_range<32>(a, s);
+        default: return launch_probe_range<64>(a, s);
+    }
 }
 
 }  // namespace
@@ -126,43 +133,51 @@ extern "C" int dtree_range_count(const dtree_t* query, const dtree_t* ref, doubl
     if (!offsets || !total) return DTREE_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t launches0 = g_launches.load();
-    // scratch: four counters and the scan's block sums
+    const dtree_t* tq = query ? query : ref;
+    // scratch: four counters, the look's result and the scan's block sums
     unsigned long long* cnt = nullptr;
-    DT_CHECK(cudaMallocAsync((void**)&cnt, (4 + (size_t)scan_blocks(a.nq)) * sizeof(unsigned long long), s));
-    int64_t* sums = reinterpret_cast<int64_t*>(cnt + 4);
+    constexpr size_t n_look = (sizeof(ProbeOut) + 7) / 8;
+    DT_CHECK(cudaMallocAsync((void**)&cnt, (4 + n_look + (size_t)scan_blocks(a.nq)) * sizeof(unsigned long long), s));
+    ProbeOut* look = reinterpret_cast<ProbeOut*>(cnt + 4);
+    int64_t* sums = reinterpret_cast<int64_t*>(cnt + 4 + n_look);
     g_allocs.fetch_add(1, std::memory_order_relaxed);
     a.counts = offsets;
     a.stats = cnt;
-    unsigned long long h[4] = {0, 0, 0, 0};
+    unsigned long long h[5] = {0, 0, 0, 0, 0};  // the counters, and the look's verdict (its low half)
     dtree_stats tst{};  // the block search's counters
     cudaEvent_t ev[2] = {};
     const bool timed = st && cudaEventCreate(&ev[0]) == cudaSuccess && cudaEventCreate(&ev[1]) == cudaSuccess;
     cudaGetLastError();
-    do {
-        if (cudaMemsetAsync(cnt, 0, 4 * sizeof(unsigned long long), s) != cudaSuccess) {
+    bool ask = range_tiles_fit(tq, ref), tiles = false;
+    for (;;) {
+        a.gate = ask ? &look->gate : nullptr;
+        if (cudaMemsetAsync(cnt, 0, 5 * sizeof(unsigned long long), s) != cudaSuccess) {
             rc = cuda_status(cudaGetLastError());
             break;
         }
         if (timed) cudaEventRecord(ev[0], s);
-        bool tiles = false;
-        rc = range_tiles_fit(query ? query : ref, ref, d_hi, s, &tiles);
-        if (rc != DTREE_OK) break;
+        if (ask && (rc = range_look(tq, ref, a, look, s)) != DTREE_OK) break;
         if (tiles) {
-            rc = range_by_tiles(query ? query : ref, ref, a.mono != 0, range_out(a, false), s, st ? &tst : nullptr);
+            rc = range_by_tiles(tq, ref, a.mono != 0, range_out(a, false), s, st ? &tst : nullptr);
             if (rc == DTREE_ERR_OOM) tiles = false;  // (the walk needs no memory)
             else if (rc != DTREE_OK) break;
         }
-        if (!tiles) rc = range_launch(ref->dp, a, false, range_grid(a.nq), s);
-        if (rc != DTREE_OK) break;
+        if (!tiles && (rc = range_launch(ref->dp, a, false, range_grid(a.nq), s)) != DTREE_OK) break;
+        // (before the verdict is known: sums of nothing in particular where the
+        // walks stood back)
         rc = exclusive_scan(offsets, a.nq, sums, s);
         if (rc != DTREE_OK) break;
         if (timed) cudaEventRecord(ev[1], s);
         if (cudaMemcpyAsync(total, offsets + a.nq, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaMemcpyAsync(h, cnt, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess) {
+            cudaMemcpyAsync(h, cnt, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess) {
             rc = cuda_status(cudaGetLastError());
             break;
         }
-    } while (false);
+        if (!ask || (uint32_t)h[4] == 0) break;
+        ask = false;
+        tiles = true;
+    }
     cudaFreeAsync(cnt, s);
     if (cudaStreamSynchronize(s) != cudaSuccess && rc == DTREE_OK) rc = cuda_status(cudaGetLastError());
     if (st && rc == DTREE_OK) {
@@ -195,14 +210,23 @@ extern "C" int dtree_range_fill(const dtree_t* query, const dtree_t* ref, double
     a.offsets = offsets;
     a.out_idx = out_idx;
     a.out_dist = out_dist;
-    bool tiles = false;
-    rc = range_tiles_fit(query ? query : ref, ref, d_hi, s, &tiles);
-    if (rc != DTREE_OK) return rc;
-    if (tiles) {
-        rc = range_by_tiles(query ? query : ref, ref, a.mono != 0, range_out(a, true), s, nullptr);
-        if (rc == DTREE_ERR_OOM) tiles = false;
+    const dtree_t* tq = query ? query : ref;
+    int verdict = 0;
+    ProbeOut* look = nullptr;
+    if (range_tiles_fit(tq, ref) && scratch(&look, 1, s) == DTREE_OK) {
+        a.gate = &look->gate;
+        rc = range_look(tq, ref, a, look, s);
     }
-    if (!tiles) rc = range_launch(ref->dp, a, true, range_grid(a.nq), s);
+    if (rc == DTREE_OK) rc = range_launch(ref->dp, a, true, range_grid(a.nq), s);
+    if (rc == DTREE_OK && look && (cudaMemcpyAsync(&verdict, &look->gate, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+                                   cudaStreamSynchronize(s) != cudaSuccess))
+        rc = cuda_status(cudaGetLastError());
+    if (look) cudaFreeAsync(look, s);
+    if (rc == DTREE_OK && verdict) {
+        a.gate = nullptr;
+        rc = range_by_tiles(tq, ref, a.mono != 0, range_out(a, true), s, nullptr);
+        if (rc == DTREE_ERR_OOM) rc = range_launch(ref->dp, a, true, range_grid(a.nq), s);
+    }
     if (cudaStreamSynchronize(s) != cudaSuccess && rc == DTREE_OK) rc = cuda_status(cudaGetLastError());
     return rc;
 }

@@ -19,6 +19,9 @@
 //     d_hi^2 carry a relative margin of 1e-12, far above any float64
 //     rounding, so such a decision is the float64 one.  Every other point is
 //     decided on its float64 distance.
+// Large problems in d > 8 whose walks would visit much for few results go through
+// the block search of knn.cu (range.cu's range_tiles_fit and probe.cuh say which).
+//
 // Counting and filling take the same decisions, so a query's count is the
 // length of its filled segment.
 #pragma once
@@ -48,6 +51,7 @@ struct RangeArgs {
     int64_t* out_idx;
     float* out_dist;
     unsigned long long* stats;    // [0] distances, [1] leaves, [2] nodes pruned, [3] float64 decisions
+    const int* gate;              // set on the device: the block search serves the call; or null
 };
 
 template <int DP, bool FILL>
@@ -56,6 +60,10 @@ __global__ void __launch_bounds__(128) k_range(const RangeArgs a) {
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    // the gate is set by an earlier kernel; every thread of the grid reads the same
+    // (as a C++ return it changed the register allocation of the walk: 5% slower
+    // at d = 32)
+    if (a.gate && *a.gate) asm volatile("exit;");
     const bool mono = a.mono != 0;
     const float eps = rel_eps<DP>();
     const float box_dn = 1.f - (DP + 4) * 1.2e-7f, box_up = 1.f + (DP + 4) * 1.2e-7f;
