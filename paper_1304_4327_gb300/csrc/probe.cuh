@@ -101,27 +101,31 @@ __device__ __forceinline__ bool probe_extents(const ProbeArgs& a, float& radius)
 }
 
 // The rule, from what a walk would visit of the reference tree per query (share
-// of the leaves, number of them) and how many points the tile's band would hold
-// (near, where scale leaves stand behind each scored one).
+// of the leaves) and how many of the evaluated points the tile's band would hold
+// (near).
 //
 // A walk per query visits few leaves where the points' intrinsic dimension is
 // low, whatever the space they lie in, and then beats the tiles, whose blocks
 // must visit what any of 128 queries needs.  Walks and tiles, by the share
-// estimated: 300k x 50k points of d = 16 with three latent dimensions 0.1%, 0.77
-// and 1.52 ms; with seven 1.1%, 8.7 and 6.9; with ten 3.6%, 33 and 7.7; 1M x 20k
-// of d = 32, four latent dimensions 0.2%, 1.4 and 6.8 ms; six 1.1%, 9.2 and 15.8;
-// eight 2.1%, 19 and 16; the mixture, d = 10, 1M x 100k 3%, 69 and 18 ms, d = 16, 1M x
-// 200k 8%, 312 and 41.  Few leaves in all: 20k x 100k, four latent dimensions 1%,
-// 11 of 1024 leaves, 1.5 and 1.8 ms.  Lists of 64 (k > 18) cost the tiles half
-// as much again, and few queries leave the GPU to the latency of either:
-// mixture, d = 10, 250k x 8,200, k = 30, 570 leaves, 3.5 and 4.0 ms; 1M x 4,100, 1,090
-// leaves, 6.7 and 5.3; 250k x 16,400, 6.2 and 5.2.
+// of the leaves: 300k x 50k points of d = 16 with three latent dimensions 0.1%, 0.77
+// and 1.52 ms; with six 0.6%, 6.2 and 6.3; with ten 4.6%, 33 and 7.7; 1M x 20k of d =
+// 32, four latent dimensions 0.1%, 1.4 and 6.8 ms; seven 0.7%, 11 and 16; eight 1.3%,
+// 19 and 16; the mixture, d = 10, 1M x 100k 4%, 69 and 18 ms, d = 16, 1M x 200k 11%, 312
+// and 41.  Few points in all: 20k x 100k, four latent dimensions 1.5%, 300 points,
+// 1.5 and 1.8 ms; five 3.5%, 700, 2.7 and 2.1; 30k x 40k of d = 10 with three in 32
+// leaves, of which a walk visits two, 1.1 and 1.5.  Lists of 64 (k > 18) cost the tiles
+// half as much again, and few queries leave the GPU to the latency of either:
+// mixture, d = 10, k = 30, 250k x 8,200, 20,000 points, 3.5 and 4.0 ms; 1M x 4,100,
+// 51,000 points, 6.7 and 5.3; 250k x 16,400, 6.2 and 5.2.
 // Where the band holds more than a list (equal or nearly equal distances), the
 // tiles' work is done twice: queries at the centre of a sphere 16.8 against 14.2
 // ms.  A healthy band holds about k points of all, or about one of those sampled.
-__device__ __forceinline__ bool far_by_tiles(int k, int64_t nq, float share, float visits, float near, float scale) {
-    return share >= 0.018f && visits >= 24.f && (k <= 18 || nq >= 16384 || visits >= 800.f) &&
-           near <= fmaxf(k + 14.f, 2.f * (k + scale));
+template <int DP>
+__device__ __forceinline__ bool far_by_tiles(const ProbeArgs& a, float share, float near) {
+    const float leaves = share * (float)a.nleaves, points = share * (float)a.nr;
+    const float scale = (float)a.nleaves / (float)a.leaves;  // leaves behind each scored one
+    return share >= (DP <= 16 ? 0.011f : 0.016f) && leaves >= 8.f && points >= 480.f &&
+           (a.k <= 18 || a.nq >= 16384 || points >= 24000.f) && near * scale <= fmaxf(a.k + 14.f, 2.f * (a.k + scale));
 }
 
 // The furthest neighbours: the query's k-th furthest distance is estimated from
@@ -209,9 +213,8 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_far(const ProbeArgs a) 
     float radius;
     const bool extents = probe_extents<DP>(a, radius);
     if (lane == 0) {
-        const float scale = (float)a.nleaves / (float)S;
-        const float kept_q = (float)all_kept / (float)gridDim.x, near_q = (float)all_near / (float)gridDim.x;
-        a.out->gate = extents && far_by_tiles(a.k, a.nq, kept_q / (float)S, kept_q * scale, near_q * scale, scale);
+        a.out->gate = extents && far_by_tiles<DP>(a, (float)all_kept / ((float)gridDim.x * (float)S),
+                                                  (float)all_near / (float)gridDim.x);
     }
 }
 

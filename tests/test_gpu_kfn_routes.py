@@ -67,6 +67,12 @@ def test_wide_bands_walk(dt):
     assert not search(dt, repeated(60_000, 16, 1), repeated(20_000, 16, 2), 10)
 
 
+def test_points_are_counted_not_leaves(dt):
+    # 32 leaves of some 900 points each
+    assert search(dt, mixture(30_000, 10, 5), mixture(40_000, 10, 6), 10, 1_000)
+    assert not search(dt, latent(30_000, 10, 3, 5), latent(40_000, 10, 3, 6), 10, 1_000)
+
+
 @pytest.mark.parametrize("nq,m", [(4_096, 250_000), (1_000_000, 1_010)])
 def test_few_queries_and_few_references(dt, nq, m):
     # (1,010 points in 64 leaves: every leaf is scored)
