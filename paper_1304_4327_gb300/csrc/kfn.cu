@@ -131,8 +131,9 @@ extern "C" int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, in
             rc = kfn_by_tiles(tq, ref, mono, k, out_idx, out_dist, s, st);
             tiles = rc == DTREE_OK;
             // (its operand rows or candidate pairs may not fit where the walks,
-            // which need 4 bytes a query, do)
-            if (rc != DTREE_ERR_OOM) break;
+            // which need 4 bytes a query, do, and its waits are bounded where the
+            // walks wait for nothing)
+            if (rc != DTREE_ERR_OOM && rc != DTREE_ERR_TIMEOUT) break;
             if (st) memset(st, 0, sizeof(*st));
             continue;
         }

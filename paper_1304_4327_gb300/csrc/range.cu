@@ -159,7 +159,7 @@ extern "C" int dtree_range_count(const dtree_t* query, const dtree_t* ref, doubl
         if (ask && (rc = range_look(tq, ref, a, look, s)) != DTREE_OK) break;
         if (tiles) {
             rc = range_by_tiles(tq, ref, a.mono != 0, range_out(a, false), s, st ? &tst : nullptr);
-            if (rc == DTREE_ERR_OOM) tiles = false;  // (the walk needs no memory)
+            if (rc == DTREE_ERR_OOM || rc == DTREE_ERR_TIMEOUT) tiles = false;  // (the walk needs no memory and has no waits)
             else if (rc != DTREE_OK) break;
         }
         if (!tiles && (rc = range_launch(ref->dp, a, false, range_grid(a.nq), s)) != DTREE_OK) break;
@@ -225,7 +225,7 @@ extern "C" int dtree_range_fill(const dtree_t* query, const dtree_t* ref, double
     if (rc == DTREE_OK && verdict) {
         a.gate = nullptr;
         rc = range_by_tiles(tq, ref, a.mono != 0, range_out(a, true), s, nullptr);
-        if (rc == DTREE_ERR_OOM) rc = range_launch(ref->dp, a, true, range_grid(a.nq), s);
+        if (rc == DTREE_ERR_OOM || rc == DTREE_ERR_TIMEOUT) rc = range_launch(ref->dp, a, true, range_grid(a.nq), s);
     }
     if (cudaStreamSynchronize(s) != cudaSuccess && rc == DTREE_OK) rc = cuda_status(cudaGetLastError());
     return rc;
