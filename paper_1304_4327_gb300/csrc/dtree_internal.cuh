@@ -33,13 +33,13 @@ struct dtree {
     int32_t* ncnt = nullptr;
     int device = 0;
     void* block = nullptr;  // the arrays above but pts and idx
-    // frontier capacity that sufficed for the last traversal against this
+    // frontier capacity that sufficed for the last kNN traversal against this
     // reference tree (a sizing hint only; results never depend on it)
     int64_t cap_hint = 0;
     // learned proposal attached to this reference tree (not owned), or null
     const dtree_model* proposal = nullptr;
     // tensor-core operand rows of the points (TF32, split BF16), made by the
-    // first search that needs them and owned by the handle
+    // first kNN search that asks for that precision and owned by the handle
     void* tc_ops[2] = {nullptr, nullptr};
 };
 

@@ -761,8 +761,10 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
     P.s = s;
     P.arena = arena;
     if (fmt) {
-        // the reference points as tensor-core operand rows (made once per
-        // tree and format, or carved from the fixed range for this call)
+        // the reference points as tensor-core operand rows: made once per tree and
+        // format and kept there, but in this call's scratch for a fixed range, and
+        // for the searches that need not have asked for tiles (k-furthest, range:
+        // the caller chose no precision, and the walks leave nothing in the tree)
         for (int i = 0; i < np; ++i) {
             const dtree_t* tr = hp[i].tr;
             const int64_t maxleaf = (tr->n + tr->nleaves - 1) / tr->nleaves;
@@ -771,7 +773,7 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
             void* ops = cache;
             if (!ops) {
                 const size_t bytes = (size_t)tr->nleaves * ls * tc_ops_row_bytes<DP>(fmt);
-                if (arena) {
+                if (arena || OP != OP_NEAR) {
                     unsigned char* p = nullptr;
                     DT_TRY(P.get(&p, bytes));
                     ops = p;
@@ -916,7 +918,8 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
 
     // 3. level-synchronous pruning dual-tree traversal
     int64_t cap = std::max<int64_t>(1 << 20, (int64_t)NB * 256);
-    if (np == 1) cap = std::max<int64_t>(cap, hp[0].tr->cap_hint);
+    // (a hint of kNN searches for kNN searches: the others keep more pairs)
+    if (OP == OP_NEAR && np == 1) cap = std::max<int64_t>(cap, hp[0].tr->cap_hint);
     if (arena) {
         // a fixed range: the pair buffers take what is left, once (the three
         // blocks' alignment costs at most 3 x 255 bytes)
@@ -1041,7 +1044,7 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
         }
         P.release(F[1]);
         P.release(F[0]);
-        if (np == 1)
+        if (OP == OP_NEAR && np == 1)
             const_cast<dtree_t*>(hp[0].tr)->cap_hint = std::max(fcap[0], std::max(fcap[1], ocap));
         DT_TRY(finish_csr((int)used));
     } else {
