@@ -247,7 +247,9 @@ __global__ void __launch_bounds__(128) k_emst_nn(const EmstArgs a) {
         }
         if (need) {
             done = br >= 0 && key_up<DP>(best) <= cub;
-            if (sub == 0) a.lb[pos] = fmaxf(__fmul_rd(fminf(best, cub), 1.f - 8.f * rel_eps<DP>()) - kKeyTiny, 0.f);
+            // (an overflowing key stands for the largest float at least, as in packet.cuh)
+            const float least = fminf(fminf(best, cub), kKeyMax);
+            if (sub == 0) a.lb[pos] = fmaxf(__fmul_rd(least, 1.f - 8.f * rel_eps<DP>()) - kKeyTiny, 0.f);
         }
     }
     if (in && sub == 0) {
