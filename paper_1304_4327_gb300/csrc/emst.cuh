@@ -108,10 +108,19 @@ __global__ void __launch_bounds__(128) k_emst_prep(const EmstArgs a) {
     if (in && lane == __ffs(peers) - 1 && best < INFINITY) emst_publish(a.cub + mine, best);
 }
 
+// The smallest of a value over a point's G lanes (a power of two).
+__device__ __forceinline__ float emst_lanes_min(float v, int G) {
+    for (int off = G >> 1; off > 0; off >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, off));
+    return v;
+}
+
 // The nearest point outside its component of every point that can still hold
 // its component's shortest edge, by packets (packet.cuh) that walk the tree
 // nearer child first.  The G lanes of a point share its bound and keep a best
-// edge each, the best of which is taken at the end.
+// edge each, the best of which is taken at the end.  Other warps lower a
+// component's bound meanwhile, so that the lanes may read different values:
+// each takes the smallest, or what one lane pruned by a smaller bound would be
+// missing from what the point's first lane then records (done, lb).
 //
 // Score: a lane prunes a node when all the node's points lie in its own
 // component, or when the squared d_min, rounded down, exceeds the smaller of
@@ -148,8 +157,9 @@ __global__ void __launch_bounds__(128) k_emst_nn(const EmstArgs a) {
     int32_t br = -1;
     bool have64 = false, need = in, done = false;
     float cub = INFINITY;
+    if (!a.first && in) cub = __uint_as_float(*reinterpret_cast<volatile uint32_t*>(a.cub + mine));
+    cub = emst_lanes_min(cub, G);
     if (!a.first && in) {
-        cub = __uint_as_float(*reinterpret_cast<volatile uint32_t*>(a.cub + mine));
         br = a.br[pos];
         bd = a.bd[pos];
         have64 = br >= 0;
@@ -215,14 +225,13 @@ __global__ void __launch_bounds__(128) k_emst_nn(const EmstArgs a) {
                         }
                     }
                 }
-                float best = bk;
-                for (int off = G >> 1; off > 0; off >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, off));
+                const float up = key_up<DP>(emst_lanes_min(bk, G));
                 if (want) {
-                    const float up = key_up<DP>(best);
                     if (up < cub) emst_publish(a.cub + mine, up);
                     cub = fminf(cub, __uint_as_float(*reinterpret_cast<volatile uint32_t*>(a.cub + mine)));
-                    bound = fminf(up, cub);
                 }
+                cub = emst_lanes_min(cub, G);
+                bound = fminf(up, cub);
                 continue;
             }
             const int64_t l = 2 * (int64_t)n + 1;
