@@ -740,10 +740,16 @@ __global__ void __launch_bounds__(32 * (4 * NG + 3), 1) k_tile_tc(const TileArgs
                     }
                     const int lo = max(gs, g0), hi = min(ge, g1);
                     const bool over = hi > lo;
+                    const long long tcp = TC_TIMED ? clock64() : 0;
                     if (over)
                         tc::bulk_g2s(sB + op * TN * S::RB + (lo - g0) * S::GB,
                                      rops + ((int64_t)e.z * ls8 + (lo - gs)) * S::GB, (uint32_t)(hi - lo) * S::GB,
                                      &op_full[op]);
+                    if (TC_TIMED) {
+                        __syncwarp();
+                        if (pl == 0 && lane == 0)
+                            atomicAdd(&x.timers[TT_PLAN_COPY], (unsigned long long)(clock64() - tcp));
+                    }
                     if (lane == 0) ometa[op] = (g1 - g0) * 8;
                     // the row-group table: lane l describes group g0 + l, of
                     // the last entry that starts at or before it
