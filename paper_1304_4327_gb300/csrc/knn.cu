@@ -936,7 +936,7 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
         npairs = n;
         DT_TRY(P.get(&csr_leaf, std::max(npairs, 1)));
         DT_TRY(P.get(&csr_dmin, std::max(npairs, 1)));
-        DT_TRY(P.get(&csr_key, std::max(npairs, 1)));
+        DT_TRY(P.get(&csr_key, OP == OP_RANGE ? 0 : std::max(npairs, 1)));  // (ranges have no order)
         DT_LAUNCH(k_scan, 1, 1024, 0, s, bcount, NB, off);
         DT_CHECK(cudaMemsetAsync(bcur, 0, NB * sizeof(int), s));
         if constexpr (OP == OP_RANGE) {
@@ -956,7 +956,7 @@ int knn_batch_impl(const HostProb* hp, int np, int qb_cap, int seed_pts, int cap
             const int sgrid = std::min(NB, occupancy_grid((const void*)k_csr_sort, 256, kCsrSortSmem));
             DT_LAUNCH(k_csr_sort, sgrid, 256, kCsrSortSmem, s, off, NB, csr_leaf, csr_dmin, csr_key);
         }
-        P.release(csr_key);  // only the order needed it
+        if (OP != OP_RANGE) P.release(csr_key);  // only the order needed it
         P.release(outp);
         return DTREE_OK;
     };
@@ -1331,11 +1331,10 @@ int kfn_by_tiles(const dtree_t* tq, const dtree_t* tr, bool mono, int k, int64_t
     constexpr int qb = 128, seed = 64, cap = 8, prec = DTREE_PREC_BF16, spin = 1 << 20;
     int rc;
     switch (tr->dp) {
-        case 4: rc = knn_batch_impl<4, OP_FAR>(&hp, 1, qb, seed, cap, prec, spin, 0, DTREE_BOUND_BOX, s, st, nullptr); break;
-        case 8: rc = knn_batch_impl<8, OP_FAR>(&hp, 1, qb, seed, cap, prec, spin, 0, DTREE_BOUND_BOX, s, st, nullptr); break;
         case 16: rc = knn_batch_impl<16, OP_FAR>(&hp, 1, qb, seed, cap, prec, spin, 0, DTREE_BOUND_BOX, s, st, nullptr); break;
         case 32: rc = knn_batch_impl<32, OP_FAR>(&hp, 1, qb, seed, cap, prec, spin, 0, DTREE_BOUND_BOX, s, st, nullptr); break;
-        default: rc = knn_batch_impl<64, OP_FAR>(&hp, 1, qb, seed, cap, prec, spin, 0, DTREE_BOUND_BOX, s, st, nullptr); break;
+        case 64: rc = knn_batch_impl<64, OP_FAR>(&hp, 1, qb, seed, cap, prec, spin, 0, DTREE_BOUND_BOX, s, st, nullptr); break;
+        default: return DTREE_ERR_UNSUPPORTED;  // (kfn.cu's rule keeps d <= 8 with the walks)
     }
     if (rc != DTREE_OK) cudaStreamSynchronize(s);
     return rc;
