@@ -740,6 +740,29 @@ WORKLOAD_KFN = WORKLOAD.replace("exact kNN", "exact k-furthest neighbours")
 METRIC_RANGE = "exact range-search queries/s (oracle-identical)"
 
 
+def kfn_range_line(is_range, d, st, sms, ms_step):
+    """What a k-furthest or range step's counters say: the arithmetic it ran, its
+    phases, and the roofline of the launch that did most of it (for a range
+    search, of its counting pass).  Large problems in d > 8 run the block search
+    (query_blocks > 0), whose point_pairs include the seed pass's; the others a
+    walk per query."""
+    if st["query_blocks"] > 0:
+        parts = {"seed": st["ns_seed"], "traverse": st["ns_traverse"], "tiles": st["ns_basecase"],
+                 "fallback": st["ns_fallback"]}
+        phases = {("count_" if is_range else "") + p: ns / 1e6 for p, ns in parts.items()}
+        roof = roofline("bf16", d, st["point_pairs"] - st["seed_point_pairs"], st["ns_basecase"], sms, None)
+        dtype = "bf16"
+        precision = ("split BF16 tensor-core filter, float32 and float64 decisions" if is_range else
+                     "split BF16 tensor-core keys, exact re-rank")
+    else:
+        phases = {"range_count" if is_range else "kfn": st["ns_basecase"] / 1e6}
+        roof = roofline("fp32", d, st["point_pairs"], st["ns_basecase"], sms, None)
+        roof["kernel"] = ("k_range count launch" if is_range else "k_kfn") + " (one warp per query, float32 keys)"
+        dtype, precision = "f32", "fp32 keys, f64 decisions"
+    phases["build_and_rest"] = ms_step - sum(phases.values())
+    return {"dtype": dtype, "precision": precision, "roofline": roof, "phases_ms": phases}
+
+
 def run_kfn(args, rank, world, local):
     """--op kfn: one step = build the reference tree + build the query tree +
     dtree_kfn (the block search with negated distances at this size; small
@@ -869,41 +892,20 @@ def run_kfn(args, rank, world, local):
     f1.record(stream)
     torch.cuda.synchronize()
     e2e_value = job_rate(world, nq, max_over_ranks(f0.elapsed_time(f1) / args.e2e_steps, world, "cuda"))
-    ns = sum(s["ns_basecase"] for s in stats) / len(stats)
-    pairs = sum(s["point_pairs"] for s in stats) / len(stats)
-    sms = props.multi_processor_count
-    peaks = {}
-    try:
-        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
-            peaks = json.load(f)
-    except (OSError, ValueError):
-        pass
-    sm_max = float(peaks.get("sm_max_mhz", 2070.0))
-    flops = 3.0 * d * pairs  # d subtractions + d FMAs per point distance
-    peak = 2.0 * 128 * sms * sm_max * 1e6 / 1e12
-    achieved = flops / (ns * 1e-9) / 1e12 if ns > 0 else 0.0
+    mean = {k2: sum(s[k2] for s in stats) / len(stats) for k2 in stats[0]}
+    how = kfn_range_line(is_range, d, mean, props.multi_processor_count, ms_max)
     s0 = stats[-1]
     line = {
         "metric": metric, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_max, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "f32", "data": "synthetic",
-        "config": {"workload": workload, "precision": "fp32 keys, f64 decisions", "leaf_size": args.leaf,
+        "vs_baseline": None, "dtype": how["dtype"], "data": "synthetic",
+        "config": {"workload": workload, "precision": how["precision"], "leaf_size": args.leaf,
                    "step": "build ref tree + build query tree + "
                            + ("dtree_range (count, scan, fill)" if is_range else "dtree_kfn"),
                    "l2": "inputs (320 MB) larger than the 129 MB L2; no flush",
                    "parallelism": f"{world} GPU(s), one query shard each, reference replicated"},
-        # large problems in d > 8 run the block search: tensor-core tiles
-        "roofline": roofline("bf16", d, pairs, ns, sms, None) if s0["query_blocks"] > 0 else
-                    {"bound": "alu",
-                     "kernel": ("k_range count launch" if is_range else "k_kfn")
-                     + " (one warp per query, float32 keys)",
-                     "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                     "frac": achieved / peak if peak else None, "traffic": None,
-                     "peak_source": f"2 x 128 FP32 lanes x {sms} SMs x {sm_max:.0f} MHz",
-                     "algorithmic_flops_per_step": flops, "point_pairs_per_step": pairs,
-                     "kernel_ms": ns / 1e6},
-        "phases_ms": {("range_count" if is_range else "kfn"): ns / 1e6,
-                      "build_and_rest": ms_max - ns / 1e6},
+        "roofline": how["roofline"],
+        "phases_ms": how["phases_ms"],
         "counters": {k2: s0[k2] for k2 in ("point_pairs", "leaf_pairs_evaluated",
                                           "node_pairs_pruned", "fallback_queries",
                                           "rerank_candidates")},
@@ -1035,14 +1037,15 @@ def run_emst(args, rank, world, local):
     line = {
         "metric": METRIC_EMST, "value": value, "unit": "points/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_max, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "f64", "data": "synthetic",
+        "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": workload, "step": "build tree + dtree_emst (Boruvka rounds)",
+                   "precision": "float32 keys; ties, near-ties and the edges' lengths in float64",
                    "l2": "inputs (12 MB) fit the 129 MB L2: a 256 MB buffer is written before each timed step, outside its events",
                    "parallelism": f"{world} GPU(s), one problem each"},
-        "roofline": {"bound": "fp64", "kernel": "k_emst_nn (one warp per point, float64 distances)",
+        "roofline": {"bound": "latency", "kernel": "k_emst_nn (packets of up to 32 points, float32 keys)",
                      "achieved": None, "peak": None, "unit": None, "frac": None, "traffic": None,
-                     "note": "the float64 pipe is the limit (about 80% busy in the ncu capture, "
-                             "profiles/k_emst_nn_uniform3.md); no algorithmic-flop count is claimed"},
+                     "note": "chains of dependent loads, one walk of the tree per packet and Boruvka round; "
+                             "no counter capture of this kernel and no algorithmic-flop count is claimed"},
         "phases_ms": {"emst": ns / 1e6, "build_and_rest": ms_max - ns / 1e6},
         "counters": {"point_pairs": pairs, "leaf_pairs_evaluated": stats[-1]["leaf_pairs_evaluated"]},
         "e2e": {"value": e2e_value, "unit": "points/s", "h2d_bytes_per_step": int(P.nbytes),

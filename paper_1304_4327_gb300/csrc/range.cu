@@ -181,13 +181,16 @@ extern "C" int dtree_range_count(const dtree_t* query, const dtree_t* ref, doubl
     cudaFreeAsync(cnt, s);
     if (cudaStreamSynchronize(s) != cudaSuccess && rc == DTREE_OK) rc = cuda_status(cudaGetLastError());
     if (st && rc == DTREE_OK) {
-        st->point_pairs = (int64_t)h[0] + tst.point_pairs;
-        st->leaf_pairs_evaluated = (int64_t)h[1] + tst.leaf_pairs_evaluated;
-        st->node_pairs_pruned = (int64_t)h[2] + tst.node_pairs_pruned;
-        st->rerank_candidates = (int64_t)h[3] + tst.rerank_candidates;
-        st->query_blocks = tst.query_blocks;
         float ms = 0.f;
-        if (timed && cudaEventElapsedTime(&ms, ev[0], ev[1]) == cudaSuccess) st->ns_basecase = (int64_t)(ms * 1e6);
+        if (tiles) {
+            *st = tst;  // its counters and phases
+        } else {
+            st->point_pairs = (int64_t)h[0];
+            st->leaf_pairs_evaluated = (int64_t)h[1];
+            st->node_pairs_pruned = (int64_t)h[2];
+            st->rerank_candidates = (int64_t)h[3];
+            if (timed && cudaEventElapsedTime(&ms, ev[0], ev[1]) == cudaSuccess) st->ns_basecase = (int64_t)(ms * 1e6);
+        }
         st->kernel_launches = g_launches.load() - launches0;
     }
     if (timed) {
