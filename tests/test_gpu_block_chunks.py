@@ -1,9 +1,12 @@
 """The block search of k-furthest neighbours and range searches: that it is what
 runs at the sizes its tests are made for, and on query blocks of several chunks
 of 128 (query leaves of more points), whole, odd and in pairs."""
+import numpy as np
 import pytest
 import torch
 
+from oracle import kfn as okfn
+from oracle import rangesearch as orange
 from test_gpu_kfn_routes import mixture
 from test_gpu_kfn_tiles import clusters, cuda, lattice
 
@@ -96,3 +99,28 @@ def test_range_ends_hit_exactly(dt):
     R = torch.randint(0, 4, (40_000, 16), generator=g, device="cuda").float()
     Q = torch.randint(0, 4, (25_001, 16), generator=g, device="cuda").float()
     within(dt, R, Q, 2.0, 3.0, 32, 32)
+
+
+@pytest.mark.parametrize("d,k,qleaf", [(16, 10, 32), (33, 1, 400), (64, 50, 32)])
+def test_sampled_queries_against_the_oracle(dt, d, k, qleaf):
+    R, Q = mixture(60_001, d, 3), mixture(100_001 if qleaf > 128 else 20_001, d, 4)
+    pick = torch.arange(0, Q.shape[0], 1_571)
+    rows, sample = R.cpu().numpy(), Q[pick.cuda()].cpu().numpy()
+    tr, tq = dt.dtree_build(R, 32), dt.dtree_build(Q, qleaf)
+    idx, dist, st = dt.dtree_kfn(tq, tr, k, with_stats=True)
+    assert st["query_blocks"] > 0
+    ti, td2 = okfn.kfn_brute(rows, sample, k)
+    assert np.array_equal(idx[pick.cuda()].cpu().numpy(), ti)
+    assert np.array_equal(dist[pick.cuda()].cpu().numpy(), np.sqrt(td2).astype(np.float32))
+    lo, hi = 0.4 * (2 * d) ** 0.5, 0.5 * (2 * d) ** 0.5
+    off, idx, dist, st = dt.dtree_range(tq, tr, lo, hi, with_stats=True)
+    assert st["query_blocks"] > 0
+    to, ti, td = orange.range_brute(rows, sample, lo, hi)
+    off, idx, dist = off.cpu().numpy(), idx.cpu().numpy(), dist.cpu().numpy()
+    for n, q in enumerate(pick.tolist()):
+        i, e = idx[off[q]:off[q + 1]], dist[off[q]:off[q + 1]]
+        order = np.argsort(i)
+        assert np.array_equal(i[order], ti[to[n]:to[n + 1]])
+        assert np.array_equal(e[order], td[to[n]:to[n + 1]].astype(np.float32))
+    tr.free()
+    tq.free()
