@@ -7,7 +7,7 @@ power-law covariance spectrum (eigenvalue i proportional to i^-1.5, random
 rotation), k = 50, leaf size 32.  The headline arm is the learned proposal
 (trained once, before the timed region, on the method's own answers for
 200,000 disjoint training queries) with split-BF16 tensor-core BaseCase tiles
-and the float64 re-rank; the same run times the same precision without the
+and the exact re-rank; the same run times the same precision without the
 proposal and the plain FP32 GPU dual-tree (CUDA-core tiles) on the same
 inputs, and reports value / plain as `vs_plain_fp32`.  --workload latent3
 (10M x 1M, d = 8, k = 10) and gmm16 (4M x 1M, d = 16, k = 10) run the same
@@ -15,7 +15,7 @@ contract.
 
 One step = the whole path: build the reference kd-tree, build the query
 kd-tree, run the exact kNN search (seed, per-query caps, bounds, pruning
-dual-tree traversal, BaseCase tiles, float64 re-rank, output).  `value` =
+dual-tree traversal, BaseCase tiles, exact re-rank, output).  `value` =
 queries/s of the whole job (all ranks' queries / the slowest rank's time).
 The inputs exceed the 129 MB L2, so no flush is needed between steps.
 
@@ -497,7 +497,7 @@ def run_knn(args, rank, world, local):
     roof = roofline(precision, d, pairs, ns_tile, sms, traffic_of(args.workload, precision, pairs))
     s0 = stats[-1]
     arm_name = ("learned proposal (M=%d) + " % M if M else "") + precision.upper() + (
-        " tensor-core tiles + float64 re-rank" if precision != "fp32" else " CUDA-core tiles")
+        " tensor-core tiles + exact re-rank" if precision != "fp32" else " CUDA-core tiles")
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_max, "higher_is_better": True,

@@ -54,9 +54,11 @@ typedef enum dtree_status {
 } dtree_status;
 
 /* Distance arithmetic of the BaseCase tiles.  Whatever the choice, results
- * are exact: candidates near each query's k-th distance are re-ranked in
- * float64, and a query whose candidate band overflows is recomputed in
- * float64 (see dtree_knn). */
+ * are exact: candidates near each query's k-th distance are re-ranked by their
+ * float64 distances (the tensor-core searches by pairs of float32 with a proven
+ * bound where that settles the order and the rounding, else in float64), and a
+ * query whose candidate band overflows is recomputed with float32 keys, then
+ * in float64 (see dtree_knn). */
 typedef enum dtree_precision {
     DTREE_PREC_FP32 = 0,   /* CUDA-core float32 differences and squares */
     DTREE_PREC_TF32 = 1,   /* tensor cores (tcgen05), TF32 inputs, FP32 accumulate */
@@ -112,7 +114,7 @@ typedef struct dtree_stats {
     int64_t leaf_pairs_skipped;  /* emitted pairs pruned later by the tightened B */
     int64_t leaf_pairs_evaluated;/* pairs whose BaseCase tile ran (seed pairs included) */
     int64_t point_pairs;         /* BaseCase(p_q, p_r) evaluations of the main pass */
-    int64_t rerank_candidates;   /* candidates re-ranked in float64 */
+    int64_t rerank_candidates;   /* candidates re-ranked by their exact distances */
     int64_t fallback_queries;    /* queries whose error band overflowed the candidate list
                                     and were recomputed over their own candidate leaves
                                     (float32 keys, float64 re-rank of the band) */
@@ -171,7 +173,7 @@ int dtree_build(const float* pts, int64_t n, int32_t d, const dtree_opts* opts, 
  *   out_dist  device, n_q x k float32, Euclidean distances (not squared),
  *             the float64 distance rounded to float32.
  *   opts      nullable; uses precision, query_block, seed_points, proposal,
- *             spin_budget.
+ *             spin_budget, cap_leaves, bound.
  *   stream    cudaStream_t or NULL.
  *   stats     nullable; receives the call's counters.
  *
@@ -203,18 +205,29 @@ int dtree_knn(const dtree_t* query, const dtree_t* ref, int32_t k, int64_t* out_
  *             (distance), ties by the lower index
  *   out_dist  device, n_q x k float32: the Euclidean distance, computed in
  *             float64 and rounded once
- *   opts      nullable; precision must be DTREE_PREC_FP32 (float32 keys with a
- *             float64 re-rank, float64 keys for queries whose error band
- *             overflows: results are exact either way); other fields ignored
+ *   opts      nullable; precision must be DTREE_PREC_FP32; other fields ignored.
+ *             Small problems, d <= 8, k > 50 and points of low intrinsic
+ *             dimension are searched by a walk of the tree per query (float32
+ *             keys with a float64 re-rank, float64 keys for queries whose error
+ *             band overflows).  Large ones in d > 8 go through dtree_knn's
+ *             passes with every distance negated and split-BF16 tensor-core
+ *             keys; their band is re-ranked as dtree_knn's, and queries whose
+ *             band overflows are walked.  Results are exact, and the same,
+ *             either way
  *   stream    cudaStream_t or NULL
- *   stats     nullable; point_pairs (point distances evaluated),
- *             leaf_pairs_evaluated (leaves visited), node_pairs_pruned,
- *             fallback_queries, kernel_launches, ns_basecase
+ *   stats     nullable; point_pairs (point distances evaluated, the seed pass's
+ *             among them), leaf_pairs_evaluated (leaves visited),
+ *             node_pairs_pruned, fallback_queries, fallback64_queries,
+ *             kernel_launches, ns_basecase; query_blocks is positive where the
+ *             tensor-core passes ran, which fill the other fields too
  * Status: DTREE_ERR_INVALID_ARG (null tree or outputs, dimension mismatch,
  * trees on another device, non-zero reserved options), DTREE_ERR_INVALID_K,
  * DTREE_ERR_UNSUPPORTED (k > 63, another precision, a reference tree deeper
- * than 30 levels), or a CUDA error.  Waits for the result.  Scratch comes
- * from the device's stream-ordered pool.
+ * than 30 levels), or a CUDA error.  Where the tensor-core passes find no memory
+ * or a bounded wait of theirs gives up, the walks take over.  Waits for the
+ * result.  Scratch comes from the device's stream-ordered pool (the tensor-core
+ * passes' includes the reference points as operand rows, 96 to 288 bytes each,
+ * unless a dtree_knn call left them in the tree); nothing is kept in the trees.
  */
 int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, int64_t* out_idx,
               float* out_dist, const dtree_opts* opts, void* stream, dtree_stats* stats);
@@ -231,14 +244,23 @@ int dtree_kfn(const dtree_t* query, const dtree_t* ref, int32_t k, int64_t* out_
  *     the outputs (rows in the caller's query order), and *total (host) gets
  *     offsets[n_q]; stats (nullable): point_pairs (distances evaluated),
  *     leaf_pairs_evaluated, node_pairs_pruned, rerank_candidates (points
- *     decided in float64), kernel_launches, ns_basecase.
+ *     decided in float64), kernel_launches, ns_basecase; query_blocks is
+ *     positive where the tensor-core passes below ran, which fill ns_traverse
+ *     too.
  *   dtree_range_fill writes each query's segment: out_idx (device, int64,
  *     *total) the caller's reference row indices, out_dist (device, float32)
  *     the distances rounded once from float64.  Within a segment the order is
  *     the search's visit order (the problem's lists are sets); it is the same
  *     from call to call.
  * The same trees and range must be passed to both.  opts: nullable,
- * precision must be DTREE_PREC_FP32.  Status: DTREE_ERR_INVALID_ARG (null
+ * precision must be DTREE_PREC_FP32.  Most searches walk the tree once per query.
+ * Large ones in d > 8 whose queries would visit much for few results take
+ * dtree_knn's block traversal and split-BF16 tensor-core tiles as a filter, whose
+ * candidates are decided as ever; their scratch, from the stream-ordered pool,
+ * holds the reference points as operand rows (unless a dtree_knn call left them
+ * in the tree) and up to 1 GB of candidate bits.  Without that memory, or where
+ * a bounded wait of theirs gives up, the walks take over.  Nothing is kept in the
+ * trees.  Status: DTREE_ERR_INVALID_ARG (null
  * tree or buffer, dimension mismatch, d_lo < 0, d_hi < d_lo, NaN, trees on
  * another device), DTREE_ERR_UNSUPPORTED (another precision, a reference tree
  * deeper than 30 levels), or a CUDA error.  Both wait for the result.
@@ -253,8 +275,9 @@ int dtree_range_fill(const dtree_t* query, const dtree_t* ref, double d_lo, doub
 /*
  * dtree_emst -- the Euclidean minimum spanning tree of a tree's points by
  * Boruvka rounds (Section 7): each round, every component's shortest edge to
- * a point outside it (a pruning search per point, float64 distances), then
- * the components joined by those edges merge.  Edges compare by float64
+ * a point outside it (pruning walks by packets of neighbouring points; float32
+ * keys with float64 for ties, near-ties and the edges' lengths), then the
+ * components joined by those edges merge.  Edges compare by float64
  * squared length, equal lengths by (lower index, higher index), so the tree
  * is unique.
  *   tree      the points (any dimension the library builds)
@@ -423,7 +446,8 @@ int dtree_attach_proposal(dtree_t* ref, const dtree_model* model);
  *           W3 [C x 256], b3 [C] (row-major, W_l maps layer l-1 to layer l)
  *   X       device FP32 [n x d] inputs (used as given, not standardised)
  *   T       device FP32 [n x C] target distributions (rows sum to 1)
- *   loss    host: mean over rows of -sum_c T log softmax(Z)
+ *   loss    host: mean over rows of -sum_c T log softmax(Z), summed in float64 in
+ *           an order that depends on n alone
  *   grads   device FP32, the gradients of `loss`, shaped like params
  * GEMMs run in FP16 on the tensor cores with FP32 accumulation.  n <= 4096.
  */
@@ -431,7 +455,9 @@ int dtree_mlp_loss_grad(int32_t d, int32_t C, const float* const* params, const 
                         const float* T, int32_t n, float* loss, float* const* grads, void* stream);
 
 /* dtree_free -- release every device allocation of the handle.  NULL-safe.
- * Must not be called while work that uses the handle is still in flight. */
+ * Must not be called while work that uses the handle is still in flight: the
+ * memory of small trees (arrays up to 64 MB) goes to a pool of the library's own
+ * without waiting for it; the pool keeps at most 256 MB for later builds. */
 void dtree_free(dtree_t* tree);
 
 /* Number of points / dimension / depth (leaves sit at this depth) / leaf

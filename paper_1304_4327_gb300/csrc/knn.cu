@@ -26,11 +26,12 @@
 //                exceeds it, then re-ranks the candidates near the k-th
 //                distance exactly and writes the outputs;
 //   5. fallback  a query whose band of near-k-th candidates overflowed its
-//                list is recomputed exactly in float64 over its block's
-//                candidate leaves (one CTA per such query).
+//                list is recomputed over its block's candidate leaves (one
+//                CTA per such query), with float32 keys and, where that band
+//                overflows too, in float64.
 //
 // The same passes serve k-furthest neighbours (OP_FAR) and range searches
-// (OP_RANGE) of large problems.
+// (OP_RANGE) of large problems, where probe.cuh's look finds that they pay.
 #include <algorithm>
 #include <cmath>
 #include <vector>

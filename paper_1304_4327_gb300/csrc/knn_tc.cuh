@@ -28,9 +28,10 @@
 //     ub = sqrt(S + alpha' (a^2 + bb^2)) + e1 (a + bb),  bb = 1.03 (a + sqrt S)
 // bounds the true k-th distance (it feeds B_1, B_2 and Score), and every
 // true k-nearest neighbour has s <= T = (ub + e1 (a + bu))^2 + alpha' (a^2 + bu^2),
-// bu = 1.01 (a + ub).  Candidates with s <= T are re-ranked in float64; a
-// list too short to hold them all sends the query to the float64 pass.  The
-// bounds hold for any centring point; the root centre trades a wider band
+// bu = 1.01 (a + ub).  Candidates with s <= T are re-ranked by their exact
+// distances (pairs of float32 where their bound settles order and rounding, else
+// float64); a list too short to hold them all sends the query to the fallback
+// passes (float32 keys, then float64).  The bounds hold for any centring point; the root centre trades a wider band
 // (larger a, b) for converting each reference point once instead of once
 // per tile.
 #pragma once
@@ -126,7 +127,7 @@ struct TcSmem {
     static constexpr int OFF_CEN = OFF_BUF + NG * CB * kQB * 8;      // DP float
     static constexpr int END = OFF_CEN + DP * 4;
     // at a block's end everything above is idle: the merge of two groups'
-    // lists (float + int per entry) and the float64 re-rank (double + int per
+    // lists (float + int per entry) and the re-rank (eight bytes + int per
     // entry) reuse it from offset 0
     static constexpr int FIN = QH * kQB * KC * 12;
     static constexpr int BYTES = END > FIN ? END : FIN;
@@ -1402,7 +1403,9 @@ int launch_tile_tc(const TileArgs& a, int fmt, int kc, int items, bool wide, int
     // two epilogue groups where their lists leave room for a second group's
     // registers (eleven warps put three on a sub-partition: 168 registers a
     // thread); else one group.  Items of two halves where the caller's blocks
-    // hold them (wide), a group per half
+    // hold them (wide), a group per half (at d = 64 these spill 60 to 128 bytes;
+    // 200k x 200k power-law points, k = 10, blocks of 512 in pairs against blocks of
+    // 128: 19.0 against 21.2 ms in BF16, 17.2 against 19.9 in TF32)
 #define DT_TC_CASE(FMTV, KCV)                                                                     \
     if (F == FMTV && kc == KCV) {                                                                 \
         if constexpr (KCV <= 32)                                                                  \

@@ -426,7 +426,8 @@ __global__ void __launch_bounds__(256) k_topm(const float* Z, int Cc, int M, int
 // ---------------------------------------------------------------------------
 
 // Slices of K for an M x N x K product: enough CTAs for the GPU (304: two per
-// SM), no more than its chunks.
+// SM of 152, a constant so that the order of the sums never depends on the device),
+// no more than its chunks.
 int gemm_slices(int M, int N, int K) {
     const int64_t tiles = (int64_t)((M + 127) / 128) * ((N + 127) / 128);
     const int64_t s = std::min<int64_t>(304 / tiles, (K + kGK - 1) / kGK);
