@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_far(const ProbeArgs a) 
         const int rows = min(tcnt[t], kProbeRows);
         if (t % (kProbeThreads / 32) == warp)
             for (int r = lane; r < rows; r += 32)
-                pv[np + r] = approx_d2<DP>(q, a.rpts + ((int64_t)tbeg[t] + r) * DP);
+                pv[np + r] = approx_d2<DP>(q, a.rpts + (tbeg[t] + probe_pick(r, tcnt[t], rows)) * DP);
         np += rows;
         all += tcnt[t];
     }
@@ -232,9 +232,12 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_far(const ProbeArgs a) 
 // three latent dimensions at 0.4 1.1% and 45%, 40 -> 243; 1M x 20k of six in d = 32 at
 // 0.6 0.2% and 0.5%, 6.5 -> 8.6; at 1.0 0.8% and 2.2%, 24 -> 72; distances of 9 to 20
 // among Gaussian points, where nearly all points lie within the upper end, 64 -> 207).
+// Leaves of more than 64 points halve what a walk pays per point (leaves of 390, the
+// mixture at 3.2 0.4%, 2.5 -> 2.9; d = 10 at 1.9, of 490, 0.3%, 10.9 -> 15.1).
 template <int DP>
-__device__ __forceinline__ bool range_by_tiles_pays(float share, float points, float within) {
-    return share >= 0.0025f && points >= 150.f && within <= (DP <= 16 ? 0.0045f : 0.008f);
+__device__ __forceinline__ bool range_by_tiles_pays(const ProbeArgs& a, float share, float within) {
+    const float few = (DP <= 16 ? 0.0045f : 0.008f) * (a.nr > 64 * a.nleaves ? 0.5f : 1.f);
+    return share >= 0.0025f && share * (float)a.nr >= 150.f && within <= few;
 }
 
 // Range searches: kept counts the sampled leaves that meet the range, near the
@@ -284,11 +287,11 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_range(const ProbeArgs a
     const int nt = min(found, kProbeRangeTop);
     for (int t = 0; t < nt; ++t) {
         const int64_t nd = a.rleaf0 + probe_pick(list[probe_pick(t, found, nt)], a.nleaves, S);
-        const int rows = min(a.rcnt[nd], kProbeRows);
+        const int rc = a.rcnt[nd], rows = min(rc, kProbeRows);
         pts += rows;
         if (t % (kProbeThreads / 32) != warp) continue;
         for (int r = lane; r < rows; r += 32)
-            near += approx_d2<DP>(q, a.rpts + ((int64_t)a.rbeg[nd] + r) * DP) <= a.hi2_up;
+            near += approx_d2<DP>(q, a.rpts + (a.rbeg[nd] + probe_pick(r, rc, rows)) * DP) <= a.hi2_up;
     }
     // (each query by the leaves it stands for: sixteen times found / nt)
     const int weight = nt == kProbeRangeTop ? found : kProbeRangeTop;
@@ -301,7 +304,7 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_range(const ProbeArgs a
         // (a range far below the extents: the tensor-core keys' error, about 1e-4
         // of their square, would add too many candidates)
         a.out->gate = extents && a.hi_up * a.hi_up >= 4e-4f * radius * radius &&
-                      range_by_tiles_pays<DP>(share, share * (float)a.nr, (float)all_near / fmaxf((float)all_pts, 1.f));
+                      range_by_tiles_pays<DP>(a, share, (float)all_near / fmaxf((float)all_pts, 1.f));
     }
 }
 
